@@ -774,7 +774,7 @@ def hall(args, g, torch):
             "value": n * M * M / t_mom, "kb_moments_s": t_mom, "kubo_bastin_s": t_kb,
             "kernels": {"k_kb_step_ms_per_launch": prof_ms[7] / max(int(prof_n[7]), 1),
                         "k_kb_step_launches": int(prof_n[7]) // steps, "contraction_ms": gemm_s * 1e3,
-                        "k_kb_integrand_ms": prof_ms[9] / max(int(prof_n[9]), 1)},
+                        "k_kb_series_ms": prof_ms[9] / max(int(prof_n[9]), 1)},
             "roofline": roof, "sigma_xy_gap_centre_e2_over_h": float(s_np[i0])}
     if 0 in sigmas:
         for mode, key in ((1, "tensor_core_split_tf32"), (2, "fp32_chains_tensor_core")):

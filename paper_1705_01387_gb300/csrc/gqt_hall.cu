@@ -18,8 +18,8 @@
 // (4 M^2 N R FP64 FMAs) -- as a register-blocked FP64 GEMM with a deterministic
 // split over the contraction; k_kb_gemm_tma does the same contraction in split
 // TF32 on the tcgen05 tensor cores, its operands brought in by TMA.
-// k_kb_integrand evaluates the double sum on an energy grid (a bilinear form per
-// energy), and k_kb_scan integrates it.
+// k_kb_collapse turns the double sum over the moments into a series of 2M - 1 angles,
+// k_kb_series evaluates it on an energy grid, and k_kb_scan integrates it.
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -553,90 +553,145 @@ __global__ void k_kb_reduce(const double2* __restrict__ part, int S, int M, doub
   }
 }
 
-// F(x_e) = (1 - x^2)^-2 Re sum_mn Gamma_mn(x) W_mn Lambda_mn for EB energies per
-// CTA, W_mn = w_m w_n (w = c_n g_n).  Per energy the sum is
-//   sum_m Tw_m z1_m + conj(aw_m) z2_m,  z1_m = sum_n Lambda_mn aw_n,  z2_m = sum_n Lambda_mn Tw_n,
-// Tw_n = w_n T_n(x), aw_n = w_n e^{-i n th}(x + i n sin th) (and w_m e^{i m th}(x - i m sin th)
-// = conj(aw_m)).  Tables in shared memory; one warp per row m, lanes over n.
-template <int EB>
-__global__ void __launch_bounds__(256) k_kb_integrand(const double2* __restrict__ lam, int M,
-                                                      const double* __restrict__ E, int NE, double inv_dE,
-                                                      const double* __restrict__ w, double* __restrict__ F) {
-  extern __shared__ double kb_sm[];
-  double2* aw = reinterpret_cast<double2*>(kb_sm);  // [EB][M], first: 16-byte aligned for any M
-  double* Tw = kb_sm + 2 * EB * M;                   // [EB][M]
-  __shared__ double2 red[EB][8];
-  const int e0 = blockIdx.x * EB;
-  for (int t = threadIdx.x; t < EB * M; t += blockDim.x) {
-    const int e = t / M, n = t - e * M;
-    double x = 0.0;
-    if (e0 + e < NE) x = E[e0 + e] * inv_dE;
-    const double th = acos(x), s = sin(th);
-    double sn, cn;
-    sincos((double)n * th, &sn, &cn);
-    Tw[t] = w[n] * cn;
-    // e^{-i n th}(x + i n s) = (cn - i sn)(x + i n s)
-    aw[t] = make_double2(w[n] * (cn * x + sn * n * s), w[n] * (cn * n * s - sn * x));
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  double2 acc[EB];
-#pragma unroll
-  for (int e = 0; e < EB; ++e) acc[e] = make_double2(0.0, 0.0);
-  for (int m = warp; m < M; m += nw) {
-    double2 z1[EB], z2[EB];
-#pragma unroll
-    for (int e = 0; e < EB; ++e) z1[e] = z2[e] = make_double2(0.0, 0.0);
-    const double2* row = lam + (size_t)m * M;
-    for (int nn = lane; nn < M; nn += 32) {
-      const double2 l = row[nn];
-#pragma unroll
-      for (int e = 0; e < EB; ++e) {
-        const double2 a = aw[e * M + nn];
-        const double t = Tw[e * M + nn];
-        z1[e].x = fma(l.x, a.x, fma(-l.y, a.y, z1[e].x));
-        z1[e].y = fma(l.x, a.y, fma(l.y, a.x, z1[e].y));
-        z2[e].x = fma(l.x, t, z2[e].x);
-        z2[e].y = fma(l.y, t, z2[e].y);
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < EB; ++e) {
-      for (int off = 16; off > 0; off >>= 1) {
-        z1[e].x += __shfl_xor_sync(0xffffffffu, z1[e].x, off);
-        z1[e].y += __shfl_xor_sync(0xffffffffu, z1[e].y, off);
-        z2[e].x += __shfl_xor_sync(0xffffffffu, z2[e].x, off);
-        z2[e].y += __shfl_xor_sync(0xffffffffu, z2[e].y, off);
-      }
-      if (lane == 0) {
-        const double tm = Tw[e * M + m];
-        const double2 am = aw[e * M + m];  // conj(am) multiplies z2
-        acc[e].x += tm * z1[e].x + am.x * z2[e].x + am.y * z2[e].y;
-        acc[e].y += tm * z1[e].y + am.x * z2[e].y - am.y * z2[e].x;
-      }
-    }
-  }
-  if (lane == 0)
-#pragma unroll
-    for (int e = 0; e < EB; ++e) red[e][warp] = acc[e];
-  __syncthreads();
-  if ((int)threadIdx.x < EB && e0 + (int)threadIdx.x < NE) {
-    const int e = threadIdx.x;
-    double s = 0.0;
-    for (int q = 0; q < nw; ++q) s += red[e][q].x;
-    const double x = E[e0 + e] * inv_dE;
-    F[e0 + e] = s / ((1.0 - x * x) * (1.0 - x * x));
+// The Kubo-Bastin integrand F(x) = (1 - x^2)^-2 Re sum_mn Gamma_mn(x) W_mn, W_mn =
+// w_m w_n Lambda_mn (w = c_n g_n), as one trigonometric series.  With cos m th cos n th
+// and cos m th sin n th turned into sums over the angles (m +- n) th, the M^2 terms
+// collapse, once for all energies, onto 2M - 1 angles k th (x = cos th, s = sin th,
+// W = a + i b):
+//   (1 - x^2)^2 F = sum_k cos k th (x A_k + s B_k) + sin k th (s k A_k / 2 - x V_k),
+//   A_k = sum_{m+n=k} a_mn + sum_{|m-n|=k} a_mn,
+//   V_k = sum_{m-n=k} b_mn - sum_{n-m=k} b_mn   (V_0 = 0),
+//   B_k = (sum_{m+n=k} (m - n) b_mn + k V_k) / 2.
+// Per energy that is 4M FMA-pairs instead of 6 M^2 FMA: at M = 500 and 2001 energies
+// the bilinear form per energy took 10.85 ms on the FP64 pipe, the series takes 58 us
+// after 42 us for the collapse and its coefficients.
+
+// w_n = c_n g_n: Jackson factors (Eq. 31) or 1, times c_0 = 1, c_n = 2.
+__global__ void k_kb_weights(int M, int jackson, double* __restrict__ w) {
+  const double a = 1.0 / (M + 1.0), cot = cospi(a) / sinpi(a);
+  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < M; n += gridDim.x * blockDim.x) {
+    const double g = jackson ? (1.0 - n * a) * cospi(n * a) + a * sinpi(n * a) * cot : 1.0;
+    w[n] = (n == 0 ? 1.0 : 2.0) * g;
   }
 }
 
-// sigma_j = pref * sum_{k<j} (x_{k+1} - x_k)(F_k + F_{k+1})/2 (one thread: a running sum).
-__global__ void k_kb_scan(const double* __restrict__ F, const double* __restrict__ E, int NE, double inv_dE,
-                          double pref, double* __restrict__ sigma) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+// Diagonal sums of rows [rows_per * y, ..) of W: thread t of the grid's x extent takes
+// antidiagonal m + n = t and the diagonals n - m = t - (M - 1), so that neighbouring
+// threads read neighbouring columns of a row.  out: [4][splits][2M - 1] (sum a and sum
+// (m - n) b of the antidiagonals, sum a and sum b of the diagonals by n - m + M - 1).
+__global__ void __launch_bounds__(128) k_kb_collapse(const double2* __restrict__ lam, int M,
+                                                     const double* __restrict__ w, int rows_per,
+                                                     double* __restrict__ out) {
+  const int nk = 2 * M - 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nk) return;
+  const int r0 = blockIdx.y * rows_per, r1 = min(M, r0 + rows_per);
+  double pa = 0.0, pb = 0.0, da = 0.0, db = 0.0;
+#pragma unroll 4
+  for (int m = r0; m < r1; ++m) {
+    const double wm = __ldg(w + m);
+    const int ca = t - m, cd = t - (M - 1) + m;
+    if (ca >= 0 && ca < M) {
+      const double2 l = __ldg(lam + (size_t)m * M + ca);
+      const double ww = wm * __ldg(w + ca);
+      pa = fma(ww, l.x, pa);
+      pb = fma(ww * (double)(m - ca), l.y, pb);
+    }
+    if (cd >= 0 && cd < M) {
+      const double2 l = __ldg(lam + (size_t)m * M + cd);
+      const double ww = wm * __ldg(w + cd);
+      da = fma(ww, l.x, da);
+      db = fma(ww, l.y, db);
+    }
+  }
+  const size_t S = gridDim.y, y = blockIdx.y;
+  out[(0 * S + y) * nk + t] = pa;
+  out[(1 * S + y) * nk + t] = pb;
+  out[(2 * S + y) * nk + t] = da;
+  out[(3 * S + y) * nk + t] = db;
+}
+
+// Sums the splits in order and forms coef[k] = (A_k, B_k, k A_k / 2, V_k).
+__global__ void k_kb_coef(const double* __restrict__ part, int M, int S, double4_16a* __restrict__ coef) {
+  const int nk = 2 * M - 1;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= nk) return;
+  auto sum = [&](int q, int t) {
+    double v = 0.0;
+    for (int y = 0; y < S; ++y) v += part[((size_t)q * S + y) * nk + t];
+    return v;
+  };
+  double a = sum(0, k), u = sum(1, k), v = 0.0;
+  if (k < M) {
+    const int hi = M - 1 + k, lo = M - 1 - k;  // n - m = k and n - m = -k
+    a += k == 0 ? sum(2, hi) : sum(2, hi) + sum(2, lo);
+    v = k == 0 ? 0.0 : sum(3, lo) - sum(3, hi);
+  }
+  double4_16a c;
+  c.x = a;
+  c.y = 0.5 * (u + k * v);
+  c.z = 0.5 * k * a;
+  c.w = v;
+  coef[k] = c;
+}
+
+// F at one energy per warp: lane l takes the angles k = l, l + 32, ..; cos k th and
+// sin k th advance by a rotation of 32 th and are taken afresh every 16 rotations,
+// which keeps their error at a few roundings.
+__global__ void __launch_bounds__(128) k_kb_series(const double4_16a* __restrict__ coef, int nk,
+                                                   const double* __restrict__ E, int NE, double inv_dE,
+                                                   double* __restrict__ F) {
+  const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (e >= NE) return;
+  const double x = E[e] * inv_dE, s = sqrt((1.0 - x) * (1.0 + x)), th = acos(x);
+  double rs, rc;
+  sincos(32.0 * th, &rs, &rc);
+  double cx = 0.0, cs = 0.0;  // coefficients of x and of s
+  for (int k0 = lane; k0 < nk; k0 += 512) {
+    double sn, cn;
+    sincos((double)k0 * th, &sn, &cn);
+    const int kend = min(nk, k0 + 512);
+#pragma unroll 4
+    for (int k = k0; k < kend; k += 32) {
+      const double4_16a c = coef[k];
+      cx = fma(c.x, cn, fma(-c.w, sn, cx));
+      cs = fma(c.y, cn, fma(c.z, sn, cs));
+      const double t = fma(cn, rc, -sn * rs);
+      sn = fma(sn, rc, cn * rs);
+      cn = t;
+    }
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    cx += __shfl_xor_sync(0xffffffffu, cx, off);
+    cs += __shfl_xor_sync(0xffffffffu, cs, off);
+  }
+  if (lane == 0) F[e] = (x * cx + s * cs) / ((1.0 - x * x) * (1.0 - x * x));
+}
+
+// sigma_j = pref * sum_{k<j} (x_{k+1} - x_k)(F_k + F_{k+1})/2: one CTA, each thread a
+// contiguous run of energies, the runs' sums scanned over the CTA (one thread walking
+// the grid took 0.22 ms per 1000 energies).
+__global__ void __launch_bounds__(1024) k_kb_scan(const double* __restrict__ F, const double* __restrict__ E, int NE,
+                                                  double inv_dE, double pref, double* __restrict__ sigma) {
+  __shared__ double wsum[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = (NE + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int j0 = min(NE, (int)threadIdx.x * per), j1 = min(NE, j0 + per);
+  auto panel = [&](int j) { return j == 0 ? 0.0 : 0.5 * (E[j] - E[j - 1]) * inv_dE * (F[j] + F[j - 1]); };
   double run = 0.0;
-  for (int j = 0; j < NE; ++j) {
-    if (j > 0) run += 0.5 * (E[j] - E[j - 1]) * inv_dE * (F[j] + F[j - 1]);
-    sigma[j] = pref * run;
+  for (int j = j0; j < j1; ++j) run += panel(j);
+  double inc = run;  // inclusive scan over the warp
+  for (int off = 1; off < 32; off <<= 1) {
+    const double v = __shfl_up_sync(0xffffffffu, inc, off);
+    if (lane >= off) inc += v;
+  }
+  if (lane == 31) wsum[warp] = inc;
+  __syncthreads();
+  double base = inc - run;
+  for (int q = 0; q < warp; ++q) base += wsum[q];
+  for (int j = j0; j < j1; ++j) {
+    base += panel(j);
+    sigma[j] = pref * base;
   }
 }
 
@@ -672,11 +727,6 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   }();
   if (!fn) throw Error(GQT_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
   return fn;
-}
-
-double jackson_g(int n, int M) {
-  const double a = 1.0 / (M + 1.0), pi = 3.14159265358979323846;
-  return (1.0 - n * a) * std::cos(pi * n * a) + a * std::sin(pi * n * a) / std::tan(pi * a);
 }
 
 int grid_for(size_t total) {
@@ -914,45 +964,52 @@ extern "C" gqt_status gqt_set_kb_contraction(gqt_ham* h, int mode) {
   return GQT_OK;
 }
 
-// Device F (the Kubo-Bastin integrand) on the energy grid into buf + M (buf: M
-// weights then NE values); returns an error code of the launches.
-static cudaError_t kb_integrand_dev(const double* d_lambda, int M, const double* d_E, int NE, double energy_scale,
-                                    int kernel, double* buf, cudaStream_t st) {
-  std::vector<double> hw(M);
-  for (int n = 0; n < M; ++n) hw[n] = (n == 0 ? 1.0 : 2.0) * (kernel == 0 ? jackson_g(n, M) : 1.0);
-  // energies per CTA: as many as keep the tables (24 B per energy and moment) within 200 KB
-  const int EB = (size_t)4 * M * 24 <= 200 * 1024 ? 4 : ((size_t)2 * M * 24 <= 200 * 1024 ? 2 : 1);
-  const size_t smem = (size_t)EB * M * (sizeof(double) + sizeof(double2));
-  const void* kern = EB == 4 ? (const void*)k_kb_integrand<4>
-                             : (EB == 2 ? (const void*)k_kb_integrand<2> : (const void*)k_kb_integrand<1>);
-  cudaError_t err = cudaSuccess;
-  if (smem > 48 * 1024) err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  double* w = buf;
-  double* F = buf + M;
-  const double inv = 1.0 / energy_scale;
-  if (err == cudaSuccess) err = cudaMemcpyAsync(w, hw.data(), M * sizeof(double), cudaMemcpyHostToDevice, st);
-  if (err == cudaSuccess) {
-    // the host copy of the weights must outlive the copy: wait for it here
-    err = cudaStreamSynchronize(st);
-  }
-  if (err == cudaSuccess) {
-    const dim3 grid((NE + EB - 1) / EB);
-    const double2* lam = (const double2*)d_lambda;
-    const size_t pi = prof_begin(st);
-    if (EB == 4)
-      k_kb_integrand<4><<<grid, 256, smem, st>>>(lam, M, d_E, NE, inv, w, F);
-    else if (EB == 2)
-      k_kb_integrand<2><<<grid, 256, smem, st>>>(lam, M, d_E, NE, inv, w, F);
-    else
-      k_kb_integrand<1><<<grid, 256, smem, st>>>(lam, M, d_E, NE, inv, w, F);
-    err = cudaGetLastError();
-    if (err == cudaSuccess) {
-      check_launch("k_kb_integrand");
-      prof_end(pi, 9, st);
-    }
-  }
-  return err;
+// Scratch of the Kubo-Bastin sums in doubles: weights, split diagonal sums, series
+// coefficients, F.  Splits of the collapse: 32 rows each, so that M = 256 already
+// gives 8 x 4 CTAs, and at most 32 of them (17 MB of partial sums at M = 8192).
+static int kb_rows(int M) { return std::max(32, (M + 31) / 32); }
+static size_t kb_off_coef(int M) {
+  const size_t S = (M + kb_rows(M) - 1) / kb_rows(M), nk = 2 * (size_t)M - 1;
+  return ((size_t)M + 4 * S * nk + 1) / 2 * 2;  // 16-byte aligned coefficients
 }
+static size_t kb_off_F(int M) { return kb_off_coef(M) + 4 * (2 * (size_t)M - 1); }
+static size_t kb_scratch(int M, int NE) { return kb_off_F(M) + NE; }
+
+// The energy-independent part: weights, diagonal sums and series coefficients in buf.
+static void kb_collapse(const double* d_lambda, int M, int kernel, double* buf, cudaStream_t st) {
+  const int S = (M + kb_rows(M) - 1) / kb_rows(M), nk = 2 * M - 1;
+  double* part = buf + M;
+  k_kb_weights<<<(M + 127) / 128, 128, 0, st>>>(M, kernel == 0, buf);
+  check_launch("k_kb_weights");
+  k_kb_collapse<<<dim3((nk + 127) / 128, S), 128, 0, st>>>((const double2*)d_lambda, M, buf, kb_rows(M), part);
+  check_launch("k_kb_collapse");
+  k_kb_coef<<<(nk + 127) / 128, 128, 0, st>>>(part, M, S, (double4_16a*)(buf + kb_off_coef(M)));
+  check_launch("k_kb_coef");
+}
+
+// Device F on the energy grid (returned pointer, inside buf).
+static const double* kb_integrand_dev(int M, const double* d_E, int NE, double energy_scale, double* buf,
+                                      cudaStream_t st) {
+  double* F = buf + kb_off_F(M);
+  const size_t pi = prof_begin(st);
+  k_kb_series<<<(NE + 3) / 4, 128, 0, st>>>((const double4_16a*)(buf + kb_off_coef(M)), 2 * M - 1, d_E, NE,
+                                            1.0 / energy_scale, F);
+  check_launch("k_kb_series");
+  prof_end(pi, 9, st);
+  return F;
+}
+
+// Stream-ordered scratch of one call, given back on every way out.
+struct StreamBuf {
+  double* p = nullptr;
+  cudaStream_t st;
+  StreamBuf(size_t doubles, cudaStream_t s) : st(s) {
+    check_cuda(cudaMallocAsync((void**)&p, doubles * sizeof(double), st), "cudaMallocAsync");
+  }
+  ~StreamBuf() { cudaFreeAsync(p, st); }
+  StreamBuf(const StreamBuf&) = delete;
+  StreamBuf& operator=(const StreamBuf&) = delete;
+};
 
 static std::vector<double> check_energies(const double* d_E, int NE, double energy_scale, cudaStream_t st) {
   std::vector<double> hE(NE);
@@ -974,17 +1031,11 @@ extern "C" gqt_status gqt_kubo_bastin(const double* d_lambda, int M, const doubl
       throw Error(GQT_EINVAL, "gqt_kubo_bastin: bad argument");
     cudaStream_t st = (cudaStream_t)stream;
     check_energies(d_E, NE, energy_scale, st);
-    // device scratch owned by this call (no handle): weights and F
-    double* buf = nullptr;
-    check_cuda(cudaMallocAsync((void**)&buf, (size_t)(M + NE) * sizeof(double), st), "cudaMallocAsync");
-    cudaError_t err = kb_integrand_dev(d_lambda, M, d_E, NE, energy_scale, kernel, buf, st);
-    if (err == cudaSuccess) {
-      k_kb_scan<<<1, 32, 0, st>>>(buf + M, d_E, NE, 1.0 / energy_scale, 2.0 / area, d_sigma);
-      err = cudaGetLastError();
-      if (err == cudaSuccess) check_launch("k_kb_scan");
-    }
-    cudaFreeAsync(buf, st);
-    check_cuda(err, "gqt_kubo_bastin");
+    StreamBuf buf(kb_scratch(M, NE), st);
+    kb_collapse(d_lambda, M, kernel, buf.p, st);
+    const double* F = kb_integrand_dev(M, d_E, NE, energy_scale, buf.p, st);
+    k_kb_scan<<<1, 1024, 0, st>>>(F, d_E, NE, 1.0 / energy_scale, 2.0 / area, d_sigma);
+    check_launch("k_kb_scan");
     check_cuda(cudaStreamSynchronize(st), "gqt_kubo_bastin");
     return GQT_OK;
   } catch (const Error& e) {
@@ -1009,17 +1060,11 @@ extern "C" gqt_status gqt_kubo_bastin_fermi(const double* d_lambda, int M, const
       throw Error(GQT_EINVAL, "gqt_kubo_bastin_fermi: bad argument");
     cudaStream_t st = (cudaStream_t)stream;
     check_energies(d_E, NE, energy_scale, st);
-    double* buf = nullptr;
-    check_cuda(cudaMallocAsync((void**)&buf, (size_t)(M + NE) * sizeof(double), st), "cudaMallocAsync");
-    cudaError_t err = kb_integrand_dev(d_lambda, M, d_E, NE, energy_scale, kernel, buf, st);
-    if (err == cudaSuccess) {
-      k_kb_fermi<<<(Nmu + 127) / 128, 128, 0, st>>>(buf + M, d_E, NE, 1.0 / energy_scale, d_mu, Nmu, kT, 2.0 / area,
-                                                    d_sigma);
-      err = cudaGetLastError();
-      if (err == cudaSuccess) check_launch("k_kb_fermi");
-    }
-    cudaFreeAsync(buf, st);
-    check_cuda(err, "gqt_kubo_bastin_fermi");
+    StreamBuf buf(kb_scratch(M, NE), st);
+    kb_collapse(d_lambda, M, kernel, buf.p, st);
+    const double* F = kb_integrand_dev(M, d_E, NE, energy_scale, buf.p, st);
+    k_kb_fermi<<<(Nmu + 127) / 128, 128, 0, st>>>(F, d_E, NE, 1.0 / energy_scale, d_mu, Nmu, kT, 2.0 / area, d_sigma);
+    check_launch("k_kb_fermi");
     check_cuda(cudaStreamSynchronize(st), "gqt_kubo_bastin_fermi");
     return GQT_OK;
   } catch (const Error& e) {
