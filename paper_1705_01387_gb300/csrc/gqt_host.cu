@@ -539,6 +539,15 @@ static void reset_flag(gqt_ham* h, cudaStream_t st) {
   check_cuda(cudaMemsetAsync(h->d_flag.p, 0, sizeof(int), st), "flag reset");
 }
 
+// Segment sums of the partial slots slot0 .. slot0 + nslots - 1 (and slot extra, if
+// >= 0), in place, before k_reduce, k_reduce_dbl or a norm check reads them.
+static void launch_slot_sums(double2* partial, int nblocks, int R, const int* seg_blk, int nseg, int slot0, int nslots,
+                             int extra, cudaStream_t st) {
+  const long long items = (long long)(nslots + (extra >= 0 ? 1 : 0)) * nseg;
+  k_slot_sums<<<(unsigned)std::min<long long>(items, 1 << 20), 256, 0, st>>>(partial, nblocks, R, seg_blk, nseg, slot0, nslots, extra);
+  check_launch("k_slot_sums");
+}
+
 // ====================================================================== moments core
 
 // Wavefront-ordered moment kernels for the common neighbour counts (2, 3, 4, 6
@@ -960,6 +969,7 @@ static void launch_moments_df(gqt_ham* h, const void* l, const void* r, int M, v
       rows(std::integral_constant<bool, false>());
     else
       rows(std::integral_constant<bool, true>());
+    launch_slot_sums(partial, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 0, M, pair ? 2 * steps : -1, s2);
     k_reduce_dbl<<<rb, 256, 0, s2>>>(partial, M, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 1.0 + tol, (double*)out,
                                      (int*)h->d_flag.p, pair ? 2 * steps : -1);
     check_launch("k_reduce_dbl");
@@ -1117,6 +1127,7 @@ void gqt::launch_moments(gqt_ham* h, const void* l, const void* r, int R, int M,
     if (done) {
       const int segs[2] = {0, C};
       check_cuda(cudaMemcpyAsync(cseg.p, segs, sizeof segs, cudaMemcpyHostToDevice, st), "cluster table");
+      launch_slot_sums(partial, C, 1, (const int*)cseg.p, 1, 0, M, kind == 2 ? -1 : slot_norm, st);
       if (kind == 2)
         k_reduce_dbl<<<rb, 256, 0, st>>>(partial, M, C, 1, (const int*)cseg.p, 1, 1.0 + tol, (double*)out,
                                          (int*)h->d_flag.p);
@@ -1242,10 +1253,12 @@ void gqt::launch_moments(gqt_ham* h, const void* l, const void* r, int R, int M,
       }
     });
     if (kind == 2 || pair) {
+      launch_slot_sums(partial, nb, R, (const int*)T.d_seg_blk.p, h->nseg, 0, M, pair ? 2 * ((M + 1) / 2) : -1, s2);
       k_reduce_dbl<<<rb, 256, 0, s2>>>(partial, M, nb, R, (const int*)T.d_seg_blk.p, h->nseg, 1.0 + tol, (double*)out,
                                        (int*)h->d_flag.p, pair ? 2 * ((M + 1) / 2) : -1);
       check_launch("k_reduce_dbl");
     } else {
+      launch_slot_sums(partial, nb, R, (const int*)T.d_seg_blk.p, h->nseg, 0, M, slot_norm, s2);
       k_reduce<<<rb, 256, 0, s2>>>(partial, M, nb, R, (const int*)T.d_seg_blk.p, h->nseg, slot_norm,
                                    (1.0 + tol) * (1.0 + tol), out, kind == 0 ? 0 : 1, (int*)h->d_flag.p);
       check_launch("k_reduce");
@@ -1368,6 +1381,7 @@ static void launch_evolve_df(gqt_ham* h, void* const* psi, const std::vector<dou
       else
         orders(std::false_type());
     });
+    launch_slot_sums(partial, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 0, 2 * NSET, -1, s2);
     k_norm_check<<<1, 256, 0, s2>>>(partial, NSET, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 1e-10, d_norms,
                                     (int*)h->d_flag.p);
     check_launch("k_norm_check");
@@ -1447,6 +1461,7 @@ static void launch_msd_df(gqt_ham* h, void* p, void* px, const std::vector<doubl
       else
         orders(std::false_type());
     });
+    launch_slot_sums(partial, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 0, 4, -1, s2);
     k_norm_check_msd<<<1, 256, 0, s2>>>(partial, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 1e-10,
                                         (int*)h->d_flag.p);
     check_launch("k_norm_check_msd");
@@ -1519,6 +1534,7 @@ static void launch_evolve_sets(gqt_ham* h, void* const* psi, int R, const std::v
       }
     });
     const double tol = h->prec == GQT_FP64 ? 1e-10 : 1e-5;
+    launch_slot_sums(partial, nb, R, (const int*)T.d_seg_blk.p, h->nseg, 0, 2 * NSET, -1, s2);
     k_norm_check<<<1, 256, 0, s2>>>(partial, NSET, nb, R, (const int*)T.d_seg_blk.p, h->nseg, tol, d_norms,
                                     (int*)h->d_flag.p);
     check_launch("k_norm_check");
@@ -1588,6 +1604,7 @@ static void launch_msd_step(gqt_ham* h, void* p, void* px, int R, const std::vec
     });
     // only |U p| vs |p| is a unitarity check; the px norm changes by construction.
     const double tol = h->prec == GQT_FP64 ? 1e-10 : 1e-5;
+    launch_slot_sums(partial, nb, R, (const int*)T.d_seg_blk.p, h->nseg, 0, 4, -1, s2);
     k_norm_check_msd<<<1, 256, 0, s2>>>(partial, nb, R, (const int*)T.d_seg_blk.p, h->nseg, tol, (int*)h->d_flag.p);
     check_launch("k_norm_check_msd");
   });

@@ -355,10 +355,53 @@ __global__ void k_cheb(Ell<FP64, CH> H, const int* __restrict__ blk, int R, int 
   }
 }
 
-// Deterministic second pass: out[s][r][m] = sum over the segment's CTAs, in
-// CTA order, of partial[m][b][r].  mode 0: complex out (double2), mode 1: real
-// part (double).  Bound check: |mu_m|^2 <= bound_factor |l|^2 |r|^2 (norms
-// from slot slot_norm), failure sets bit 1 of *flag; NaN/Inf sets bit 2.
+// Second pass, part 1: the sum over a segment's CTAs of every slot, in place of the
+// segment's first entry.  One CTA per (slot, segment); its threads stride over the
+// contiguous (CTA, vector) entries, so that a thread keeps one vector (R divides 32),
+// and a fixed tree adds them up (deterministic).  Slots are slot0 .. slot0 + nslots - 1
+// and, when extra >= 0, slot `extra` besides.  One thread walking a segment's entries
+// with a stride of R took 238 us per row at 500 slots of 456 CTAs (863 us at 400 slots
+// of 760 CTAs x 8 vectors); this pass and the combination after it take RED_US us
+// (RED8_US us).
+static __global__ void __launch_bounds__(256) k_slot_sums(double2* partial, int nblocks, int R,
+                                                          const int* __restrict__ seg_blk, int nseg, int slot0,
+                                                          int nslots, int extra) {
+  __shared__ double2 sh[8 * 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long items = (long long)(nslots + (extra >= 0 ? 1 : 0)) * nseg;
+  for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+    const int q = (int)(it / nseg), s = (int)(it % nseg);
+    const int slot = q < nslots ? slot0 + q : extra;
+    const int b0 = seg_blk[s], b1 = seg_blk[s + 1];
+    double2* p = partial + ((size_t)slot * nblocks + b0) * R;
+    const int len = (b1 - b0) * R;
+    double2 v = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int e = threadIdx.x; e < len; e += 256) {
+      const double2 t = p[e];
+      v.x += t.x;
+      v.y += t.y;
+    }
+    for (int off = 16; off >= R; off >>= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+    }
+    if (lane < R) sh[warp * R + lane] = v;
+    __syncthreads();  // every entry has been read
+    if ((int)threadIdx.x < R) {
+      for (int w = 1; w < 8; ++w) {
+        v.x += sh[w * R + threadIdx.x].x;
+        v.y += sh[w * R + threadIdx.x].y;
+      }
+      p[threadIdx.x] = v;
+    }
+    __syncthreads();  // sh is free for the next item
+  }
+}
+
+// Part 2 (after k_slot_sums): out[s][r][m] from the segment sums.  mode 0: complex out
+// (double2), mode 1: real part (double).  Bound check: |mu_m|^2 <= bound_factor |l|^2
+// |r|^2 (norms from slot slot_norm), failure sets bit 1 of *flag; NaN/Inf sets bit 2.
 static __global__ void k_reduce(const double2* __restrict__ partial, int nslots_m, int nblocks, int R,
                          const int* __restrict__ seg_blk, int nseg, int slot_norm, double bound_factor, void* out,
                          int mode, int* __restrict__ flag) {
@@ -367,18 +410,8 @@ static __global__ void k_reduce(const double2* __restrict__ partial, int nslots_
     const int r = (int)(t % R);
     const int m = (int)((t / R) % nslots_m);
     const int s = (int)(t / ((size_t)R * nslots_m));
-    double2 acc = make_double2(0.0, 0.0);
-    double2 nrm = make_double2(0.0, 0.0);
-    for (int b = seg_blk[s]; b < seg_blk[s + 1]; ++b) {
-      const double2 p = partial[((size_t)m * nblocks + b) * R + r];
-      acc.x += p.x;
-      acc.y += p.y;
-      if (slot_norm >= 0) {
-        const double2 q = partial[((size_t)slot_norm * nblocks + b) * R + r];
-        nrm.x += q.x;
-        nrm.y += q.y;
-      }
-    }
+    const int b = seg_blk[s];
+    const double2 acc = partial[((size_t)m * nblocks + b) * R + r];
     const size_t o = ((size_t)s * R + r) * nslots_m + m;
     if (mode == 0)
       reinterpret_cast<double2*>(out)[o] = acc;
@@ -386,6 +419,7 @@ static __global__ void k_reduce(const double2* __restrict__ partial, int nslots_
       reinterpret_cast<double*>(out)[o] = acc.x;
     if (!isfinite(acc.x) || !isfinite(acc.y)) atomicOr(flag, 4);
     if (slot_norm >= 0) {
+      const double2 nrm = partial[((size_t)slot_norm * nblocks + b) * R + r];
       const double bound = nrm.x * nrm.y * bound_factor + 1e-300;
       if (acc.x * acc.x + acc.y * acc.y > bound) atomicOr(flag, 2);
     }
@@ -650,52 +684,46 @@ __global__ void k_cheb_dbl(Ell<FP64, CH> H, const int* __restrict__ blk, int R, 
   }
 }
 
-// Second pass of k_cheb_dbl: mu[s][r][k] = s_k for k < 2, 2 s_k - s_{k mod 2} otherwise,
-// each s summed over the segment's CTAs in CTA order.  Bound |mu_k| <= (1+tol) mu_0.
+// k_reduce for the product identities (after k_slot_sums): mu[s][r][k] = s_k for k < 2,
+// 2 s_k - s_{k mod 2} otherwise.  slot_norm < 0: l = r, |mu_k| <= mu_0 (1 + tol);
+// otherwise slot_norm holds (|l|^2, |r|^2) and |mu_k| <= |l| |r| (1 + tol).
 static __global__ void k_reduce_dbl(const double2* __restrict__ partial, int M, int nblocks, int R,
                              const int* __restrict__ seg_blk, int nseg, double bound_factor, double* __restrict__ out,
                              int* __restrict__ flag, int slot_norm = -1) {
-  // slot_norm < 0: l = r, |mu_k| <= mu_0 (1 + tol); otherwise slot_norm holds
-  // (|l|^2, |r|^2) and |mu_k| <= |l| |r| (1 + tol).
   const size_t total = (size_t)nseg * R * M;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
     const int r = (int)(t % R);
     const int k = (int)((t / R) % M);
     const int s = (int)(t / ((size_t)R * M));
-    double sk = 0.0, s0 = 0.0, sp = 0.0, nl = 0.0, nr = 0.0;
-    const int kp = k & 1;
-    for (int b = seg_blk[s]; b < seg_blk[s + 1]; ++b) {
-      sk += partial[((size_t)k * nblocks + b) * R + r].x;
-      s0 += partial[((size_t)0 * nblocks + b) * R + r].x;
-      sp += partial[((size_t)kp * nblocks + b) * R + r].x;
-      if (slot_norm >= 0) {
-        const double2 q = partial[((size_t)slot_norm * nblocks + b) * R + r];
-        nl += q.x;
-        nr += q.y;
-      }
-    }
+    const size_t b = (size_t)seg_blk[s];
+    const double sk = partial[((size_t)k * nblocks + b) * R + r].x;
+    const double sp = partial[((size_t)(k & 1) * nblocks + b) * R + r].x;
     const double mu = (k < 2) ? sk : 2.0 * sk - sp;
     out[((size_t)s * R + r) * M + k] = mu;
     if (!isfinite(mu)) atomicOr(flag, 4);
-    const double bound = (slot_norm >= 0 ? sqrt(nl * nr) : s0) * bound_factor + 1e-300;
-    if (fabs(mu) > bound) atomicOr(flag, 2);
+    double top;
+    if (slot_norm >= 0) {
+      const double2 q = partial[((size_t)slot_norm * nblocks + b) * R + r];
+      top = sqrt(q.x * q.y);
+    } else {
+      top = partial[b * R + r].x;
+    }
+    if (fabs(mu) > top * bound_factor + 1e-300) atomicOr(flag, 2);
   }
 }
 
-// Norm check of an evolution: slots q (before) and NSET + q (after) hold the
-// partial squared norms of set q.  | |after| - |before| | > tol |before| sets
-// bit 3 of *flag.  norms (optional) receives [nseg][R][NSET][2] squared norms.
+// Norm check of an evolution (after k_slot_sums): slots q (before) and NSET + q (after)
+// hold the squared norms of set q.  | |after| - |before| | > tol |before| sets bit 3 of
+// *flag.  norms (optional) receives [nseg][R][NSET][2] squared norms.
 static __global__ void k_norm_check(const double2* __restrict__ partial, int nset, int nblocks, int R,
                              const int* __restrict__ seg_blk, int nseg, double tol, double* __restrict__ norms,
                              int* __restrict__ flag) {
   const int total = nseg * R * nset;
   for (int t = threadIdx.x; t < total; t += blockDim.x) {
     const int q = t % nset, r = (t / nset) % R, s = t / (nset * R);
-    double a = 0.0, z = 0.0;
-    for (int b = seg_blk[s]; b < seg_blk[s + 1]; ++b) {
-      a += partial[((size_t)q * nblocks + b) * R + r].x;
-      z += partial[((size_t)(nset + q) * nblocks + b) * R + r].x;
-    }
+    const size_t b = (size_t)seg_blk[s];
+    const double a = partial[((size_t)q * nblocks + b) * R + r].x;
+    const double z = partial[((size_t)(nset + q) * nblocks + b) * R + r].x;
     if (norms) {
       norms[(size_t)t * 2] = a;
       norms[(size_t)t * 2 + 1] = z;
@@ -705,18 +733,17 @@ static __global__ void k_norm_check(const double2* __restrict__ partial, int nse
   }
 }
 
-// MSD step: slot 0 = |p|^2 before, slot 2 = |U p|^2 after (slot 3 = |px|^2, unchecked).
+// MSD step (after k_slot_sums): slot 0 = |p|^2 before, slot 2 = |U p|^2 after (slot 3 =
+// |px|^2, unchecked).
 static __global__ void k_norm_check_msd(const double2* __restrict__ partial, int nblocks, int R,
                                  const int* __restrict__ seg_blk, int nseg, double tol, int* __restrict__ flag) {
   const int total = nseg * R;
   for (int t = threadIdx.x; t < total; t += blockDim.x) {
     const int r = t % R, s = t / R;
-    double a = 0.0, z = 0.0, x = 0.0;
-    for (int b = seg_blk[s]; b < seg_blk[s + 1]; ++b) {
-      a += partial[((size_t)0 * nblocks + b) * R + r].x;
-      z += partial[((size_t)2 * nblocks + b) * R + r].x;
-      x += partial[((size_t)3 * nblocks + b) * R + r].x;
-    }
+    const size_t b = (size_t)seg_blk[s];
+    const double a = partial[b * R + r].x;
+    const double z = partial[((size_t)2 * nblocks + b) * R + r].x;
+    const double x = partial[((size_t)3 * nblocks + b) * R + r].x;
     if (!isfinite(z) || !isfinite(x)) atomicOr(flag, 4);
     if (fabs(sqrt(z) - sqrt(a)) > tol * sqrt(a) + 1e-300) atomicOr(flag, 8);
   }

@@ -38,6 +38,7 @@ using gqt_na::gqt::Ell;
 using gqt_na::gqt::Prec;
 using gqt_na::gqt::k_cheb;
 using gqt_na::gqt::k_reduce;
+using gqt_na::gqt::k_slot_sums;
 
 // The scratch array: every GPU that loads the library holds these bytes until
 // the process exits.  Its name is only a host-side stand-in in host code; the
@@ -149,6 +150,8 @@ void run(const gqt_ham* h, const void* phi, int R, int rs, int M, double* d_mu, 
   const double tol = FP64 ? 1e-6 : 1e-3;
   const size_t total = (size_t)R * M;
   const int rb = (int)std::min<size_t>((total + 255) / 256, 4096);
+  k_slot_sums<<<M + 1, 256, 0, st>>>(partial, nb, R, seg_blk, 1, 0, M, slot_norm);
+  gqt::check_launch("k_slot_sums(no-alloc)");
   k_reduce<<<rb, 256, 0, st>>>(partial, M, nb, R, seg_blk, 1, slot_norm, (1.0 + tol) * (1.0 + tol), d_mu, 1, flag);
   gqt::check_launch("k_reduce(no-alloc)");
 }
