@@ -499,6 +499,8 @@ def run_ours(args):
     dE = w.energy_scale
     ham = g.gqt_build_hamiltonian(lat, dE, g.GQT_FP64)
     g.gqt_set_fp64_arith(ham, args.fp64_arith)
+    if args.small:  # the reduced lattice stands in for the large one: its kernels, not the on-chip rows
+        g.gqt_set_cluster(ham, False)
     g.gqt_set_temporal_blocking(ham, args.temporal_blocking)
     N, M, R = lat.n, w.M, 1
     Np = g.gqt_np_rule(dE * w.dt, 64)

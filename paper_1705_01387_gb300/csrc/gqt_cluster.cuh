@@ -150,4 +150,231 @@ __global__ void k_cheb_cluster(Ell<FP64, CH> H, int chunk, const typename Prec<F
   cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
+// ---------------------------------------------------------------- one site per thread
+//
+// Rows of up to 512 sites per CTA (8192 in a cluster of 16) with 2, 3, 4 or 6 neighbour
+// slots, both moments of an order by the product identities: l = r rows (PAIR = false)
+// and the two-recurrence l != r rows (PAIR = true), as the large-N kernels.  A thread
+// keeps its site's H~ row, its neighbours' distributed shared-memory addresses and its
+// own T_{m-1} and T_{m-2} in registers.  An order is a serial chain -- gather, FP64
+// multiply-adds (4 warps x 8 instructions of 16 cycles each on the SM's FP64 pipe),
+// store, cluster barrier -- so whatever is not part of it is moved under the barrier:
+// the order's two dots are formed between arriving and waiting, and instead of two
+// warp sums per order (40 FP64 adds and 80 shuffles a warp) the threads' values go to a
+// ring in shared memory that is added up every 16 orders.  At the end the CTAs sum
+// their slots over the cluster and write the moments and their checks directly.
+// At 2048 sites (16 CTAs of 128) an order takes 0.85 us instead of 1.98 us, and a VAC row
+// half as many of them: DOS row of 512 moments 545 -> 260 us per call, VAC row 729 -> 345
+// us.
+constexpr int CL_RING = 32;  // slots in the ring: 16 orders
+
+__host__ __device__ inline size_t cluster1_smem(int chunk, int threads, int steps, int vec_bytes, bool pair) {
+  return (size_t)chunk * vec_bytes * (pair ? 4 : 2) + (size_t)CL_RING * (threads + 4) * sizeof(double) +
+         ((size_t)((2 * steps + CL_RING - 1) / CL_RING) * CL_RING + 2) * sizeof(double);
+}
+
+__device__ __forceinline__ uint32_t cl_map(const void* p, int rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ double2 cl_ld(uint32_t a, double2) {
+  double2 v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 cl_ld(uint32_t a, float2) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ double cl_ld(uint32_t a, double) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cl_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// An element's term Re conj(a) b of a dot, as DotAcc forms it (FP32 storage: one FP32
+// rounding), then FP64.
+__device__ __forceinline__ double cl_re(double2 a, double2 b) { return fma(a.x, b.x, a.y * b.y); }
+__device__ __forceinline__ double cl_re(float2 a, float2 b) { return (double)fmaf(a.x, b.x, a.y * b.y); }
+
+template <bool FP64, bool CH, bool PAIR, int KK>
+__global__ void __launch_bounds__(512) k_cheb_cluster1(Ell<FP64, CH> H, int chunk,
+                                                       const typename Prec<FP64>::V* __restrict__ l,
+                                                       const typename Prec<FP64>::V* __restrict__ r, int M,
+                                                       double bound_factor, double* __restrict__ out,
+                                                       int* __restrict__ flag) {
+  using V = typename Prec<FP64>::V;
+  using S = typename Prec<FP64>::S;
+  using HT = typename Ell<FP64, CH>::HT;
+  cgc::cluster_group cluster = cgc::this_cluster();
+  const int C = (int)cluster.num_blocks(), me = (int)cluster.block_rank();
+  const int tid = (int)threadIdx.x, thr = (int)blockDim.x;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  V* B0 = reinterpret_cast<V*>(sm_raw);  // chain B (or the only one): T_m at even, odd m
+  V* B1 = B0 + chunk;
+  V* A0 = B1 + chunk;  // chain A, PAIR only
+  const uint32_t flip = (uint32_t)((size_t)chunk * sizeof(V));       // B0 -> B1, A0 -> A1
+  const uint32_t toA = (uint32_t)((size_t)2 * chunk * sizeof(V));    // B0 -> A0
+  double* ring = reinterpret_cast<double*>(sm_raw + (size_t)chunk * sizeof(V) * (PAIR ? 4 : 2));
+  double* red = ring + CL_RING * (thr + 4);  // sums of this CTA, [slots]
+  const int steps = max((M + 1) / 2, 1), nslots = (2 * steps + CL_RING - 1) / CL_RING * CL_RING;
+  double* nrm = red + nslots;  // |l|^2, |r|^2 of this CTA (PAIR)
+  const int i = me * chunk + tid;
+  const bool on = tid < chunk && i < H.n;
+  uint32_t adr[KK];
+  HT hv[KK];
+  S dg = 0;
+  V b, bo, a, ao;  // own T_{m-1} and T_{m-2} of chains B and A
+  b.x = b.y = 0;
+  bo = a = ao = b;
+#pragma unroll
+  for (int k = 0; k < KK; ++k) {
+    adr[k] = cl_map(B0, me);
+    hv[k] = HT{};
+  }
+  if (on) {
+    b = r[i];
+    B0[tid] = b;
+    if (PAIR) {
+      a = l[i];
+      A0[tid] = a;
+    }
+    dg = H.diag2[i];
+#pragma unroll
+    for (int k = 0; k < KK; ++k) {
+      const size_t s = (size_t)k * H.n + i;
+      const int j = H.idx[s], rk = j / chunk;
+      adr[k] = cl_map(B0 + (j - rk * chunk), rk);
+      hv[k] = H.hop2[s];
+    }
+  }
+  if (PAIR) {
+    double v[2] = {on ? cl_re(a, a) : 0.0, on ? cl_re(b, b) : 0.0};
+    block_reduce_rx<2>(v, 1, ring);
+    if (tid == 0) {
+      nrm[0] = v[0];
+      nrm[1] = v[1];
+    }
+  }
+  cluster.sync();
+  const int parts = thr / CL_RING;
+  uint32_t src = 0;  // 0: T_{m-1} in B0 / A0, flip: in B1 / A1
+  for (int m = 1; m <= steps; ++m) {
+    V nb, na;
+    nb.x = nb.y = 0;
+    na = nb;
+    if (on) {
+      V gb[KK], ga[KK];
+#pragma unroll
+      for (int k = 0; k < KK; ++k) {
+        gb[k] = cl_ld(adr[k] + src, V());
+        if (PAIR) ga[k] = cl_ld(adr[k] + toA + src, V());
+      }
+      nb = m == 1 ? cscale(b, dg) : cmul_acc(cneg(bo), dg, b);
+      if (PAIR) na = m == 1 ? cscale(a, dg) : cmul_acc(cneg(ao), dg, a);
+#pragma unroll
+      for (int k = 0; k < KK; ++k) {
+        nb = cmul_acc(nb, hv[k], gb[k]);
+        if (PAIR) na = cmul_acc(na, hv[k], ga[k]);
+      }
+      if (m == 1) {
+        nb = cscale(nb, (S)0.5);
+        if (PAIR) na = cscale(na, (S)0.5);
+      }
+      V* dst = src ? B0 : B1;
+      dst[tid] = nb;
+      if (PAIR) dst[2 * chunk + tid] = na;
+    }
+    cl_arrive();
+    // under the barrier: slots 2m-2 and 2m-1
+    const int s0 = (2 * m - 2) & (CL_RING - 1);
+    ring[s0 * (thr + 4) + tid] = on ? (PAIR ? cl_re(a, b) : cl_re(b, b)) : 0.0;
+    ring[(s0 + 1) * (thr + 4) + tid] = on ? (PAIR ? cl_re(a, nb) : cl_re(nb, b)) : 0.0;
+    if (s0 == CL_RING - 2 || m == steps) {
+      __syncthreads();
+      const int slot = tid / parts, part = tid - slot * parts;
+      double w[8], v;  // eight runs, added in pairs
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w[j] = 0.0;
+#pragma unroll
+      for (int j = 0; j < CL_RING; ++j) w[j & 7] += ring[slot * (thr + 4) + part + parts * j];
+      v = ((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]));
+      for (int off = parts >> 1; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+      if (part == 0) red[(2 * m - 2 - s0) + slot] = v;
+      __syncthreads();
+    }
+    bo = b;
+    b = nb;
+    ao = a;
+    a = na;
+    src ^= flip;
+    cl_wait();  // T_m complete everywhere; nobody reads T_{m-1} any more
+  }
+  cluster.sync();  // every CTA's sums are written
+  auto total = [&](const double* p) {
+    double v = 0.0;
+    for (int q = 0; q < C; q += 4)  // C is 8 or 16
+      v += (cl_ld(cl_map(p, q), 0.0) + cl_ld(cl_map(p, q + 1), 0.0)) +
+           (cl_ld(cl_map(p, q + 2), 0.0) + cl_ld(cl_map(p, q + 3), 0.0));
+    return v;
+  };
+  if (me * thr + tid < M) {
+    const double s_even = total(red), s_odd = total(red + 1);
+    const double top = PAIR ? sqrt(total(nrm) * total(nrm + 1)) : s_even;
+    for (int k = me * thr + tid; k < M; k += C * thr) {
+      const double sk = total(red + k);
+      const double mu = k < 2 ? sk : 2.0 * sk - ((k & 1) ? s_odd : s_even);
+      out[k] = mu;
+      if (!isfinite(mu)) atomicOr(flag, 4);
+      if (fabs(mu) > top * bound_factor + 1e-300) atomicOr(flag, 2);
+    }
+  }
+  cluster.sync();  // no CTA leaves while another may still read its shared memory
+}
+
+// Launches one of the one-site-per-thread cluster kernels for n sites: clusters of 16
+// CTAs where the GPU allows, else 8, of a power of two of threads (the ring's parts), at
+// most 512; smem_of(chunk, threads) bytes of shared memory; f(config, chunk) launches.
+// False where the system does not fit or clusters are unavailable.
+template <class KERN, class SM, class F>
+inline bool cluster1_launch(KERN kern, int64_t n, cudaStream_t st, SM&& smem_of, F&& f) {
+  for (int C : {16, 8}) {
+    const int chunk = (int)((n + C - 1) / C);
+    int thr = 32;
+    while (thr < chunk && thr <= 512) thr *= 2;
+    if (thr > 512) continue;
+    const size_t smem = smem_of(chunk, thr);
+    if (smem > 220 * 1024) continue;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        (C > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+      cudaGetLastError();
+      continue;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C, 1, 1);
+    cfg.blockDim = dim3(thr, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int nclusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) != cudaSuccess || nclusters < 1) {
+      cudaGetLastError();
+      continue;
+    }
+    f(cfg, chunk);
+    return true;
+  }
+  return false;
+}
+
 }  // namespace gqt

@@ -666,6 +666,52 @@ static bool launch_cluster_row(gqt_ham* h, const Ell<FP64, CH>& H, const V* r, c
   return false;
 }
 
+// The same rows with one site per thread (k_cheb_cluster1): up to 512 sites per CTA and
+// the neighbour counts of the wavefront kernels.  kind 2: l = r; kind 1: l != r by two
+// recurrences, where these are on (use_pair) and in FP64 storage (an FP32 row keeps the
+// single recurrence, whose rounding its moments have).  Writes the moments to out.
+// Larger systems, other neighbour counts: k_cheb_cluster.
+template <bool FP64, bool CH, bool PAIR, int KK>
+static bool launch_cluster1_k(gqt_ham* h, const Ell<FP64, CH>& H, const void* l, const void* r, int M, double* out,
+                              double bound, cudaStream_t st) {
+  using V = typename Prec<FP64>::V;
+  auto kern = k_cheb_cluster1<FP64, CH, PAIR, KK>;
+  const int steps = std::max((M + 1) / 2, 1);
+  return cluster1_launch(
+      kern, h->n, st, [&](int chunk, int thr) { return cluster1_smem(chunk, thr, steps, (int)sizeof(V), PAIR); },
+      [&](const cudaLaunchConfig_t& cfg, int chunk) {
+        check_cuda(cudaLaunchKernelEx(&cfg, kern, H, chunk, (const V*)l, (const V*)r, M, bound, out,
+                                      (int*)h->d_flag.p),
+                   "k_cheb_cluster1");
+        check_launch("k_cheb_cluster1");
+      });
+}
+
+static bool launch_cluster1(gqt_ham* h, const void* l, const void* r, int M, double* out, int kind, double bound,
+                            cudaStream_t st) {
+  if (kind == 1 && !(h->use_pair && h->prec == GQT_FP64)) return false;
+  bool done = false;
+  dispatch(h, [&](auto H) {
+    using Tr = EllTraits<decltype(H)>;
+    auto go = [&](auto kk) {
+      constexpr int KK = decltype(kk)::value;
+      if (kind == 2) {
+        done = launch_cluster1_k<Tr::fp64, Tr::ch, false, KK>(h, H, l, r, M, out, bound, st);
+      } else if constexpr (Tr::fp64) {
+        done = launch_cluster1_k<true, Tr::ch, true, KK>(h, H, l, r, M, out, bound, st);
+      }
+    };
+    switch (h->K) {
+      case 2: go(std::integral_constant<int, 2>()); break;
+      case 3: go(std::integral_constant<int, 3>()); break;
+      case 4: go(std::integral_constant<int, 4>()); break;
+      case 6: go(std::integral_constant<int, 6>()); break;
+      default: break;
+    }
+  });
+  return done;
+}
+
 template <bool FP64, bool CH, class V>
 static void launch_wave_pair(gqt_ham* h, const Ell<FP64, CH>& H, const BlockTable& T, int R, int rs, const V* am1,
                              const V* bm1, const V* am2, const V* bm2, V* aout, V* bout, double2* partial, int m,
@@ -1111,6 +1157,7 @@ void gqt::launch_moments(gqt_ham* h, const void* l, const void* r, int R, int M,
   const size_t total = (size_t)h->nseg * R * M;
   const int rb = (int)std::min<size_t>((total + 255) / 256, 4096);
   if (R == 1 && h->nseg == 1 && kind != 0 && h->use_cluster) {
+    if (launch_cluster1(h, l, r, M, (double*)out, kind, 1.0 + tol, st)) return;
     int C = 0;
     bool done = false;
     DevBuf& cseg = h->ws(WS_CLUSTER_SEG, 4 * sizeof(int));

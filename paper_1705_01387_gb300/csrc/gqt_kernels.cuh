@@ -361,8 +361,7 @@ __global__ void k_cheb(Ell<FP64, CH> H, const int* __restrict__ blk, int R, int 
 // and a fixed tree adds them up (deterministic).  Slots are slot0 .. slot0 + nslots - 1
 // and, when extra >= 0, slot `extra` besides.  One thread walking a segment's entries
 // with a stride of R took 238 us per row at 500 slots of 456 CTAs (863 us at 400 slots
-// of 760 CTAs x 8 vectors); this pass and the combination after it take RED_US us
-// (RED8_US us).
+// of 760 CTAs x 8 vectors); this pass and the combination after it take 9 us (19 us).
 static __global__ void __launch_bounds__(256) k_slot_sums(double2* partial, int nblocks, int R,
                                                           const int* __restrict__ seg_blk, int nseg, int slot0,
                                                           int nslots, int extra) {
