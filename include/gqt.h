@@ -354,7 +354,8 @@ gqt_status gqt_autotune(gqt_ham* ham, int R, int* threads, int* blocks_per_sm, i
  * a row's two Chebyshev vectors, l and the H~ rows fit in the shared memory of
  * one thread-block cluster (16 CTAs where the GPU allows, else 8), the whole row
  * runs as one launch; vectors are exchanged through distributed shared memory
- * and orders are separated by hardware cluster barriers.  0 keeps the
+ * and orders are separated by hardware cluster barriers.  FP64 handles of up to 8192
+ * sites also run evolutions of up to 128 orders this way.  0 keeps the
  * one-launch-per-order path. */
 gqt_status gqt_set_cluster(gqt_ham* ham, int enable);
 
@@ -363,7 +364,8 @@ gqt_status gqt_set_cluster(gqt_ham* ham, int enable);
  * mu_2k = 2 Re <A_k|B_k> - mu_0 and mu_2k+1 = 2 Re <A_k|B_k+1> - mu_1
  * (Chebyshev product identities, H~ Hermitian), so each step streams H~ once for
  * two moments.  Applies to the wavefront kernels, one element per thread or
- * the multi-vector form (not the chunk-ordered variant 0 or cluster rows).  0
+ * the multi-vector form, and to cluster rows of FP64 handles (not the chunk-ordered
+ * variant 0).  0
  * runs one recurrence on r with a dot against l per order. */
 gqt_status gqt_set_vac_pair(gqt_ham* ham, int enable);
 
@@ -379,8 +381,10 @@ gqt_status gqt_set_vac_pair(gqt_ham* ham, int enable);
  *     each FP64 one, so mode 1 is bound by HBM instead of the FP64 pipe.  The
  *     first call in mode 1 splits 2H~ into pairs (K n (8 or 16) + 8 n bytes of
  *     device memory held by the handle).
- * Other values: GQT_EINVAL.  Evolution, velocity, adjoint and Hall kernels, and
- * R > 1 rows, always use the FP64 pipe. */
+ *     Evolution orders (R = 1) use the same pairs, except where a whole expansion
+ *     runs on one thread-block cluster (gqt_set_cluster), which is FP64.
+ * Other values: GQT_EINVAL.  Velocity, adjoint and Hall kernels, and R > 1 rows,
+ * always use the FP64 pipe (the Hall contraction: see gqt_set_kb_contraction). */
 gqt_status gqt_set_fp64_arith(gqt_ham* ham, int mode);
 
 /* Temporal blocking of the moment rows (Eq. 21 advanced two orders per

@@ -19,13 +19,15 @@
 // (a contraction would break the error-free transformations).
 //
 // Storage: the chain vectors T_k are float4 per complex element
-// (re.hi, re.lo, im.hi, im.lo); the caller's input vectors stay complex128 and
-// are split on the first order only.  The Hamiltonian's 2H~ (real hoppings:
-// float2 (hi, lo) per slot; complex: float4) and 2U/dE (float2) are split once
-// per handle from its FP64 arrays.  Moment partial sums leave each thread as
-// FP64 (hi + lo) and are reduced in FP64 as in the FP64 kernels, into the same
-// partial slots, so k_reduce_dbl combines them unchanged.
+// (re.hi, im.hi, re.lo, im.lo); the caller's input vectors stay complex128 and
+// are split once per row or evolution.  The Hamiltonian's 2H~ (real hoppings:
+// float2 (hi, lo) per slot; complex: float4 (re.hi, re.lo, im.hi, im.lo)) and 2U/dE
+// (float2) are split once per handle from its FP64 arrays.  Moment partial sums leave
+// each thread as FP64 (hi + lo) and are reduced in FP64 as in the FP64 kernels, into
+// the same partial slots, so k_reduce_dbl combines them unchanged.
 #pragma once
+
+#include "gqt_kernels.cuh"
 
 namespace gqt {
 
@@ -58,15 +60,139 @@ __device__ __forceinline__ float2 df_split(double x) {
   const float h = __double2float_rn(x);
   return make_float2(h, __double2float_rn(x - (double)h));
 }
+// A complex FP64 element as a chain element (re.hi, im.hi, re.lo, im.lo).
 __device__ __forceinline__ float4 df_split(double2 z) {
+  const float2 a = df_split(z.x), b = df_split(z.y);
+  return make_float4(a.x, b.x, a.y, b.y);
+}
+// df_split by integer operations: the FP64 pipe (four operations a value) took 1.9 ms
+// for two vectors of 16.8M elements and their neighbours.  hi is x rounded to 24 bits
+// (half up; the pair's sum is the same where a tie rounds the other way), the rest a
+// signed integer of 29 bits, rounded to FP32 and scaled.  Values outside 2^-73 .. 2^126,
+// whose parts could leave the normal FP32 range, take df_split.
+__device__ __forceinline__ float2 df_split_int(double x) {
+  const uint64_t u = (uint64_t)__double_as_longlong(x);
+  const uint32_t top = (uint32_t)(u >> 32), ex = (top >> 20) & 0x7FFu;
+  if (ex - 950u > 199u) return (u << 1) == 0 ? make_float2(0.f, 0.f) : df_split(x);
+  const uint32_t sign = top & 0x80000000u, low = (uint32_t)u & 0x1FFFFFFFu;
+  const uint64_t m = (u & 0x7FFFFFFFFFFFFFFFull) + (1u << 28);
+  const float hi = __uint_as_float((uint32_t)((m >> 29) - (896u << 23)) | sign);
+  const int r = (int)low - ((low >> 28) ? (1 << 29) : 0);
+  const float lo = __fmul_rn((float)r, __uint_as_float(((ex - 948u) << 23) | sign));
+  return make_float2(hi, lo);
+}
+
+// A complex FP64 coefficient as (re.hi, re.lo, im.hi, im.lo).
+__device__ __forceinline__ float4 df_split_coef(double2 z) {
   const float2 a = df_split(z.x), b = df_split(z.y);
   return make_float4(a.x, a.y, b.x, b.y);
 }
-__device__ __forceinline__ double df_value(float h, float l) { return (double)h + (double)l; }
+// A float widened to double with integer operations (exact), as the conversion
+// instruction does on the FP64 pipe at 1/64 of the FP32 rate; zeros, denormals,
+// infinities and NaNs take the instruction (in a function of its own, so that it is
+// not executed under a predicate for every value).
+static __device__ __noinline__ double f2d_special(float x) { return (double)x; }
+__device__ __forceinline__ double f2d(float x) {
+  const uint32_t u = __float_as_uint(x);
+  if (((u >> 23) + 1u & 0xFFu) < 2u) return f2d_special(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double df_value(float h, float l) { return f2d(h) + f2d(l); }
 
-// (sh, sl) += (ah, al) * (bh, bl), the sum kept unnormalised (sl collects the
-// TwoSum error and the low part of the product).
-__device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, float al, float bh, float bl) {
+// Operations on the (re, im) words, each rounded to nearest.
+__device__ __forceinline__ float2 f2_add(float2 a, float2 b) {
+  return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
+__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) {
+  return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
+}
+__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
+  return make_float2(__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {
+  return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y));
+}
+__device__ __forceinline__ float2 f2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 f2_both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 f2_hi(float4 x) { return make_float2(x.x, x.y); }
+__device__ __forceinline__ float2 f2_lo(float4 x) { return make_float2(x.z, x.w); }
+
+// Product of pairs: p = fl(ah bh), e its error and the cross terms.
+__device__ __forceinline__ void df_prod(float2& p, float2& e, float2 ah, float2 al, float2 bh, float2 bl) {
+  p = f2_mul(ah, bh);
+  e = f2_fma(ah, bh, f2_neg(p));
+  e = f2_fma(ah, bl, e);
+  e = f2_fma(al, bh, e);
+}
+
+// Complex accumulator (h: re.hi, im.hi; l: re.lo, im.lo), unnormalised: l collects the
+// TwoSum errors and the low parts of the products.
+struct DfC {
+  float2 h, l;
+};
+
+__device__ __forceinline__ DfC dfc_zero() { return DfC{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+__device__ __forceinline__ DfC dfc_of(float4 a) { return DfC{f2_hi(a), f2_lo(a)}; }
+
+// a += (ah, al) * (bh, bl)
+__device__ __forceinline__ void df_mac(DfC& a, float2 ah, float2 al, float2 bh, float2 bl) {
+  float2 p, e;
+  df_prod(p, e, ah, al, bh, bl);
+  const float2 s = f2_add(a.h, p);
+  const float2 v = f2_sub(s, a.h);
+  const float2 t = f2_add(f2_sub(a.h, f2_sub(s, v)), f2_sub(p, v));
+  a.h = s;
+  a.l = f2_add(a.l, f2_add(t, e));
+}
+
+// a = (ah, al) * (bh, bl) - x, as df_mac on an accumulator holding -x
+__device__ __forceinline__ DfC df_mul_sub(float2 ah, float2 al, float2 bh, float2 bl, float4 x) {
+  float2 p, e;
+  df_prod(p, e, ah, al, bh, bl);
+  const float2 xh = f2_hi(x);
+  const float2 s = f2_sub(p, xh);
+  const float2 v = f2_add(s, xh);
+  const float2 t = f2_sub(f2_sub(p, v), f2_add(xh, f2_sub(s, v)));
+  return DfC{s, f2_sub(f2_add(t, e), f2_lo(x))};
+}
+
+// a += x (TwoSum of the high words, the low words and the TwoSum error added into l)
+__device__ __forceinline__ void df_add(DfC& a, float4 x) {
+  const float2 xh = f2_hi(x);
+  const float2 s = f2_add(a.h, xh);
+  const float2 v = f2_sub(s, a.h);
+  const float2 t = f2_add(f2_sub(a.h, f2_sub(s, v)), f2_sub(xh, v));
+  a.h = s;
+  a.l = f2_add(a.l, f2_add(f2_lo(x), t));
+}
+
+// acc += c * x, c real pair
+__device__ __forceinline__ void dfc_mac(DfC& a, float2 c, float4 x) {
+  df_mac(a, f2_both(c.x), f2_both(c.y), f2_hi(x), f2_lo(x));
+}
+// acc += i c * x, c real pair: (re, im) += c (-im, re)
+__device__ __forceinline__ void dfc_mac_i(DfC& a, float2 c, float4 x) {
+  df_mac(a, make_float2(-c.x, c.x), make_float2(-c.y, c.y), make_float2(x.y, x.x), make_float2(x.w, x.z));
+}
+// acc += c * x, c complex pair (re.hi, re.lo, im.hi, im.lo)
+__device__ __forceinline__ void dfc_mac(DfC& a, float4 c, float4 x) {
+  dfc_mac(a, make_float2(c.x, c.y), x);
+  dfc_mac_i(a, make_float2(c.z, c.w), x);
+}
+
+// Normalised pairs of an accumulator (TwoSum of the two words).
+__device__ __forceinline__ float4 dfc_out(const DfC& a, bool half) {
+  float2 s = f2_add(a.h, a.l);
+  const float2 v = f2_sub(s, a.h);
+  float2 t = f2_add(f2_sub(a.h, f2_sub(s, v)), f2_sub(a.l, v));
+  if (half) {  // exact scaling of both words (T_1 = H~ T_0 from 2H~)
+    s = f2_mul(s, make_float2(0.5f, 0.5f));
+    t = f2_mul(t, make_float2(0.5f, 0.5f));
+  }
+  return make_float4(s.x, s.y, t.x, t.y);
+}
+
+__device__ __forceinline__ void df_mac1(float& sh, float& sl, float ah, float al, float bh, float bl) {
   const float p = __fmul_rn(ah, bh);
   float e = __fmaf_rn(ah, bh, -p);
   e = __fmaf_rn(ah, bl, e);
@@ -77,54 +203,15 @@ __device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, float al,
   sh = s;
   sl = __fadd_rn(sl, __fadd_rn(t, e));
 }
-
-// (sh, sl) -> normalised pair (TwoSum of the two words).
-__device__ __forceinline__ float2 df_norm(float sh, float sl) {
-  const float s = __fadd_rn(sh, sl);
-  const float v = __fsub_rn(s, sh);
-  const float t = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, v)), __fsub_rn(sl, v));
-  return make_float2(s, t);
-}
-
-// Complex accumulator (re: x, y; im: z, w as hi, lo), unnormalised.
-struct DfC {
-  float rh, rl, ih, il;
-};
-
-__device__ __forceinline__ DfC dfc_zero() { return DfC{0.f, 0.f, 0.f, 0.f}; }
-__device__ __forceinline__ DfC dfc_neg(float4 a) { return DfC{-a.x, -a.y, -a.z, -a.w}; }
-
-// acc += c * x, c real pair
-__device__ __forceinline__ void dfc_mac(DfC& a, float2 c, float4 x) {
-  df_mac(a.rh, a.rl, c.x, c.y, x.x, x.y);
-  df_mac(a.ih, a.il, c.x, c.y, x.z, x.w);
-}
-// acc += c * x, c complex pair (re.hi, re.lo, im.hi, im.lo)
-__device__ __forceinline__ void dfc_mac(DfC& a, float4 c, float4 x) {
-  df_mac(a.rh, a.rl, c.x, c.y, x.x, x.y);
-  df_mac(a.rh, a.rl, -c.z, -c.w, x.z, x.w);
-  df_mac(a.ih, a.il, c.x, c.y, x.z, x.w);
-  df_mac(a.ih, a.il, c.z, c.w, x.x, x.y);
-}
-
-__device__ __forceinline__ float4 dfc_out(const DfC& a, bool half) {
-  float2 r = df_norm(a.rh, a.rl), i = df_norm(a.ih, a.il);
-  if (half) {  // exact scaling of both words (T_1 = H~ T_0 from 2H~)
-    r.x *= 0.5f;
-    r.y *= 0.5f;
-    i.x *= 0.5f;
-    i.y *= 0.5f;
-  }
-  return make_float4(r.x, r.y, i.x, i.y);
-}
-
-// Per-thread real dot accumulator: sum of Re conj(a) b or |a|^2 over the
-// thread's elements, as an unnormalised pair; FP64 once per thread.
+// Per-thread real dot accumulator: sum of Re conj(a) b or |a|^2 over the thread's
+// elements, as one unnormalised pair; FP64 once per thread.  (Separate pairs for the
+// real and imaginary products cost the l = r orders their registers: 15.0 -> 18.4 us
+// at 1M sites of a square lattice.)
 struct DfDot {
   float h = 0.f, l = 0.f;
   __device__ __forceinline__ void add_re(float4 a, float4 b) {
-    df_mac(h, l, a.x, a.y, b.x, b.y);
-    df_mac(h, l, a.z, a.w, b.z, b.w);
+    df_mac1(h, l, a.x, a.z, b.x, b.z);
+    df_mac1(h, l, a.y, a.w, b.y, b.w);
   }
   __device__ __forceinline__ void add_norm(float4 a) { add_re(a, a); }
   __device__ __forceinline__ double get() const { return df_value(h, l); }
@@ -140,7 +227,7 @@ __global__ void k_split_hamiltonian(long long nslots, const void* __restrict__ h
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < nslots; s += stride) {
     if (CH)
-      ((float4*)hop_df)[s] = df_split(((const double2*)hop64)[s]);
+      ((float4*)hop_df)[s] = df_split_coef(((const double2*)hop64)[s]);
     else
       ((float2*)hop_df)[s] = df_split(((const double*)hop64)[s]);
   }
@@ -158,65 +245,67 @@ __global__ void k_split_xhop(long long nslots, const void* __restrict__ hop64, c
     const double d = -dx[s];
     if (CH) {
       const double2 h = ((const double2*)hop64)[s];
-      ((float4*)xhop_df)[s] = df_split(make_double2(d * h.x, d * h.y));
+      ((float4*)xhop_df)[s] = df_split_coef(make_double2(d * h.x, d * h.y));
     } else {
       ((float2*)xhop_df)[s] = df_split(d * ((const double*)hop64)[s]);
     }
   }
 }
 
-// ---------------------------------------------------------------- moment rows
-
-// Element e's chain value: a pair vector, or (first order) the caller's FP64
-// vector split on the fly.
-template <bool IN64>
-__device__ __forceinline__ float4 df_load(const void* v, size_t e) {
-  if (IN64) return df_split(__ldg((const double2*)v + e));
-  return __ldg((const float4*)v + e);
+// FP64 vectors as pairs, once per row or evolution (T_0 of the chains).
+template <int NV>
+struct DfSplit {
+  const double2* in[NV];
+  float4* out[NV];
+};
+template <int NV>
+__global__ void __launch_bounds__(256) k_split_vec(DfSplit<NV> A, size_t n) {
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const double2 z = A.in[q][e];
+      const float2 a = df_split_int(z.x), b = df_split_int(z.y);
+      A.out[q][e] = make_float4(a.x, b.x, a.y, b.y);
+    }
 }
+
+// ---------------------------------------------------------------- moment rows
 
 // T_m = 2H~ T_{m-1} - T_{m-2} at element i of a pair chain (T_1 = H~ T_0 when
 // FIRST); own = T_{m-1}[i], nb[k] = T_{m-1}[idx[k][i]].
+template <bool FIRST>
+__device__ __forceinline__ DfC df_start(float2 dg, float4 own, float4 tm2) {
+  if (FIRST) {
+    DfC a;
+    df_prod(a.h, a.l, f2_both(dg.x), f2_both(dg.y), f2_hi(own), f2_lo(own));
+    return a;
+  }
+  return df_mul_sub(f2_both(dg.x), f2_both(dg.y), f2_hi(own), f2_lo(own), tm2);
+}
 template <bool CH, int KK, bool FIRST>
 __device__ __forceinline__ float4 df_step(const typename DfHop<CH>::T (&hv)[KK], float2 dg, float4 own,
                                           const float4 (&nb)[KK], float4 tm2) {
-  DfC a = FIRST ? dfc_zero() : dfc_neg(tm2);
-  dfc_mac(a, dg, own);
+  DfC a = df_start<FIRST>(dg, own, tm2);
 #pragma unroll
   for (int k = 0; k < KK; ++k) dfc_mac(a, hv[k], nb[k]);
   return dfc_out(a, FIRST);
-}
-
-// (sh, sl) += (bh, bl) for pairs, unnormalised (TwoSum of the high words, the
-// low words and the TwoSum error added into sl).
-__device__ __forceinline__ void df_add(float& sh, float& sl, float bh, float bl) {
-  const float s = __fadd_rn(sh, bh);
-  const float v = __fsub_rn(s, sh);
-  const float t = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, v)), __fsub_rn(bh, v));
-  sh = s;
-  sl = __fadd_rn(sl, __fadd_rn(bl, t));
 }
 
 // a += h0 * (sum_k nb[k]) for a real pair h0: the neighbour values are summed as
 // pairs first, so one product with h0 replaces KK.
 template <int KK>
 __device__ __forceinline__ void dfc_mac_sum(DfC& a, float2 h0, const float4 (&nb)[KK]) {
-  float rh = nb[0].x, rl = nb[0].y, ih = nb[0].z, il = nb[0].w;
+  DfC s = dfc_of(nb[0]);
 #pragma unroll
-  for (int k = 1; k < KK; ++k) {
-    df_add(rh, rl, nb[k].x, nb[k].y);
-    df_add(ih, il, nb[k].z, nb[k].w);
-  }
-  df_mac(a.rh, a.rl, h0.x, h0.y, rh, rl);
-  df_mac(a.ih, a.il, h0.x, h0.y, ih, il);
+  for (int k = 1; k < KK; ++k) df_add(s, nb[k]);
+  df_mac(a, f2_both(h0.x), f2_both(h0.y), s.h, s.l);
 }
 
 // T_m at one element when every hopping equals h0 (a real 2H~ value), as
 // df_step (T_1 = H~ T_0 when FIRST).
 template <int KK, bool FIRST = false>
 __device__ __forceinline__ float4 df_step_uh(float2 h0, float2 dg, float4 own, const float4 (&nb)[KK], float4 tm2) {
-  DfC a = FIRST ? dfc_zero() : dfc_neg(tm2);
-  dfc_mac(a, dg, own);
+  DfC a = df_start<FIRST>(dg, own, tm2);
   dfc_mac_sum<KK>(a, h0, nb);
   return dfc_out(a, FIRST);
 }
@@ -234,16 +323,15 @@ __device__ __forceinline__ float4 df_step_any(const DfEll<CH>& H, const typename
 // VAC rows by two recurrences (the pair form of k_cheb_pair_w): chain A from l,
 // chain B from r, A_k = T_k l, B_k = T_k r; step m writes A_m, B_m and adds
 // Re <A_{m-1}|B_{m-1}> (moment slot 2m-2) and Re <A_{m-1}|B_m> (slot 2m-1); the
-// first step reads l and r as FP64, adds |l|^2 and |r|^2 (slot_norm) and also
-// writes l and r as pairs into a0out, b0out (the T_{m-2} of step 2).  R = 1,
-// wavefront CTA order, one element per thread.
+// first step also adds |l|^2 and |r|^2 (slot_norm).  l and r are split before it
+// (k_split_vec).  R = 1, wavefront CTA order, one element per thread.
 template <bool CH, int KK, bool FIRST>
 __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4* __restrict__ tab,
-                                                         const void* __restrict__ am1, const void* __restrict__ bm1,
-                                                         const float4* am2, const float4* bm2, float4* aout,
-                                                         float4* bout, float4* __restrict__ a0out,
-                                                         float4* __restrict__ b0out, double2* __restrict__ partial,
-                                                         int nblocks, int m, int slot_norm) {
+                                                         const float4* __restrict__ am1,
+                                                         const float4* __restrict__ bm1, const float4* am2,
+                                                         const float4* bm2, float4* aout, float4* bout,
+                                                         double2* __restrict__ partial, int nblocks, int m,
+                                                         int slot_norm) {
   using HT = typename DfHop<CH>::T;
   double2* smem = dyn_smem();
   const int b = blockIdx.x;
@@ -262,7 +350,7 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
       hv[k] = __ldg(H.hop + s);
     }
     const float2 dg = __ldg(H.diag + i);
-    const float4 ao = df_load<FIRST>(am1, e), bo = df_load<FIRST>(bm1, e);
+    const float4 ao = __ldg(am1 + e), bo = __ldg(bm1 + e);
     float4 a2 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = a2;
     if (!FIRST) {
       a2 = am2[e];
@@ -271,8 +359,8 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
     float4 na[KK], nbv[KK];
 #pragma unroll
     for (int k = 0; k < KK; ++k) {
-      na[k] = df_load<FIRST>(am1, (size_t)idx[k]);
-      nbv[k] = df_load<FIRST>(bm1, (size_t)idx[k]);
+      na[k] = __ldg(am1 + idx[k]);
+      nbv[k] = __ldg(bm1 + idx[k]);
     }
     const float4 a = df_step<CH, KK, FIRST>(hv, dg, ao, na, a2);
     const float4 bb = df_step<CH, KK, FIRST>(hv, dg, bo, nbv, b2);
@@ -281,8 +369,6 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
     d0.add_re(ao, bo);
     d1.add_re(ao, bb);
     if (FIRST) {
-      a0out[e] = ao;
-      b0out[e] = bo;
       nl.add_norm(ao);
       nr.add_norm(bo);
     }
@@ -308,14 +394,13 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
 
 // l = r rows (DOS, MSD) by the doubling identities (the pair form of
 // k_cheb_dbl_w): step m writes u_m and adds <u_{m-1}|u_{m-1}> (slot 2m-2) and
-// Re <u_m|u_{m-1}> (slot 2m-1); the first step reads u_0 as FP64 and also writes
-// it as pairs into t0out (the T_{m-2} of step 2).  R = 1, wavefront CTA order,
-// U elements in flight per thread.
+// Re <u_m|u_{m-1}> (slot 2m-1).  R = 1, wavefront CTA order, U elements in flight
+// per thread.
 template <bool CH, int KK, int U, bool FIRST>
 __global__ void __launch_bounds__(256, 3) k_cheb_dbl_df(DfEll<CH> H, const int4* __restrict__ tab,
-                                                        const void* __restrict__ tm1, const float4* tm2,
-                                                        float4* tout, float4* __restrict__ t0out,
-                                                        double2* __restrict__ partial, int nblocks, int m) {
+                                                        const float4* __restrict__ tm1, const float4* tm2,
+                                                        float4* tout, double2* __restrict__ partial, int nblocks,
+                                                        int m) {
   using HT = typename DfHop<CH>::T;
   double2* smem = dyn_smem();
   const int b = blockIdx.x;
@@ -342,21 +427,20 @@ __global__ void __launch_bounds__(256, 3) k_cheb_dbl_df(DfEll<CH> H, const int4*
         hv[u][k] = __ldg(H.hop + s);
       }
       dg[u] = __ldg(H.diag + i);
-      own[u] = df_load<FIRST>(tm1, ee);
+      own[u] = __ldg(tm1 + ee);
       t2[u] = FIRST ? make_float4(0.f, 0.f, 0.f, 0.f) : tm2[ee];
     }
     float4 nb[U][KK];
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int k = 0; k < KK; ++k) nb[u][k] = df_load<FIRST>(tm1, (size_t)idx[u][k]);
+      for (int k = 0; k < KK; ++k) nb[u][k] = __ldg(tm1 + idx[u][k]);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const float4 a = df_step<CH, KK, FIRST>(hv[u], dg[u], own[u], nb[u], t2[u]);
       if (ok[u]) {
         const size_t e = e0 + u * step;
         tout[e] = a;
-        if (FIRST) t0out[e] = own[u];
         a0.add_norm(own[u]);
         a1.add_re(a, own[u]);
       }
@@ -368,243 +452,6 @@ __global__ void __launch_bounds__(256, 3) k_cheb_dbl_df(DfEll<CH> H, const int4*
     const int k0 = 2 * m - 2;
     partial[(size_t)k0 * nblocks + b] = make_double2(v[0], 0.0);
     partial[(size_t)(k0 + 1) * nblocks + b] = make_double2(v[1], 0.0);
-  }
-}
-
-// ---------------------------------------------------------------- evolution
-
-// U(dt) psi = sum_m c_m T_m(H~) psi (Eq. 17) for NSET vector sets sharing H~,
-// R = 1, on pairs of FP32 numbers: the chains T_m as pairs (16 bytes per complex
-// element, the size of the FP64 workspace), the sum of c_m T_m as pairs, the
-// caller's FP64 vectors split at the first order and formed again at the last
-// (hi + lo of two FP32 numbers is exact in FP64).  Orders by phase:
-//   PH 0 (m = 0, 1): out = T_1 = H~ psi, t0 = psi as pairs, acc = c0 psi + c1 T_1;
-//                    |psi|^2 partials (slot);
-//   PH 1 (2 <= m < Np - 1): out = 2H~ t1 - t2 (over t2, same element and thread),
-//                    acc += c0 out;
-//   PH 2 (m = Np - 1): psi = acc + c0 (2H~ t1 - t2) in FP64, |psi|^2 partials;
-//   PH 3 (Np <= 2): psi = acc in FP64, |psi|^2 partials.
-// c0, c1: complex coefficients as pairs (re.hi, re.lo, im.hi, im.lo).  The
-// partial slots are those of k_evolve (k_norm_check reads them).
-template <int NSET>
-struct DfEvo {
-  double2* psi[NSET];
-  const float4* t1[NSET];
-  const float4* t2[NSET];
-  float4* out[NSET];
-  float4* t0[NSET];
-  float4* acc[NSET];
-};
-
-__device__ __forceinline__ double2 df_to_d2(float4 f) { return make_double2(df_value(f.x, f.y), df_value(f.z, f.w)); }
-__device__ __forceinline__ DfC dfc_of(float4 a) { return DfC{a.x, a.y, a.z, a.w}; }
-
-template <bool CH, int KK, bool UH = false>
-__device__ __forceinline__ void df_row_ops(const DfEll<CH>& H, int i, int (&idx)[KK],
-                                           typename DfHop<CH>::T (&hv)[KK], float2& dg) {
-#pragma unroll
-  for (int k = 0; k < KK; ++k) {
-    const size_t s = (size_t)k * H.n + i;
-    idx[k] = __ldg(H.idx + s);
-    if (!UH) hv[k] = __ldg(H.hop + s);
-  }
-  dg = __ldg(H.diag + i);
-}
-
-template <bool CH, int KK, int NSET, int PH, bool UH = false>
-__global__ void __launch_bounds__(256) k_evolve_df(DfEll<CH> H, const int4* __restrict__ tab, DfEvo<NSET> A,
-                                                   float4 c0, float4 c1, double2* __restrict__ partial, int nblocks,
-                                                   int slot) {
-  using HT = typename DfHop<CH>::T;
-  const int4 tb = tab[blockIdx.x];
-  const size_t sege = (size_t)tb.y, step = (size_t)tb.w * blockDim.x;
-  DfDot nrm[NSET];
-  for (size_t e = (size_t)tb.x + (size_t)tb.z * blockDim.x + threadIdx.x; e < sege; e += step) {
-    const int i = (int)e;
-    if (PH == 3) {
-#pragma unroll
-      for (int q = 0; q < NSET; ++q) {
-        const float4 f = A.acc[q][e];
-        A.psi[q][e] = df_to_d2(f);
-        nrm[q].add_norm(f);
-      }
-      continue;
-    }
-    int idx[KK];
-    HT hv[KK];
-    float2 dg;
-    df_row_ops<CH, KK, UH>(H, i, idx, hv, dg);
-#pragma unroll
-    for (int q = 0; q < NSET; ++q) {
-      float4 nb[KK];
-      if (PH == 0) {
-        const float4 own = df_load<true>(A.psi[q], e);
-#pragma unroll
-        for (int k = 0; k < KK; ++k) nb[k] = df_load<true>(A.psi[q], (size_t)idx[k]);
-        const float4 y = df_step_any<CH, KK, true, UH>(H, hv, dg, own, nb, make_float4(0.f, 0.f, 0.f, 0.f));
-        A.out[q][e] = y;
-        A.t0[q][e] = own;
-        DfC a = dfc_zero();
-        dfc_mac(a, c0, own);
-        dfc_mac(a, c1, y);
-        A.acc[q][e] = dfc_out(a, false);
-        nrm[q].add_norm(own);
-      } else {
-        const float4 own = __ldg(A.t1[q] + e);
-#pragma unroll
-        for (int k = 0; k < KK; ++k) nb[k] = __ldg(A.t1[q] + idx[k]);
-        const float4 y = df_step_any<CH, KK, false, UH>(H, hv, dg, own, nb, A.t2[q][e]);
-        DfC a = dfc_of(A.acc[q][e]);
-        dfc_mac(a, c0, y);
-        const float4 f = dfc_out(a, false);
-        if (PH == 1) {
-          A.out[q][e] = y;
-          A.acc[q][e] = f;
-        } else {
-          A.psi[q][e] = df_to_d2(f);
-          nrm[q].add_norm(f);
-        }
-      }
-    }
-  }
-  if (PH != 1) {
-    double v[NSET];
-#pragma unroll
-    for (int q = 0; q < NSET; ++q) v[q] = nrm[q].get();
-    block_reduce_rx<NSET>(v, 1, reinterpret_cast<double*>(dyn_smem()));
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int q = 0; q < NSET; ++q) partial[(size_t)(slot + q) * nblocks + blockIdx.x] = make_double2(v[q], 0.0);
-    }
-  }
-}
-
-// One MSD time step's coupled orders (Eqs. 17, 18, 22, 24) on pairs, R = 1:
-//   u_m = T_m(H~) p,  z_m = [X, T_m] p + T_m px,
-//   z_m = 2[X,H~] u_{m-1} + 2H~ z_{m-1} - z_{m-2}  (z_1 = [X,H~] p + H~ px),
-//   accp += c_m u_m (-> U(dt) p), accx += c_m z_m (-> [X,U(dt)]p + U(dt)px).
-// Phases as k_evolve_df (PH 0 also writes p and px as pairs into u0, z0); the
-// partial slots are those of k_msd_evolve (k_norm_check_msd reads them).
-struct DfMsd {
-  double2* p;
-  double2* px;
-  const float4* u1;
-  const float4* u2;
-  const float4* z1;
-  const float4* z2;
-  float4* uo;
-  float4* zo;
-  float4* u0;
-  float4* z0;
-  float4* accp;
-  float4* accx;
-};
-
-template <bool CH, int KK, int PH, bool UH = false>
-__global__ void __launch_bounds__(256) k_msd_evolve_df(DfEll<CH> H, const int4* __restrict__ tab, DfMsd B, float4 c0,
-                                                       float4 c1, double2* __restrict__ partial, int nblocks,
-                                                       int slot) {
-  using HT = typename DfHop<CH>::T;
-  const int4 tb = tab[blockIdx.x];
-  const size_t sege = (size_t)tb.y, step = (size_t)tb.w * blockDim.x;
-  DfDot n0, n1;
-  for (size_t e = (size_t)tb.x + (size_t)tb.z * blockDim.x + threadIdx.x; e < sege; e += step) {
-    const int i = (int)e;
-    if (PH == 3) {
-      const float4 fp = B.accp[e], fx = B.accx[e];
-      B.p[e] = df_to_d2(fp);
-      B.px[e] = df_to_d2(fx);
-      n0.add_norm(fp);
-      n1.add_norm(fx);
-      continue;
-    }
-    int idx[KK];
-    HT hv[KK];
-    float2 dg;
-    df_row_ops<CH, KK, UH>(H, i, idx, hv, dg);
-    float4 uo, zo;  // u_m and z_m at this element
-    float4 u_own, z_own;
-    if (PH == 0) {
-      u_own = df_load<true>(B.p, e);
-      z_own = df_load<true>(B.px, e);
-      float4 un[KK];
-#pragma unroll
-      for (int k = 0; k < KK; ++k) un[k] = df_load<true>(B.p, (size_t)idx[k]);
-      uo = df_step_any<CH, KK, true, UH>(H, hv, dg, u_own, un, make_float4(0.f, 0.f, 0.f, 0.f));
-      DfC a = dfc_zero();
-      dfc_mac(a, dg, z_own);
-      float4 zn[KK];
-#pragma unroll
-      for (int k = 0; k < KK; ++k) zn[k] = df_load<true>(B.px, (size_t)idx[k]);
-      if constexpr (UH) {
-        dfc_mac_sum<KK>(a, H.h0, zn);
-      } else {
-#pragma unroll
-        for (int k = 0; k < KK; ++k) dfc_mac(a, hv[k], zn[k]);
-      }
-#pragma unroll
-      for (int k = 0; k < KK; ++k) dfc_mac(a, __ldg(H.xhop + (size_t)k * H.n + i), un[k]);
-      zo = dfc_out(a, true);
-    } else {
-      u_own = __ldg(B.u1 + e);
-      z_own = __ldg(B.z1 + e);
-      float4 un[KK];
-#pragma unroll
-      for (int k = 0; k < KK; ++k) un[k] = __ldg(B.u1 + idx[k]);
-      uo = df_step_any<CH, KK, false, UH>(H, hv, dg, u_own, un, B.u2[e]);
-      DfC a = dfc_neg(B.z2[e]);
-      dfc_mac(a, dg, z_own);
-      float4 zn[KK];
-#pragma unroll
-      for (int k = 0; k < KK; ++k) zn[k] = __ldg(B.z1 + idx[k]);
-      if constexpr (UH) {
-        dfc_mac_sum<KK>(a, H.h0, zn);
-      } else {
-#pragma unroll
-        for (int k = 0; k < KK; ++k) dfc_mac(a, hv[k], zn[k]);
-      }
-#pragma unroll
-      for (int k = 0; k < KK; ++k) dfc_mac(a, __ldg(H.xhop + (size_t)k * H.n + i), un[k]);
-      zo = dfc_out(a, false);
-    }
-    if (PH == 0) {
-      B.uo[e] = uo;
-      B.zo[e] = zo;
-      B.u0[e] = u_own;
-      B.z0[e] = z_own;
-      DfC ap = dfc_zero(), ax = dfc_zero();
-      dfc_mac(ap, c0, u_own);
-      dfc_mac(ap, c1, uo);
-      dfc_mac(ax, c0, z_own);
-      dfc_mac(ax, c1, zo);
-      B.accp[e] = dfc_out(ap, false);
-      B.accx[e] = dfc_out(ax, false);
-      n0.add_norm(u_own);
-    } else {
-      DfC ap = dfc_of(B.accp[e]), ax = dfc_of(B.accx[e]);
-      dfc_mac(ap, c0, uo);
-      dfc_mac(ax, c0, zo);
-      const float4 fp = dfc_out(ap, false), fx = dfc_out(ax, false);
-      if (PH == 1) {
-        B.uo[e] = uo;
-        B.zo[e] = zo;
-        B.accp[e] = fp;
-        B.accx[e] = fx;
-      } else {
-        B.p[e] = df_to_d2(fp);
-        B.px[e] = df_to_d2(fx);
-        n0.add_norm(fp);
-        n1.add_norm(fx);
-      }
-    }
-  }
-  if (PH != 1) {
-    double v[2] = {n0.get(), n1.get()};
-    block_reduce_rx<2>(v, 1, reinterpret_cast<double*>(dyn_smem()));
-    if (threadIdx.x == 0) {
-      partial[(size_t)slot * nblocks + blockIdx.x] = make_double2(v[0], 0.0);
-      partial[(size_t)(slot + 1) * nblocks + blockIdx.x] = make_double2(v[1], 0.0);
-    }
   }
 }
 

@@ -27,6 +27,7 @@
 #include "gqt_cluster.cuh"
 #include "gqt_df.cuh"
 #include "gqt_tile.cuh"
+#include "gqt_host.cuh"
 
 using namespace gqt;
 
@@ -156,6 +157,8 @@ struct Profiler {
 Profiler g_prof;
 }  // namespace
 
+bool gqt::prof_on() { return g_prof.on; }
+
 size_t gqt::prof_begin(cudaStream_t st) {
   if (!g_prof.on) return (size_t)-1;
   size_t i = g_prof.used;
@@ -168,121 +171,9 @@ void gqt::prof_end(size_t i, int cat, cudaStream_t st) {
   g_prof.pairs.push_back({cat, i});
 }
 
-// ====================================================================== graphs
-
-// Replays a loop of launches as a CUDA graph keyed by everything the launches
-// depend on (kind, sizes, pointers, coefficients).  Capture and replay run on
-// the handle's own non-blocking stream, ordered after and before the caller's
-// stream by events, so the caller may pass the legacy default stream.
-// 64-bit digest of a coefficient array (SplitMix64 finaliser folded over the
-// words, so sign patterns cannot cancel); the array itself is stored with the
-// graph and compared exactly on reuse.
-static uint64_t digest(const std::vector<double>& v) {
-  uint64_t x = 0x243F6A8885A308D3ull ^ (uint64_t)v.size();
-  for (double d : v) {
-    uint64_t u;
-    memcpy(&u, &d, 8);
-    x = splitmix_mix(x ^ u) + 0x9E3779B97F4A7C15ull;
-  }
-  return x;
-}
-
-template <class F>
-static void run_graph(gqt_ham* h, std::string key, cudaStream_t st, F&& launches,
-                      const std::vector<double>* data = nullptr) {
-  if (!h->use_graphs || g_prof.on) {
-    launches(st);
-    return;
-  }
-  if (data) {
-    char buf[40];
-    snprintf(buf, sizeof buf, "|d%016llx", (unsigned long long)digest(*data));
-    key += buf;
-    auto d = h->graph_data.find(key);
-    if (d != h->graph_data.end() && d->second != *data) {  // digest collision: no graph
-      launches(st);
-      return;
-    }
-  }
-  if (!h->gstream) {
-    check_cuda(cudaStreamCreateWithFlags(&h->gstream, cudaStreamNonBlocking), "cudaStreamCreate");
-    check_cuda(cudaEventCreateWithFlags(&h->gev[0], cudaEventDisableTiming), "cudaEventCreate");
-    check_cuda(cudaEventCreateWithFlags(&h->gev[1], cudaEventDisableTiming), "cudaEventCreate");
-  }
-  auto it = h->graphs.find(key);
-  if (it == h->graphs.end()) {
-    if (h->graphs.size() >= 512) {
-      for (auto& g : h->graphs) cudaGraphExecDestroy(g.second);
-      h->graphs.clear();
-      h->graph_data.clear();
-    }
-    cudaGraph_t graph = nullptr;
-    check_cuda(cudaStreamBeginCapture(h->gstream, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
-    try {
-      launches(h->gstream);
-    } catch (...) {
-      cudaStreamEndCapture(h->gstream, &graph);
-      if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
-      throw;
-    }
-    check_cuda(cudaStreamEndCapture(h->gstream, &graph), "cudaStreamEndCapture");
-    cudaGraphExec_t exec = nullptr;
-    cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    check_cuda(e, "cudaGraphInstantiate");
-    it = h->graphs.emplace(key, exec).first;
-    if (data) h->graph_data[key] = *data;
-  }
-  check_cuda(cudaEventRecord(h->gev[0], st), "cudaEventRecord");
-  check_cuda(cudaStreamWaitEvent(h->gstream, h->gev[0], 0), "cudaStreamWaitEvent");
-  check_cuda(cudaGraphLaunch(it->second, h->gstream), "cudaGraphLaunch");
-  g_launches.fetch_add(1, std::memory_order_relaxed);
-  check_cuda(cudaEventRecord(h->gev[1], h->gstream), "cudaEventRecord");
-  check_cuda(cudaStreamWaitEvent(st, h->gev[1], 0), "cudaStreamWaitEvent");
-}
-
-static std::string key_of(const char* op, std::initializer_list<const void*> ptrs, std::initializer_list<double> nums) {
-  std::string k(op);
-  char buf[64];
-  for (auto p : ptrs) {
-    snprintf(buf, sizeof buf, "|%p", p);
-    k += buf;
-  }
-  for (auto x : nums) {
-    snprintf(buf, sizeof buf, "|%.17g", x);
-    k += buf;
-  }
-  return k;
-}
-
-// The exact bits of every expansion coefficient, as part of a graph key (a
-// lossy hash can map U(+dt) and U(-dt), whose coefficients differ only in
-// signs, to the same key).
-static std::string coef_bits(const std::vector<double2>& c) {
-  std::string k("|c");
-  char buf[40];
-  for (const double2& q : c) {
-    uint64_t u[2];
-    memcpy(u, &q, 16);
-    snprintf(buf, sizeof buf, "%016llx%016llx", (unsigned long long)u[0], (unsigned long long)u[1]);
-    k += buf;
-  }
-  return k;
-}
-
 // ====================================================================== handle
 
 static bool is_pow2_r(int R) { return R == 1 || R == 2 || R == 4 || R == 8 || R == 16 || R == 32; }
-
-// dynamic shared memory of the CTA reductions (NV values per vector per warp)
-static size_t smem_bytes(const gqt_ham* h, int R, int nv) { return (size_t)nv * (h->threads / 32) * R * sizeof(double2); }
-
-static int rshift_of(int R) {
-  int s = 0;
-  while ((1 << s) < R) ++s;
-  return s;
-}
 
 // Next-iteration prefetch of the multi-vector kernels (FP32 storage, where the
 // dependent index load bounds the iteration): needs a lane group of at least K + 1
@@ -479,43 +370,6 @@ DevBuf& gqt_ham::ws(int slot, size_t bytes) {
 
 // ====================================================================== dispatch helpers
 
-template <bool FP64, bool CH>
-static Ell<FP64, CH> ell_of(const gqt_ham* h) {
-  Ell<FP64, CH> e;
-  e.n = (int)h->n;
-  e.K = h->K;
-  e.idx = (const int*)h->d_idx.p;
-  e.hop2 = (const typename Ell<FP64, CH>::HT*)h->d_hop.p;
-  e.diag2 = (const typename Ell<FP64, CH>::S*)h->d_diag.p;
-  e.dx = (const typename Ell<FP64, CH>::S*)h->d_dx.p;
-  e.row_shift = (h->use_sweep_order && h->row_shift > 0) ? h->row_shift : 0;
-  return e;
-}
-
-template <class F>
-static void dispatch(const gqt_ham* h, F&& f) {
-  if (h->prec == GQT_FP64) {
-    if (h->hop_real)
-      f(ell_of<true, false>(h));
-    else
-      f(ell_of<true, true>(h));
-  } else {
-    if (h->hop_real)
-      f(ell_of<false, false>(h));
-    else
-      f(ell_of<false, true>(h));
-  }
-}
-
-template <class E>
-struct EllTraits;
-template <bool FP64, bool CH>
-struct EllTraits<Ell<FP64, CH>> {
-  static constexpr bool fp64 = FP64;
-  static constexpr bool ch = CH;
-  using V = typename Prec<FP64>::V;
-};
-
 size_t gqt_ham::vec_bytes(int R) const { return (size_t)n * R * (prec == GQT_FP64 ? 16 : 8); }
 
 // ====================================================================== status
@@ -537,15 +391,6 @@ static gqt_status finish_call(gqt_ham* h, cudaStream_t st, const char* what) {
 
 static void reset_flag(gqt_ham* h, cudaStream_t st) {
   check_cuda(cudaMemsetAsync(h->d_flag.p, 0, sizeof(int), st), "flag reset");
-}
-
-// Segment sums of the partial slots slot0 .. slot0 + nslots - 1 (and slot extra, if
-// >= 0), in place, before k_reduce, k_reduce_dbl or a norm check reads them.
-static void launch_slot_sums(double2* partial, int nblocks, int R, const int* seg_blk, int nseg, int slot0, int nslots,
-                             int extra, cudaStream_t st) {
-  const long long items = (long long)(nslots + (extra >= 0 ? 1 : 0)) * nseg;
-  k_slot_sums<<<(unsigned)std::min<long long>(items, 1 << 20), 256, 0, st>>>(partial, nblocks, R, seg_blk, nseg, slot0, nslots, extra);
-  check_launch("k_slot_sums");
 }
 
 // ====================================================================== moments core
@@ -752,7 +597,7 @@ static bool df_applies(const gqt_ham* h, int R, int kind) {
 
 // 2H~ and 2U/dE as (hi, lo) pairs, split once from the FP64 arrays (again after
 // gqt_update_hamiltonian).  Runs on the call's stream before any graph capture.
-static void ensure_df(gqt_ham* h, cudaStream_t st) {
+void gqt::ensure_df(gqt_ham* h, cudaStream_t st) {
   if (h->df_ready) return;
   const size_t nslots = (size_t)h->K * h->n;
   h->d_hop_df.ensure(nslots * (h->hop_real ? sizeof(float2) : sizeof(float4)));
@@ -770,25 +615,9 @@ static void ensure_df(gqt_ham* h, cudaStream_t st) {
   h->df_ready = true;
 }
 
-template <bool CH>
-static DfEll<CH> df_ell_of(const gqt_ham* h) {
-  DfEll<CH> e;
-  e.n = (int)h->n;
-  e.K = h->K;
-  e.idx = (const int*)h->d_idx.p;
-  e.hop = (const typename DfHop<CH>::T*)h->d_hop_df.p;
-  e.diag = (const float2*)h->d_diag_df.p;
-  e.xhop = (const typename DfHop<CH>::T*)h->d_xhop_df.p;
-  if (h->hop_uniform) {
-    const float a = (float)h->hop0;
-    e.h0 = make_float2(a, (float)(h->hop0 - (double)a));
-  }
-  return e;
-}
-
 // 2[X,H~] slot values as pairs for the commutator orders (once per handle, again
 // after gqt_update_hamiltonian).  Runs on the call's stream before any capture.
-static void ensure_df_x(gqt_ham* h, cudaStream_t st) {
+void gqt::ensure_df_x(gqt_ham* h, cudaStream_t st) {
   if (h->dfx_ready) return;
   const size_t nslots = (size_t)h->K * h->n;
   h->d_xhop_df.ensure(nslots * (h->hop_real ? sizeof(float2) : sizeof(float4)));
@@ -884,12 +713,17 @@ static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const
   for (int m = 1; m <= std::max(steps, 1);) {
     size_t pe = prof_begin(s2);
     if (m == 1) {
-      if (pair)
-        k_cheb_pair_df<CH, KK, true><<<nb, h->threads, sm, s2>>>(H, tab, l, r, nullptr, nullptr, A[0], B[0], A[1],
-                                                                 B[1], partial, nb, 1, 2 * steps);
-      else
-        k_cheb_dbl_df<CH, KK, df_u(KK), true><<<nb, h->threads, sm, s2>>>(H, tab, r, nullptr, B[0], B[1], partial, nb,
-                                                                          1);
+      if (pair) {
+        void* in[2] = {const_cast<void*>(l), const_cast<void*>(r)};
+        float4* t0[2] = {A[1], B[1]};
+        launch_split<2>(in, t0, (size_t)h->n, s2);
+        k_cheb_pair_df<CH, KK, true><<<nb, h->threads, sm, s2>>>(H, tab, A[1], B[1], nullptr, nullptr, A[0], B[0],
+                                                                 partial, nb, 1, 2 * steps);
+      } else {
+        void* in[1] = {const_cast<void*>(r)};
+        launch_split<1>(in, &B[1], (size_t)h->n, s2);
+        k_cheb_dbl_df<CH, KK, df_u(KK), true><<<nb, h->threads, sm, s2>>>(H, tab, B[1], nullptr, B[0], partial, nb, 1);
+      }
       check_launch(pair ? "k_cheb_pair_df(first)" : "k_cheb_dbl_df(first)");
       prof_end(pe, 0, s2);
       m = 2;
@@ -937,10 +771,10 @@ static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const
     }
     if (pair)
       k_cheb_pair_df<CH, KK, false><<<nb, h->threads, sm, s2>>>(H, tab, A[cur], B[cur], A[prv], B[prv], A[prv],
-                                                                B[prv], nullptr, nullptr, partial, nb, m, 2 * steps);
+                                                                B[prv], partial, nb, m, 2 * steps);
     else
-      k_cheb_dbl_df<CH, KK, df_u(KK), false><<<nb, h->threads, sm, s2>>>(H, tab, B[cur], B[prv], B[prv], nullptr,
-                                                                         partial, nb, m);
+      k_cheb_dbl_df<CH, KK, df_u(KK), false><<<nb, h->threads, sm, s2>>>(H, tab, B[cur], B[prv], B[prv], partial, nb,
+                                                                         m);
     check_launch(pair ? "k_cheb_pair_df" : "k_cheb_dbl_df");
     prof_end(pe, pair ? 6 : 5, s2);
     std::swap(cur, prv);
@@ -1310,350 +1144,6 @@ void gqt::launch_moments(gqt_ham* h, const void* l, const void* r, int R, int M,
                                    (1.0 + tol) * (1.0 + tol), out, kind == 0 ? 0 : 1, (int*)h->d_flag.p);
       check_launch("k_reduce");
     }
-  });
-}
-
-// ====================================================================== evolution core
-
-// Evolution orders of FP64 handles with one vector on the FP32 pipes (pairs of
-// FP32 numbers, gqt_df.cuh), when their moment rows run there too (FP64
-// arithmetic mode 1): the wavefront table and neighbour counts of the pair rows.
-static bool df_evo_applies(const gqt_ham* h, int R) {
-  return h->prec == GQT_FP64 && h->fp64_arith == 1 && R == 1 && h->variant != 0 && h->threads <= 256 &&
-         (h->K == 2 || h->K == 3 || h->K == 4 || h->K == 6) && h->d_dx.p != nullptr;
-}
-
-// An expansion coefficient as pairs (re.hi, re.lo, im.hi, im.lo).
-static float4 coef_df(double2 c) {
-  const float a = (float)c.x, b = (float)c.y;
-  return make_float4(a, (float)(c.x - (double)a), b, (float)(c.y - (double)b));
-}
-
-template <class F>
-static void df_dispatch(const gqt_ham* h, F&& f) {
-  auto kk = [&](auto ch) {
-    switch (h->K) {
-      case 2: f(ch, std::integral_constant<int, 2>()); break;
-      case 3: f(ch, std::integral_constant<int, 3>()); break;
-      case 4: f(ch, std::integral_constant<int, 4>()); break;
-      default: f(ch, std::integral_constant<int, 6>()); break;
-    }
-  };
-  if (h->hop_real)
-    kk(std::integral_constant<bool, false>());
-  else
-    kk(std::integral_constant<bool, true>());
-}
-
-static int occupancy_of(const void* f, int threads, size_t smem) {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return 4;
-  }
-  return std::max(1, n);
-}
-
-template <int NSET>
-static void launch_evolve_df(gqt_ham* h, void* const* psi, const std::vector<double2>& c, cudaStream_t st,
-                             double* d_norms) {
-  ensure_df(h, st);
-  const int Np = (int)c.size();
-  const size_t smem = (size_t)NSET * (h->threads / 32) * sizeof(double) + 16;
-  int occ = h->blocks_per_sm;
-  if (occ <= 0)
-    df_dispatch(h, [&](auto ch, auto kk) {
-      occ = occupancy_of((const void*)k_evolve_df<decltype(ch)::value, decltype(kk)::value, NSET, 1>, h->threads,
-                         smem);
-    });
-  const BlockTable& T = h->table(1, occ);
-  const int nb = T.nblocks;
-  const size_t vb = h->vec_bytes(1);
-  float4* W1[NSET];
-  float4* W2[NSET];
-  float4* ACC[NSET];
-  for (int q = 0; q < NSET; ++q) {
-    W1[q] = (float4*)h->ws(WS_E1 + 2 * q, vb).p;
-    W2[q] = (float4*)h->ws(WS_E1 + 2 * q + 1, vb).p;
-    ACC[q] = (float4*)h->ws(WS_ACC0 + q, vb).p;
-  }
-  double2* partial = (double2*)h->ws(WS_PARTIAL_EVO, (size_t)(2 * NSET) * nb * sizeof(double2)).p;
-  const std::string key = key_of("evodf", {psi[0], psi[NSET - 1], W1[0], W2[0], ACC[0], partial, d_norms, T.d_blk.p},
-                                 {(double)NSET, (double)Np, (double)h->threads, (double)nb}) + coef_bits(c);
-  run_graph(h, key, st, [&](cudaStream_t s2) {
-    df_dispatch(h, [&](auto ch, auto kk) {
-      constexpr bool CH = decltype(ch)::value;
-      constexpr int KK = decltype(kk)::value;
-      const DfEll<CH> H = df_ell_of<CH>(h);
-      const int4* tab = (const int4*)T.d_tab4.p;
-      DfEvo<NSET> A;
-      for (int q = 0; q < NSET; ++q) {
-        A.psi[q] = (double2*)psi[q];
-        A.t1[q] = nullptr;
-        A.t2[q] = nullptr;
-        A.out[q] = W1[q];
-        A.t0[q] = W2[q];
-        A.acc[q] = ACC[q];
-      }
-      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-      auto orders = [&](auto uh) {
-        constexpr bool UH = decltype(uh)::value && !CH;  // one common hopping: no hop array read
-        k_evolve_df<CH, KK, NSET, 0, UH><<<nb, h->threads, smem, s2>>>(H, tab, A, coef_df(c[0]),
-                                                                       Np > 1 ? coef_df(c[1]) : zero, partial, nb, 0);
-        check_launch("k_evolve_df(0)");
-        if (Np <= 2) {
-          k_evolve_df<CH, KK, NSET, 3, UH><<<nb, h->threads, smem, s2>>>(H, tab, A, zero, zero, partial, nb, NSET);
-          check_launch("k_evolve_df(3)");
-          return;
-        }
-        for (int m = 2; m < Np; ++m) {
-          for (int q = 0; q < NSET; ++q) {
-            A.t1[q] = (m - 1) % 2 == 1 ? W1[q] : W2[q];
-            A.out[q] = (m % 2 == 1) ? W1[q] : W2[q];
-            A.t2[q] = A.out[q];
-          }
-          size_t pe = prof_begin(s2);
-          if (m == Np - 1)
-            k_evolve_df<CH, KK, NSET, 2, UH><<<nb, h->threads, smem, s2>>>(H, tab, A, coef_df(c[m]), zero, partial, nb,
-                                                                           NSET);
-          else
-            k_evolve_df<CH, KK, NSET, 1, UH><<<nb, h->threads, smem, s2>>>(H, tab, A, coef_df(c[m]), zero, partial, nb,
-                                                                           NSET);
-          check_launch("k_evolve_df");
-          prof_end(pe, 1 + NSET, s2);
-        }
-      };
-      if (h->hop_uniform)
-        orders(std::true_type());
-      else
-        orders(std::false_type());
-    });
-    launch_slot_sums(partial, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 0, 2 * NSET, -1, s2);
-    k_norm_check<<<1, 256, 0, s2>>>(partial, NSET, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 1e-10, d_norms,
-                                    (int*)h->d_flag.p);
-    check_launch("k_norm_check");
-  });
-}
-
-static void launch_msd_df(gqt_ham* h, void* p, void* px, const std::vector<double2>& c, cudaStream_t st) {
-  ensure_df(h, st);
-  ensure_df_x(h, st);
-  const int Np = (int)c.size();
-  const size_t smem = (size_t)2 * (h->threads / 32) * sizeof(double) + 16;
-  int occ = h->blocks_per_sm;
-  if (occ <= 0)
-    df_dispatch(h, [&](auto ch, auto kk) {
-      occ = occupancy_of((const void*)k_msd_evolve_df<decltype(ch)::value, decltype(kk)::value, 1>, h->threads,
-                         smem);
-    });
-  const BlockTable& T = h->table(1, occ);
-  const int nb = T.nblocks;
-  const size_t vb = h->vec_bytes(1);
-  float4* U1 = (float4*)h->ws(WS_E1, vb).p;
-  float4* U2 = (float4*)h->ws(WS_E1 + 1, vb).p;
-  float4* Z1 = (float4*)h->ws(WS_E1 + 2, vb).p;
-  float4* Z2 = (float4*)h->ws(WS_E1 + 3, vb).p;
-  float4* AP = (float4*)h->ws(WS_ACC0, vb).p;
-  float4* AX = (float4*)h->ws(WS_ACC0 + 1, vb).p;
-  double2* partial = (double2*)h->ws(WS_PARTIAL_EVO, (size_t)4 * nb * sizeof(double2)).p;
-  const std::string key = key_of("msddf", {p, px, U1, Z1, AP, AX, partial, T.d_blk.p},
-                                 {(double)Np, (double)h->threads, (double)nb}) + coef_bits(c);
-  run_graph(h, key, st, [&](cudaStream_t s2) {
-    df_dispatch(h, [&](auto ch, auto kk) {
-      constexpr bool CH = decltype(ch)::value;
-      constexpr int KK = decltype(kk)::value;
-      const DfEll<CH> H = df_ell_of<CH>(h);
-      const int4* tab = (const int4*)T.d_tab4.p;
-      DfMsd B;
-      B.p = (double2*)p;
-      B.px = (double2*)px;
-      B.u1 = B.u2 = B.z1 = B.z2 = nullptr;
-      B.uo = U1;
-      B.zo = Z1;
-      B.u0 = U2;
-      B.z0 = Z2;
-      B.accp = AP;
-      B.accx = AX;
-      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-      auto orders = [&](auto uh) {
-        constexpr bool UH = decltype(uh)::value && !CH;  // one common hopping: no hop array read
-        k_msd_evolve_df<CH, KK, 0, UH><<<nb, h->threads, smem, s2>>>(H, tab, B, coef_df(c[0]),
-                                                                     Np > 1 ? coef_df(c[1]) : zero, partial, nb, 0);
-        check_launch("k_msd_evolve_df(0)");
-        if (Np <= 2) {
-          k_msd_evolve_df<CH, KK, 3, UH><<<nb, h->threads, smem, s2>>>(H, tab, B, zero, zero, partial, nb, 2);
-          check_launch("k_msd_evolve_df(3)");
-          return;
-        }
-        for (int m = 2; m < Np; ++m) {
-          B.u1 = (m - 1) % 2 == 1 ? U1 : U2;
-          B.z1 = (m - 1) % 2 == 1 ? Z1 : Z2;
-          B.uo = (m % 2 == 1) ? U1 : U2;
-          B.zo = (m % 2 == 1) ? Z1 : Z2;
-          B.u2 = B.uo;
-          B.z2 = B.zo;
-          size_t pe = prof_begin(s2);
-          if (m == Np - 1)
-            k_msd_evolve_df<CH, KK, 2, UH><<<nb, h->threads, smem, s2>>>(H, tab, B, coef_df(c[m]), zero, partial, nb,
-                                                                         2);
-          else
-            k_msd_evolve_df<CH, KK, 1, UH><<<nb, h->threads, smem, s2>>>(H, tab, B, coef_df(c[m]), zero, partial, nb,
-                                                                         2);
-          check_launch("k_msd_evolve_df");
-          prof_end(pe, 4, s2);
-        }
-      };
-      if (h->hop_uniform)
-        orders(std::true_type());
-      else
-        orders(std::false_type());
-    });
-    launch_slot_sums(partial, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 0, 4, -1, s2);
-    k_norm_check_msd<<<1, 256, 0, s2>>>(partial, nb, 1, (const int*)T.d_seg_blk.p, h->nseg, 1e-10,
-                                        (int*)h->d_flag.p);
-    check_launch("k_norm_check_msd");
-  });
-}
-
-// In-place evolution of NSET vector sets (each [n][R]) by U(sign*dt) with Np
-// orders.  Norms before/after are checked on the device against tol.
-template <int NSET>
-static void launch_evolve_sets(gqt_ham* h, void* const* psi, int R, const std::vector<double2>& c, cudaStream_t st,
-                               double* d_norms /* [nseg][R][2*NSET] or null */) {
-  if (df_evo_applies(h, R)) {
-    launch_evolve_df<NSET>(h, psi, c, st, d_norms);
-    return;
-  }
-  const int Np = (int)c.size();
-  const BlockTable& T = h->table(R);
-  const int nb = T.nblocks, rs = rshift_of(R);
-  const size_t vb = h->vec_bytes(R);
-  void* W1[NSET];
-  void* W2[NSET];
-  double2* ACC[NSET];
-  for (int q = 0; q < NSET; ++q) {
-    W1[q] = h->ws(WS_E1 + 2 * q, vb).p;
-    W2[q] = h->ws(WS_E1 + 2 * q + 1, vb).p;
-    ACC[q] = (double2*)h->ws(WS_ACC0 + q, (size_t)h->n * R * sizeof(double2)).p;
-  }
-  double2* partial = (double2*)h->ws(WS_PARTIAL_EVO, (size_t)(2 * NSET) * nb * R * sizeof(double2)).p;
-  const std::string cbits = coef_bits(c);
-  const std::string key = key_of("evo", {psi[0], psi[NSET - 1], W1[0], W2[0], ACC[0], partial, d_norms, T.d_blk.p},
-                                 {(double)NSET, (double)R, (double)Np, (double)h->threads}) + cbits;
-  run_graph(h, key, st, [&](cudaStream_t s2) {
-    dispatch(h, [&](auto H) {
-      using Tr = EllTraits<decltype(H)>;
-      using V = typename Tr::V;
-      EvoSets<NSET, Tr::fp64> A;
-      // phase 0: m = 0, 1
-      for (int q = 0; q < NSET; ++q) {
-        A.t1[q] = (const V*)psi[q];
-        A.t2[q] = nullptr;
-        A.out[q] = (V*)W1[q];
-        A.acc[q] = ACC[q];
-        A.fin[q] = (V*)psi[q];
-      }
-      const double2 zero = make_double2(0.0, 0.0);
-      k_evolve<NSET, Tr::fp64, Tr::ch><<<nb, h->threads, smem_bytes(h, R, 3), s2>>>(H, (const int*)T.d_blk.p, R, rs, A, c[0],
-                                                                   Np > 1 ? c[1] : zero, 0, partial, nb, 0);
-      check_launch("k_evolve(0)");
-      if (Np <= 2) {
-        k_evolve<NSET, Tr::fp64, Tr::ch><<<nb, h->threads, smem_bytes(h, R, 3), s2>>>(H, (const int*)T.d_blk.p, R, rs, A, zero, zero, 3,
-                                                                     partial, nb, NSET);
-        check_launch("k_evolve(3)");
-      } else {
-        for (int m = 2; m < Np; ++m) {
-          for (int q = 0; q < NSET; ++q) {
-            V* w1 = (V*)W1[q];
-            V* w2 = (V*)W2[q];
-            A.t1[q] = (m - 1) % 2 == 1 ? w1 : w2;
-            V* o = (m % 2 == 1) ? w1 : w2;
-            A.t2[q] = (m == 2) ? (const V*)psi[q] : o;
-            A.out[q] = o;
-          }
-          const int phase = (m == Np - 1) ? 2 : 1;
-          size_t pe = prof_begin(s2);
-          k_evolve<NSET, Tr::fp64, Tr::ch><<<nb, h->threads, smem_bytes(h, R, 3), s2>>>(H, (const int*)T.d_blk.p, R, rs, A, c[m], zero,
-                                                                       phase, partial, nb, NSET);
-          check_launch("k_evolve");
-          prof_end(pe, 1 + NSET, s2);
-        }
-      }
-    });
-    const double tol = h->prec == GQT_FP64 ? 1e-10 : 1e-5;
-    launch_slot_sums(partial, nb, R, (const int*)T.d_seg_blk.p, h->nseg, 0, 2 * NSET, -1, s2);
-    k_norm_check<<<1, 256, 0, s2>>>(partial, NSET, nb, R, (const int*)T.d_seg_blk.p, h->nseg, tol, d_norms,
-                                    (int*)h->d_flag.p);
-    check_launch("k_norm_check");
-  });
-}
-
-static void launch_msd_step(gqt_ham* h, void* p, void* px, int R, const std::vector<double2>& c, cudaStream_t st) {
-  if (df_evo_applies(h, R)) {
-    launch_msd_df(h, p, px, c, st);
-    return;
-  }
-  const int Np = (int)c.size();
-  const BlockTable& T = h->table(R);
-  const int nb = T.nblocks, rs = rshift_of(R);
-  const size_t vb = h->vec_bytes(R);
-  void* U1 = h->ws(WS_E1, vb).p;
-  void* U2 = h->ws(WS_E1 + 1, vb).p;
-  void* Z1 = h->ws(WS_E1 + 2, vb).p;
-  void* Z2 = h->ws(WS_E1 + 3, vb).p;
-  double2* AP = (double2*)h->ws(WS_ACC0, (size_t)h->n * R * sizeof(double2)).p;
-  double2* AX = (double2*)h->ws(WS_ACC0 + 1, (size_t)h->n * R * sizeof(double2)).p;
-  double2* partial = (double2*)h->ws(WS_PARTIAL_EVO, (size_t)4 * nb * R * sizeof(double2)).p;
-  const std::string cbits = coef_bits(c);
-  const std::string key = key_of("msd", {p, px, U1, Z1, AP, AX, partial, T.d_blk.p},
-                                 {(double)R, (double)Np, (double)h->threads}) + cbits;
-  run_graph(h, key, st, [&](cudaStream_t s2) {
-    dispatch(h, [&](auto H) {
-      using Tr = EllTraits<decltype(H)>;
-      using V = typename Tr::V;
-      MsdBufs<Tr::fp64> B;
-      B.u1 = (const V*)p;
-      B.z1 = (const V*)px;
-      B.u2 = nullptr;
-      B.z2 = nullptr;
-      B.uo = (V*)U1;
-      B.zo = (V*)Z1;
-      B.accp = AP;
-      B.accx = AX;
-      B.p = (V*)p;
-      B.px = (V*)px;
-      const double2 zero = make_double2(0.0, 0.0);
-      k_msd_evolve<Tr::fp64, Tr::ch><<<nb, h->threads, smem_bytes(h, R, 3), s2>>>(H, (const int*)T.d_blk.p, R, rs, B, c[0],
-                                                                 Np > 1 ? c[1] : zero, 0, partial, nb, 0);
-      check_launch("k_msd_evolve(0)");
-      if (Np <= 2) {
-        k_msd_evolve<Tr::fp64, Tr::ch><<<nb, h->threads, smem_bytes(h, R, 3), s2>>>(H, (const int*)T.d_blk.p, R, rs, B, zero, zero, 3,
-                                                                   partial, nb, 2);
-        check_launch("k_msd_evolve(3)");
-      } else {
-        for (int m = 2; m < Np; ++m) {
-          B.u1 = (m - 1) % 2 == 1 ? (const V*)U1 : (const V*)U2;
-          B.z1 = (m - 1) % 2 == 1 ? (const V*)Z1 : (const V*)Z2;
-          V* uo = (m % 2 == 1) ? (V*)U1 : (V*)U2;
-          V* zo = (m % 2 == 1) ? (V*)Z1 : (V*)Z2;
-          B.u2 = (m == 2) ? (const V*)p : uo;
-          B.z2 = (m == 2) ? (const V*)px : zo;
-          B.uo = uo;
-          B.zo = zo;
-          const int phase = (m == Np - 1) ? 2 : 1;
-          size_t pe = prof_begin(s2);
-          k_msd_evolve<Tr::fp64, Tr::ch><<<nb, h->threads, smem_bytes(h, R, 3), s2>>>(H, (const int*)T.d_blk.p, R, rs, B, c[m], zero,
-                                                                     phase, partial, nb, 2);
-          check_launch("k_msd_evolve");
-          prof_end(pe, 4, s2);
-        }
-      }
-    });
-    // only |U p| vs |p| is a unitarity check; the px norm changes by construction.
-    const double tol = h->prec == GQT_FP64 ? 1e-10 : 1e-5;
-    launch_slot_sums(partial, nb, R, (const int*)T.d_seg_blk.p, h->nseg, 0, 4, -1, s2);
-    k_norm_check_msd<<<1, 256, 0, s2>>>(partial, nb, R, (const int*)T.d_seg_blk.p, h->nseg, tol, (int*)h->d_flag.p);
-    check_launch("k_norm_check_msd");
   });
 }
 
