@@ -239,13 +239,16 @@ gqt_status gqt_bond_gradients(const double* d_g_slot, long long n_slots, const l
  * lattice with bond_dy.  FP64 handles take d_r complex128; FP32 handles
  * (GQT_FP32_ACC64) take complex64, run the chains in FP32 and need the
  * tensor-core contraction (gqt_set_kb_contraction(ham, 1)), else GQT_EINVAL.  Workspace of the handle:
- * 2 M N R + 3 N R complex vectors (the stacks T_m v~_a r and v~_b T_n r) plus
- * the split partial sums.  Synchronises the stream before returning. */
+ * 2 M N R + 3 N R complex vectors (the stacks T_m v~_a r and v~_b T_n r), the
+ * split partial sums and, in mode 0, up to 1 GiB of digit slices of the stacks (less
+ * where less memory is free).  Synchronises the stream before returning. */
 gqt_status gqt_kb_moments(gqt_ham* ham, const void* d_r, int R, int M, int alpha, int beta, double* d_lambda,
                           void* stream);
 
 /* How gqt_kb_moments contracts the two stacks (default 0):
- * 0 = FP64 (complex FP64 GEMM on the FP64 pipe; Lambda to FP64 rounding);
+ * 0 = FP64 (Lambda to FP64 rounding): every stack row is scaled by a power of two and
+ *     cut into seven 8-bit digits, whose products the tcgen05 tensor cores sum exactly
+ *     (levels down to 2^-56 of the rows' largest elements);
  * 1 = split TF32 on the tcgen05 tensor cores: both stacks are rounded to pairs of
  *     TF32 numbers (hi + lo, about 22 bits), each product is hi*hi + hi*lo + lo*hi,
  *     accumulated in FP32 over splits of at most 8192 sites and summed in FP64
@@ -256,9 +259,9 @@ gqt_status gqt_kb_moments(gqt_ham* ham, const void* d_r, int R, int M, int alpha
 gqt_status gqt_set_kb_contraction(gqt_ham* ham, int mode);
 
 /* Polls of each bounded device wait of the handle's kernels (default 2^24, a
- * few tenths of a second to seconds; 0 = give up at once).  The only kernel
- * that waits is the tensor-core Hall contraction (gqt_set_kb_contraction mode
- * 1): its single issuing thread waits on mbarriers for the bulk tensor copies of
+ * few tenths of a second to seconds; 0 = give up at once).  The kernel that takes
+ * this setting is the split-TF32 Hall contraction (gqt_set_kb_contraction mode
+ * 1; the FP64 contraction's waits always have 2^24 polls and end the same way): its single issuing thread waits on mbarriers for the bulk tensor copies of
  * each stage and for the commit of the products that read a buffer.  A wait that
  * runs out stops the pipeline; the thread then drains what is in flight (the
  * last committed products and the issued copies, 2^24 polls each, independent of

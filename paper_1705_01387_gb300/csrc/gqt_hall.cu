@@ -13,11 +13,11 @@
 //
 // Three kernels carry the work.  k_kb_step advances both Chebyshev chains one
 // order and applies v~_b to T_k r from the same neighbour gathers, writing the
-// stacks P (M vectors) and B (M vectors).  k_kb_gemm forms all M x M inner
-// products <P_m|B_n> -- a dense complex contraction over N*R, the dominant cost
-// (4 M^2 N R FP64 FMAs) -- as a register-blocked FP64 GEMM with a deterministic
-// split over the contraction; k_kb_gemm_tma does the same contraction in split
-// TF32 on the tcgen05 tensor cores, its operands brought in by TMA.
+// stacks P (M vectors) and B (M vectors).  The M x M inner products <P_m|B_n> are a
+// dense complex contraction over N*R (4 M^2 N R FP64 FMAs), the dominant cost: the
+// default runs it to FP64 rounding on the tcgen05 tensor cores by exact integer slices
+// (gqt_slices.cu; k_kb_unscale sums its splits in order), k_kb_gemm_tma in split TF32,
+// its operands brought in by TMA.
 // k_kb_collapse turns the double sum over the moments into a series of 2M - 1 angles,
 // k_kb_series evaluates it on an energy grid, and k_kb_scan integrates it.
 
@@ -34,7 +34,9 @@
 #include <vector>
 
 #include "gqt_internal.h"
+#include "gqt_slices.h"
 
+using namespace gqt;
 using gqt::check_cuda;
 using gqt::check_launch;
 using gqt::prof_begin;
@@ -44,7 +46,7 @@ using gqt::set_error;
 
 namespace {
 
-enum { WS_HALL_P = 40, WS_HALL_B, WS_HALL_Q, WS_HALL_PART, WS_HALL_F, WS_HALL_W };
+enum { WS_HALL_P = 40, WS_HALL_B, WS_HALL_Q, WS_HALL_PART, WS_HALL_F, WS_HALL_W, WS_HALL_S };
 
 // H~ of a handle in the chain kernels: FP64 (double, double2 vectors) or FP32
 // storage (float, float2 vectors; the tensor-core contraction only).
@@ -248,65 +250,6 @@ __global__ void __launch_bounds__(256) k_kb_step(HallEll<F64, CH> H,
     pout[e] = pn;
     if (ps.re_hi) store_split(ps, e, pn);
   }
-}
-
-// part[s][m][n] = sum_{k in split s} conj(P[m][k]) B[n][k], P and B row-major
-// [M][Kt].  64 x 64 output tile per CTA, 4 x 4 complex outputs per thread
-// (rows tm + 16 i, columns tn + 16 j), contraction chunks of 16 staged in
-// shared memory (columns padded by one element against bank conflicts).
-constexpr int KB_TM = 64, KB_TK = 16;
-
-__global__ void __launch_bounds__(256, 2) k_kb_gemm(const double2* __restrict__ P, const double2* __restrict__ B, int M,
-                                                    size_t Kt, size_t kchunk, double2* __restrict__ part) {
-  __shared__ double2 Ps[KB_TK][KB_TM + 1];
-  __shared__ double2 Bs[KB_TK][KB_TM + 1];
-  const int m0 = blockIdx.x * KB_TM, n0 = blockIdx.y * KB_TM;
-  const size_t kb = (size_t)blockIdx.z * kchunk;
-  const size_t ke = (kb + kchunk < Kt) ? kb + kchunk : Kt;
-  const int tid = threadIdx.x, tm = tid & 15, tn = tid >> 4;
-  double2 acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[a][c] = make_double2(0.0, 0.0);
-  for (size_t k0 = kb; k0 < ke; k0 += KB_TK) {
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int q = tid + 256 * p;
-      const int row = q >> 4, kk = q & 15;
-      const size_t k = k0 + kk;
-      const bool kin = k < ke;
-      Ps[kk][row] = (kin && m0 + row < M) ? P[(size_t)(m0 + row) * Kt + k] : make_double2(0.0, 0.0);
-      Bs[kk][row] = (kin && n0 + row < M) ? B[(size_t)(n0 + row) * Kt + k] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < KB_TK; ++kk) {
-      double2 a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = Ps[kk][tm + 16 * u];
-        b[u] = Bs[kk][tn + 16 * u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          acc[u][v].x = fma(a[u].x, b[v].x, acc[u][v].x);
-          acc[u][v].x = fma(a[u].y, b[v].y, acc[u][v].x);
-          acc[u][v].y = fma(a[u].x, b[v].y, acc[u][v].y);
-          acc[u][v].y = fma(-a[u].y, b[v].x, acc[u][v].y);
-        }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int m = m0 + tm + 16 * u, nn = n0 + tn + 16 * v;
-      if (m < M && nn < M) part[((size_t)blockIdx.z * M + m) * M + nn] = acc[u][v];
-    }
 }
 
 // ------------------------------------------------------------ tensor-core contraction
@@ -537,6 +480,29 @@ __global__ void __launch_bounds__(TM_THREADS, 1) k_kb_gemm_tma(const __grid_cons
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// lam[m][n] = scale * 2^(e_m + e_n) * sum_s part[s][m][n] from the sliced products
+// (part: [S][re, im][M][M] of rows scaled to below 1, exponents ep and eb of the P and
+// B rows), splits summed in order.  A row that holds an infinity or a NaN (biased
+// exponent 2047) makes its entries NaN.
+__global__ void k_kb_unscale(const double* __restrict__ part, int S, int M, const int* __restrict__ ep,
+                             const int* __restrict__ eb, double scale, double2* __restrict__ lam) {
+  const size_t total = (size_t)M * M;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
+    double re = 0.0, im = 0.0;
+    for (int q = 0; q < S; ++q) {
+      re += part[(2 * (size_t)q) * total + t];
+      im += part[(2 * (size_t)q + 1) * total + t];
+    }
+    const int xm = ep[t / M], xn = eb[t % M];
+    if (xm == 2047 || xn == 2047) {
+      lam[t] = make_double2(CUDART_NAN, CUDART_NAN);
+    } else {
+      const int e = (xm - 1022) + (xn - 1022);
+      lam[t] = make_double2(scale * scalbn(re, e), scale * scalbn(im, e));
+    }
+  }
 }
 
 // lam[m][n] = scale * sum_s part[s][m][n], splits summed in order (deterministic).
@@ -781,22 +747,40 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
       check_launch("k_kb_step");
       prof_end(pe, 7, st);
     }
-    // split of the contraction: about eight waves of two resident CTAs per SM, at
-    // least 512 contraction elements per split
-    const int tiles = (M + KB_TM - 1) / KB_TM;
-    const long long slots = 2LL * gqt::sm_count();
-    long long S = std::max<long long>(1, (8 * slots + (long long)tiles * tiles - 1) / ((long long)tiles * tiles));
-    S = std::min<long long>(S, std::max<long long>(1, (long long)(total / 512)));
-    const size_t kchunk = ((total + S - 1) / S + KB_TK - 1) / KB_TK * KB_TK;
-    S = (long long)((total + kchunk - 1) / kchunk);
-    double2* part = (double2*)h->ws(WS_HALL_PART, (size_t)S * mm * sizeof(double2)).p;
+    // Lambda by exact slices of the stacks on the tensor cores: the contraction in
+    // blocks of sites whose slices take at most 1 GiB (and half of the free memory, so
+    // that stacks that fill the device still go through), later blocks added to the first
+    int* exps = (int*)h->ws(WS_HALL_F, (size_t)2 * M * sizeof(int)).p;
+    launch_row_exps((const double*)Pst, 2, M, total, total, nullptr, exps, st);
+    launch_row_exps((const double*)Bst, 2, M, total, total, nullptr, exps + M, st);
+    const int nk = (int)((total + SLICE_K - 1) / SLICE_K);
+    const size_t per_chunk = slice_bytes(M, 4, 1);
+    size_t cap = (size_t)1 << 30;
+    const size_t want = std::min(cap, per_chunk * nk), held = h->ws(WS_HALL_S, 0).bytes;
+    if (held < want) {
+      size_t free_b = 0, all_b = 0;
+      check_cuda(cudaMemGetInfo(&free_b, &all_b), "cudaMemGetInfo");
+      cap = std::min(cap, std::max(held, free_b / 2));
+    }
+    const int blk = (int)std::min<size_t>(nk, std::max<size_t>(64, cap / per_chunk));
+    char* sl = (char*)h->ws(WS_HALL_S, per_chunk * blk).p;
+    const int S = slice_splits(M, M, 2, blk);
+    double* part = (double*)h->ws(WS_HALL_PART, (size_t)S * 2 * mm * sizeof(double)).p;
+    check_cuda(cudaMemsetAsync(h->d_flag.p, 0, sizeof(int), st), "flag reset");
     const size_t pg = prof_begin(st);
-    k_kb_gemm<<<dim3(tiles, tiles, (unsigned)S), 256, 0, st>>>(Pst, Bst, M, total, kchunk, part);
-    check_launch("k_kb_gemm");
+    // Re Lambda = Pre.Bre + Pim.Bim, Im Lambda = Pre.Bim - Pim.Bre
+    const SliceParts parts = {2, 2, {{0, 1}, {0, 1}}, {{0, 1}, {1, 0}}, {{0, 0}, {0, 1}}};
+    for (int c0 = 0; c0 < nk; c0 += blk) {
+      const int nc = std::min(blk, nk - c0);
+      char* sb = sl + slice_bytes(M, 2, nc);
+      launch_slice_rows((const double*)Pst, 2, M, total, total, (size_t)c0 * SLICE_K, nullptr, nc, exps, sl, st);
+      launch_slice_rows((const double*)Bst, 2, M, total, total, (size_t)c0 * SLICE_K, nullptr, nc, exps + M, sb, st);
+      launch_slice_gemm({sl, M, 2}, {sb, M, 2}, parts, nc, S, part, c0 > 0, (int*)h->d_flag.p, st);
+    }
     prof_end(pg, 8, st);
-    k_kb_reduce<<<(int)std::min<size_t>((mm + 255) / 256, 4096), 256, 0, st>>>(part, (int)S, M,
+    k_kb_unscale<<<(int)std::min<size_t>((mm + 255) / 256, 4096), 256, 0, st>>>(part, S, M, exps, exps + M,
                                                                                 (double)h->n / R, lam);
-    check_launch("k_kb_reduce");
+    check_launch("k_kb_unscale");
     return;
   }
   // tensor-core contraction: chains in the handle's precision (rolling buffers),
@@ -926,8 +910,7 @@ extern "C" gqt_status gqt_kb_moments(gqt_ham* h, const void* d_r, int R, int M, 
         run(std::integral_constant<bool, true>());
     }
     int flag = 0;
-    if (h->kb_mode != 0)
-      check_cuda(cudaMemcpyAsync(&flag, h->d_flag.p, sizeof(int), cudaMemcpyDeviceToHost, st), "flag readback");
+    check_cuda(cudaMemcpyAsync(&flag, h->d_flag.p, sizeof(int), cudaMemcpyDeviceToHost, st), "flag readback");
     check_cuda(cudaStreamSynchronize(st), "gqt_kb_moments");
     if (flag & 32)
       throw Error(GQT_ETIMEOUT, "gqt_kb_moments: a bounded tensor-core wait gave up and so did the drain of the "

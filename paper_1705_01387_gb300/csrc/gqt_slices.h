@@ -1,0 +1,42 @@
+// gqt_slices.h -- FP64 matrix products by integer slices on the tensor cores
+// (gqt_slices.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstddef>
+
+namespace gqt {
+
+constexpr int SLICES = 7;     // base-256 digits of a value
+constexpr int SLICE_K = 16;   // contraction elements per chunk
+
+// A matrix of `rows` rows (K-major) in `planes` real planes, sliced:
+// [plane * SLICES + slice][chunk][row][16] FP16.
+struct SliceOperand {
+  const void* data;
+  int rows, planes;
+};
+
+// n results of the same shape; result p is the sum over its terms of A-plane a[p][t]
+// times the transpose of B-plane b[p][t], negated where neg[p][t].
+struct SliceParts {
+  int n, terms;
+  int a[2][2], b[2][2], neg[2][2];
+};
+
+size_t slice_bytes(int rows, int planes, int nchunk);
+// Largest biased exponents (times weights w [k], or null) of the rows of x [rows][k],
+// comp doubles per element (interleaved planes), rows `stride` elements apart.
+void launch_row_exps(const double* x, int comp, int rows, size_t stride, size_t k, const double* w, int* exps,
+                     cudaStream_t st);
+// Slices of elements [k0, k0 + 16 nchunk) of each row (zeros past k).
+void launch_slice_rows(const double* x, int comp, int rows, size_t stride, size_t k, size_t k0, const double* w,
+                       int nchunk, const int* exps, void* out, cudaStream_t st);
+int slice_splits(int rows_a, int rows_b, int parts, int nchunk);
+// out[split][part][rows_a][rows_b] (+)= the products of the scaled rows: times
+// 2^(exp_a - 1022 + exp_b - 1022) for the true values.  *err: bits 16, 32 (see above).
+void launch_slice_gemm(const SliceOperand& a, const SliceOperand& b, const SliceParts& parts, int nchunk, int splits,
+                       double* out, bool add, int* err, cudaStream_t st);
+
+}  // namespace gqt
