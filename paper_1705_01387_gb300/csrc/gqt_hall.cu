@@ -719,8 +719,12 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
   const size_t total = (size_t)h->n * R;
   const size_t vb = total * sizeof(V);
   const int g = grid_for(total);
-  // FP32 chain steps: one element per thread (every neighbour gather in flight at once)
-  const int gs = F64 ? g : (int)std::min<size_t>((total + 255) / 256, (size_t)INT32_MAX);
+  // Chain steps: one element per thread (every neighbour gather in flight at once), in
+  // CTAs small enough that every SM gets four: at N R = 18,432 a grid of 72 CTAs of 256
+  // left half of the SMs without work (FP64 step 10.3 us, 7.65 in CTAs of 64).
+  int ct = 256;
+  while (ct > 64 && total < (size_t)4 * gqt::sm_count() * ct) ct /= 2;
+  const int gs = (int)std::min<size_t>((total + ct - 1) / ct, (size_t)INT32_MAX);
   V* Q = (V*)h->ws(WS_HALL_Q, vb * 3).p;
   auto qbuf = [&](int k) -> V* { return Q + (size_t)(k % 3) * total; };
   const size_t mm = (size_t)M * M;
@@ -739,7 +743,7 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
       const V* qk = k == 0 ? r : qbuf(k);
       const V* qkm1 = k == 0 ? nullptr : (k == 1 ? r : qbuf(k - 1));
       const size_t pe = prof_begin(st);
-      k_kb_step<F64, CH><<<g, 256, 0, st>>>(H, vh, R, total, Pst + (size_t)k * total,
+      k_kb_step<F64, CH><<<gs, ct, 0, st>>>(H, vh, R, total, Pst + (size_t)k * total,
                                         k == 0 ? nullptr : Pst + (size_t)(k - 1) * total,
                                         last ? nullptr : Pst + (size_t)(k + 1) * total, qk, qkm1,
                                         last ? nullptr : qbuf(k + 1), Bst + (size_t)k * total, k == 0, last, none,
@@ -817,7 +821,7 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
     const V* qk = k == 0 ? r : qbuf(k);
     const V* qkm1 = k == 0 ? nullptr : (k == 1 ? r : qbuf(k - 1));
     const size_t pe = prof_begin(st);
-    k_kb_step<F64, CH><<<gs, 256, 0, st>>>(H, vh, R, total, pbuf(k), k == 0 ? nullptr : pbuf(k - 1),
+    k_kb_step<F64, CH><<<gs, ct, 0, st>>>(H, vh, R, total, pbuf(k), k == 0 ? nullptr : pbuf(k - 1),
                                       last ? nullptr : pbuf(k + 1), qk, qkm1, last ? nullptr : qbuf(k + 1), nullptr,
                                       k == 0, last, last ? none : planes(0, k + 1), planes(4, k));
     check_launch("k_kb_step");
