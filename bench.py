@@ -597,7 +597,7 @@ def run_ours(args):
            6: (f"k_cheb_pair{sfx} (VAC row: two fused SpMV + recurrences, T_k l and T_k r, + Re <A_k|B_k>, "
                "Re <A_k|B_k+1>)", bytes_per_orbital_pair(3, ham.hop_real, R), "pair", 1),
            10: ("k_cheb2_honey_df_pair (VAC row, temporally blocked: two steps of both recurrences per launch, "
-                "the second from the first's rows in L2" + (", one common hopping" if uniform else "") + ")",
+                "the second from the first's rows in shared memory" + (", one common hopping" if uniform else "") + ")",
                 bytes_per_orbital_tiled(3, ham.hop_real, True, uniform), "pair", 2),
            11: ("k_cheb2_honey_df_dbl (MSD row, temporally blocked: two steps per launch"
                 + (", one common hopping" if uniform else "") + ")",

@@ -261,7 +261,8 @@ gqt_status gqt_set_kb_contraction(gqt_ham* ham, int mode);
 /* Polls of each bounded device wait of the handle's kernels (default 2^24, a
  * few tenths of a second to seconds; 0 = give up at once).  The kernel that takes
  * this setting is the split-TF32 Hall contraction (gqt_set_kb_contraction mode
- * 1; the FP64 contraction's waits always have 2^24 polls and end the same way): its single issuing thread waits on mbarriers for the bulk tensor copies of
+ * 1; the FP64 contraction's and the blocked FP64 moment rows' waits for their copies
+ * always have 2^24 polls and end the same way): its single issuing thread waits on mbarriers for the bulk tensor copies of
  * each stage and for the commit of the products that read a buffer.  A wait that
  * runs out stops the pipeline; the thread then drains what is in flight (the
  * last committed products and the issued copies, 2^24 polls each, independent of
@@ -401,7 +402,8 @@ gqt_status gqt_set_fp64_arith(gqt_ham* ham, int mode);
  * largest dividing L1), run by the default multi-vector kernels.  Each CTA
  * walks a band of cells (128, 64 or 32 for the FP64 handles) down the rows: per
  * row it computes T_{m+1} from T_m and T_{m-1}, and T_{m+2} two rows behind from
- * the T_{m+1} rows it wrote just before (still in L2), so per two orders each
+ * the T_{m+1} rows it made just before (kept in shared memory for the FP64 handles,
+ * still in L2 for the others), so per two orders each
  * orbital's vectors and hoppings come from DRAM once and the index array is not
  * read (FP64 VAC rows 160 bytes per orbital instead of 280, l = r rows 96
  * instead of 184; FP32 VAC rows 64 + 16/R instead of 96 + 56/R).  Each CTA

@@ -26,6 +26,7 @@
 #include "gqt_kernels.cuh"
 #include "gqt_cluster.cuh"
 #include "gqt_df.cuh"
+#include "gqt_ring.cuh"
 #include "gqt_tile.cuh"
 #include "gqt_host.cuh"
 
@@ -658,7 +659,7 @@ static int df_occupancy(int K, bool pair, int threads) {
   }
 }
 
-// Temporal blocking of the paired-FP32 rows (two orders per pass, gqt_tile.cuh):
+// Temporal blocking of the paired-FP32 rows (two orders per pass, gqt_ring.cuh):
 // honeycomb handles whose rows follow the built-in cell layout, one segment,
 // L1 a multiple of 32 cells (the band width).
 static bool tiled_applies(const gqt_ham* h) {
@@ -681,19 +682,66 @@ static Honey honey_of(const gqt_ham* h) {
 }
 
 
-// CTAs of the blocked kernel: as many as are resident at once (each takes an
-// equal share of the band rows), at most the single-order grid nb (the stride of
-// the moment partial slots).
-constexpr size_t TL_SMEM = 4 * 8 * sizeof(double);  // block_reduce_rx<4> over at most 8 warps
+// The ring kernel of a handle's blocked rows: f(kernel) for the handle's hoppings (UH: one
+// real value on every slot), NC chains and the band width.
+template <int NC, class F>
+static void with_ring(const gqt_ham* h, F&& f) {
+  auto width = [&](auto ch, auto uh) {
+    constexpr bool CH = decltype(ch)::value, UH = decltype(uh)::value;
+    switch (tl_band_width(h->honey_L1)) {
+      case 128: f(k_cheb2_honey_df<CH, NC, UH, 128>); break;
+      case 64: f(k_cheb2_honey_df<CH, NC, UH, 64>); break;
+      default: f(k_cheb2_honey_df<CH, NC, UH, 32>); break;
+    }
+  };
+  if (!h->hop_real)
+    width(std::true_type(), std::false_type());
+  else if (h->hop_uniform)
+    width(std::false_type(), std::true_type());
+  else
+    width(std::false_type(), std::false_type());
+}
 
-template <bool CH, int NC>
-static int tiled_grid(int threads) {
+// Grid of the blocked rows: one CTA per band and segment of rows, as many segments as
+// the resident CTAs allow; with more bands than resident CTAs, equal ranges of band
+// rows.
+struct RingGrid {
+  int grid = 0, nseg = 0, rows = 0;
+  size_t smem = 0;
+};
+template <int NC>
+static RingGrid ring_grid(const gqt_ham* h) {
+  RingGrid g;
+  const int bw = tl_band_width(h->honey_L1), nbands = h->honey_L1 / bw;
+  const size_t most = ring_smem(bw, NC, std::min(RG_ROWS, h->honey_L2));
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_cheb2_honey_df<CH, NC>, threads, TL_SMEM) != cudaSuccess) {
-    cudaGetLastError();
-    n = 1;
+  with_ring<NC>(h, [&](auto kern) {
+    check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most), "smem attribute");
+    check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, 2 * bw, most), "occupancy");
+  });
+  const int res = std::max(1, n) * sm_count();
+  if (nbands <= res) {
+    g.nseg = std::min(res / nbands, h->honey_L2);
+    g.grid = nbands * g.nseg;
+    g.rows = std::min(RG_ROWS, (h->honey_L2 + g.nseg - 1) / g.nseg);
+  } else {
+    g.grid = res;
+    g.rows = std::min(RG_ROWS, h->honey_L2);
   }
-  return std::max(1, n) * sm_count();
+  g.smem = ring_smem(bw, NC, g.rows);
+  return g;
+}
+
+// One blocked pass; the kernels of the other hopping type are compiled but not launched.
+template <bool CK, bool CH>
+static void ring_launch(void (*kern)(DfEll<CK>, Honey, RingHop, int, int, const float4*, const float4*, const float4*,
+                                     const float4*, float4*, float4*, float4*, float4*, double2*, int, int, int*),
+                        const DfEll<CH>& H, const Honey& G, const RingHop& hs, const RingGrid& rg, int threads,
+                        const float4* xa, const float4* ya, const float4* xb, const float4* yb, float4* za, float4* wa,
+                        float4* zb, float4* wb, double2* pout, int ostride, int nzero, int* err, cudaStream_t st) {
+  if constexpr (CK == CH)
+    kern<<<rg.grid, threads, rg.smem, st>>>(H, G, hs, rg.nseg, rg.rows, xa, ya, xb, yb, za, wa, zb, wb, pout, ostride,
+                                            nzero, err);
 }
 
 // The rows' chains live in rotating buffers (4 per chain when tiled, else 2):
@@ -702,8 +750,9 @@ static int tiled_grid(int threads) {
 // reads T_j and T_{j-1} and writes T_{j+1} and T_{j+2} into the two other buffers.
 template <bool CH, int KK>
 static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const void* l, const void* r,
-                    float4* const* A, float4* const* B, int tgrid, int tnseg, double2* partial,
+                    float4* const* A, float4* const* B, const RingGrid& rg, double2* partial,
                     double2* tscratch, cudaStream_t s2) {
+  const int tgrid = rg.grid;
   const bool tiled = tgrid > 0;
   const DfEll<CH> H = df_ell_of<CH>(h);
   const int4* tab = (const int4*)T.d_tab4.p;
@@ -741,22 +790,19 @@ static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const
         const bool fold = tgrid > nb;
         double2* pout = fold ? tscratch : partial + (size_t)(2 * m - 2) * nb;
         const int ostride = fold ? tgrid : nb, nzero = fold ? 0 : nb;
-        // handles whose slots all hold one real hopping read no hop array (UH)
-        auto blocked = [&](auto uh) {
-          constexpr bool UH = decltype(uh)::value && !CH;
-          if (pair)
-            k_cheb2_honey_df<CH, 2, UH><<<tgrid, 2 * bw, TL_SMEM, s2>>>(H, G, bw, tnseg, A[cur], A[prv], B[cur],
-                                                                       B[prv], A[f[0]], A[f[1]], B[f[0]], B[f[1]],
-                                                                       pout, ostride, nzero);
-          else
-            k_cheb2_honey_df<CH, 1, UH><<<tgrid, 2 * bw, TL_SMEM, s2>>>(H, G, bw, tnseg, B[cur], B[prv], nullptr,
-                                                                       nullptr, B[f[0]], B[f[1]], nullptr, nullptr,
-                                                                       pout, ostride, nzero);
-        };
-        if (h->hop_uniform)
-          blocked(std::true_type());
+        RingHop hs;  // hop slot of each neighbour type
+        for (int q = 0; q < 2; ++q)
+          for (int k = 0; k < 3; ++k) hs.slot[q][h->honey_type[q][k]] = k;
+        if (pair)
+          with_ring<2>(h, [&](auto kern) {
+            ring_launch(kern, H, G, hs, rg, 2 * bw, A[cur], A[prv], B[cur], B[prv], A[f[0]], A[f[1]], B[f[0]], B[f[1]],
+                        pout, ostride, nzero, (int*)h->d_flag.p, s2);
+          });
         else
-          blocked(std::false_type());
+          with_ring<1>(h, [&](auto kern) {
+            ring_launch(kern, H, G, hs, rg, 2 * bw, B[cur], B[prv], nullptr, nullptr, B[f[0]], B[f[1]], nullptr,
+                        nullptr, pout, ostride, nzero, (int*)h->d_flag.p, s2);
+          });
         check_launch("k_cheb2_honey_df");
         if (fold) {
           k_tl_fold<<<4, 128, 0, s2>>>(tscratch, tgrid, 1, partial, nb, 2 * m - 2);
@@ -815,34 +861,25 @@ static void launch_moments_df(gqt_ham* h, const void* l, const void* r, int M, v
   const double tol = 1e-6;
   const size_t total = (size_t)h->nseg * M;
   const int rb = (int)std::min<size_t>((total + 255) / 256, 4096);
-  // grid of the tiled passes: their resident CTAs (set before any capture)
-  int tgrid = 0, tnseg = 0;
+  // grid of the tiled passes (set before any capture)
+  RingGrid rg;
   double2* tscratch = nullptr;
   if (tiled) {
-    // one CTA per band and segment, the segments as many as the resident CTAs allow
-    // (the CTAs of a segment then walk its rows across all bands together)
-    const int bw = tl_band_width(h->honey_L1), thr = 2 * bw, nbands = h->honey_L1 / bw;
-    const int res = pair ? (h->hop_real ? tiled_grid<false, 2>(thr) : tiled_grid<true, 2>(thr))
-                         : (h->hop_real ? tiled_grid<false, 1>(thr) : tiled_grid<true, 1>(thr));
-    if (nbands <= res) {
-      tnseg = res / nbands;
-      tgrid = nbands * tnseg;
-    } else {
-      tgrid = res;  // more bands than resident CTAs: equal ranges of band rows
-    }
-    if (tgrid > nb) tscratch = (double2*)h->ws(WS_TILE_SCRATCH, (size_t)4 * tgrid * sizeof(double2)).p;
+    rg = pair ? ring_grid<2>(h) : ring_grid<1>(h);
+    if (rg.grid > nb) tscratch = (double2*)h->ws(WS_TILE_SCRATCH, (size_t)4 * rg.grid * sizeof(double2)).p;
   }
   const std::string key = key_of("momdf", {l, r, out, A[0], A[1], A[2], A[3], B[0], B[1], B[2], B[3], partial,
                                            T.d_blk.p, tscratch},
-                                 {(double)kind, (double)M, (double)h->threads, (double)nb, (double)tgrid, (double)tnseg});
+                                 {(double)kind, (double)M, (double)h->threads, (double)nb, (double)rg.grid, (double)rg.nseg});
   run_graph(h, key, st, [&](cudaStream_t s2) {
+    const RingGrid none;
     auto rows = [&](auto ch) {
       constexpr bool CH = decltype(ch)::value;
       switch (h->K) {
-        case 2: df_rows<CH, 2>(h, T, pair, steps, l, r, A, B, 0, 0, partial, nullptr, s2); break;
-        case 3: df_rows<CH, 3>(h, T, pair, steps, l, r, A, B, tgrid, tnseg, partial, tscratch, s2); break;
-        case 4: df_rows<CH, 4>(h, T, pair, steps, l, r, A, B, 0, 0, partial, nullptr, s2); break;
-        default: df_rows<CH, 6>(h, T, pair, steps, l, r, A, B, 0, 0, partial, nullptr, s2); break;
+        case 2: df_rows<CH, 2>(h, T, pair, steps, l, r, A, B, none, partial, nullptr, s2); break;
+        case 3: df_rows<CH, 3>(h, T, pair, steps, l, r, A, B, rg, partial, tscratch, s2); break;
+        case 4: df_rows<CH, 4>(h, T, pair, steps, l, r, A, B, none, partial, nullptr, s2); break;
+        default: df_rows<CH, 6>(h, T, pair, steps, l, r, A, B, none, partial, nullptr, s2); break;
       }
     };
     if (h->hop_real)
