@@ -23,6 +23,7 @@
 
 #include "../../include/gqt.h"
 #include "gqt_internal.h"
+#include "gqt_slices.h"
 #include "gqt_kernels.cuh"
 #include "gqt_cluster.cuh"
 #include "gqt_df.cuh"
@@ -1289,6 +1290,18 @@ static int resolve_np(gqt_ham* h, double dt, int Np) {
 
 // ====================================================================== C ABI
 
+// Stream-ordered scratch of one call, given back on every way out.
+struct StreamScratch {
+  char* p = nullptr;
+  cudaStream_t st;
+  StreamScratch(size_t bytes, cudaStream_t s) : st(s) {
+    check_cuda(cudaMallocAsync((void**)&p, bytes, st), "cudaMallocAsync");
+  }
+  ~StreamScratch() { cudaFreeAsync(p, st); }
+  StreamScratch(const StreamScratch&) = delete;
+  StreamScratch& operator=(const StreamScratch&) = delete;
+};
+
 extern "C" {
 
 const char* gqt_last_error(void) { return g_last_error.c_str(); }
@@ -1635,16 +1648,56 @@ gqt_status gqt_kpm_reconstruct(const double* d_mu, int rows, int M, const double
           "gqt_kpm_reconstruct: bad argument");
   if (rows == 0 || NE == 0) return GQT_OK;
   cudaStream_t st = (cudaStream_t)stream;
-  double* tab = nullptr;
-  check_cuda(cudaMallocAsync((void**)&tab, (size_t)M * NE * sizeof(double), st), "cudaMallocAsync");
-  const size_t total = (size_t)M * NE;
-  k_kpm_table<<<(int)std::min<size_t>((total + 255) / 256, 8192), 256, 0, st>>>(M, d_E, NE, energy_scale, n_over_omega,
-                                                                                 kernel == 0, tab);
-  check_launch("k_kpm_table");
-  dim3 grid((NE + 15) / 16, (rows + 15) / 16);
-  k_kpm_gemm<<<grid, 256, 0, st>>>(d_mu, rows, M, tab, NE, d_out);
-  check_launch("k_kpm_gemm");
-  check_cuda(cudaFreeAsync(tab, st), "cudaFreeAsync");
+  // Up to 8 rows: one pass per energy (8 rows at M = 500, NE = 1001: 64 us, 9 by the
+  // product 131; at M = 3000, NE = 4001 399 and 422).  More: the Chebyshev table and
+  // the product with it on the tensor cores, over blocks of rows and of energies whose
+  // slices take at most 256 MB each.
+  const bool sliced = rows > 8;
+  const int nk = (M + SLICE_K - 1) / SLICE_K;
+  const size_t fit = ((size_t)1 << 28) / slice_bytes(1, 1, nk);
+  const int rb = sliced ? (int)std::min<size_t>(rows, std::max<size_t>(128, fit / 128 * 128)) : 0;
+  const int eb = sliced ? (int)std::min<size_t>(NE, std::max<size_t>(64, std::min(fit, ((size_t)1 << 25) / rb))) : 0;
+  const int S = sliced ? slice_splits(rb, eb, 1, nk) : 0;
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t o_exp = up((size_t)M * 8), o_err = o_exp + up((size_t)rows * 4), o_a = o_err + 256,
+               o_b = o_a + up(sliced ? slice_bytes(rb, 1, nk) : 0), o_p = o_b + up(sliced ? slice_bytes(eb, 1, nk) : 0),
+               need = o_p + (size_t)S * rb * eb * 8;
+  StreamScratch buf(need, st);
+  double* w = (double*)buf.p;
+  k_kpm_moment_weights<<<(M + 127) / 128, 128, 0, st>>>(M, kernel == 0, w);
+  check_launch("k_kpm_moment_weights");
+  if (!sliced) {
+    const int grid = (NE + 3) / 4;
+    if (rows <= 2)
+      k_kpm_rows<2><<<grid, 128, 0, st>>>(d_mu, rows, M, w, d_E, NE, energy_scale, n_over_omega, d_out);
+    else
+      k_kpm_rows<8><<<grid, 128, 0, st>>>(d_mu, rows, M, w, d_E, NE, energy_scale, n_over_omega, d_out);
+    check_launch("k_kpm_rows");
+  } else {
+    int* exps = (int*)(buf.p + o_exp);
+    int* err = (int*)(buf.p + o_err);
+    check_cuda(cudaMemsetAsync(err, 0, sizeof(int), st), "status reset");
+    launch_row_exps(d_mu, 1, rows, M, M, w, exps, st);
+    const SliceParts one = {1, 1, {{0, 0}, {0, 0}}, {{0, 0}, {0, 0}}, {{0, 0}, {0, 0}}};
+    double* part = (double*)(buf.p + o_p);
+    for (int r0 = 0; r0 < rows; r0 += rb) {
+      const int nr = std::min(rb, rows - r0);
+      launch_slice_rows(d_mu + (size_t)r0 * M, 1, nr, M, M, 0, w, nk, exps + r0, buf.p + o_a, st);
+      for (int e0 = 0; e0 < NE; e0 += eb) {
+        const int ne = std::min(eb, NE - e0);
+        if (r0 == 0 || eb < NE) launch_cos_slices(d_E + e0, ne, energy_scale, M, nk, buf.p + o_b, st);
+        launch_slice_gemm({buf.p + o_a, nr, 1}, {buf.p + o_b, ne, 1}, one, nk, S, part, false, err, st);
+        k_kpm_unscale<<<(int)std::min<size_t>(((size_t)nr * ne + 255) / 256, 4096), 256, 0, st>>>(
+            part, S, nr, exps + r0, d_E, e0, ne, NE, energy_scale, n_over_omega, d_out + (size_t)r0 * NE);
+        check_launch("k_kpm_unscale");
+      }
+    }
+    int flag = 0;
+    check_cuda(cudaMemcpyAsync(&flag, err, sizeof(int), cudaMemcpyDeviceToHost, st), "status readback");
+    check_cuda(cudaStreamSynchronize(st), "gqt_kpm_reconstruct");
+    if (flag) throw Error(GQT_ETIMEOUT, "gqt_kpm_reconstruct: a bounded tensor-core wait gave up");
+    return GQT_OK;
+  }
   check_cuda(cudaStreamSynchronize(st), "gqt_kpm_reconstruct");
   API_END
 }

@@ -803,22 +803,78 @@ static __global__ void k_kpm_table(int M, const double* __restrict__ E, int NE, 
   }
 }
 
-// out[row][e] = sum_n mu[row][n] tab[n][e]: a small FP64 GEMM, 16x16 tiles.
-static __global__ void k_kpm_gemm(const double* __restrict__ mu, int rows, int M, const double* __restrict__ tab, int NE,
-                           double* __restrict__ out) {
-  __shared__ double As[16][17], Bs[16][17];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int row = blockIdx.y * 16 + ty, col = blockIdx.x * 16 + tx;
-  double acc = 0.0;
-  for (int k0 = 0; k0 < M; k0 += 16) {
-    As[ty][tx] = (row < rows && k0 + tx < M) ? mu[(size_t)row * M + k0 + tx] : 0.0;
-    Bs[ty][tx] = (k0 + ty < M && col < NE) ? tab[(size_t)(k0 + ty) * NE + col] : 0.0;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 16; ++k) acc = fma(As[ty][k], Bs[k][tx], acc);
-    __syncthreads();
+// Moment weights of the reconstruction, g_n (2 - delta_n0) (Eqs. 25, 31).
+static __global__ void k_kpm_moment_weights(int M, int jackson, double* __restrict__ w) {
+  const double a = 1.0 / (M + 1.0), cot = cospi(a) / sinpi(a);
+  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < M; n += gridDim.x * blockDim.x) {
+    const double g = jackson ? (1.0 - n * a) * cospi(n * a) + a * sinpi(n * a) * cot : 1.0;
+    w[n] = g * (n == 0 ? 1.0 : 2.0);
   }
-  if (row < rows && col < NE) out[(size_t)row * NE + col] = acc;
+}
+
+// Energy factor of the reconstruction, 2 (N/Omega) / (pi dE sqrt(1 - x^2)); NaN where |x| >= 1.
+__device__ __forceinline__ double kpm_scale(double x, double dE, double n_over_omega) {
+  return fabs(x) < 1.0 ? 2.0 * n_over_omega / (M_PI * dE * sqrt(1.0 - x * x)) : CUDART_NAN;
+}
+
+// A few rows (up to RB = 8) of a reconstruction: one warp per energy, lane l the orders
+// n = l, l + 32, ..; cos n th advances by a rotation of 32 th, taken afresh every 16
+// rotations.  Bound by the FP64 pipe (the rotations, and a multiply-add per row): two rows,
+// M = 2000, NE = 2001, 126 us, against 1455 for a table of cosines in memory and a
+// product on the FP64 pipe.  More rows than that share the angles' cost through the
+// table's slices and the product on the tensor cores.
+template <int RB>
+__global__ void __launch_bounds__(128) k_kpm_rows(const double* __restrict__ mu, int rows, int M,
+                                                  const double* __restrict__ w, const double* __restrict__ E, int NE,
+                                                  double dE, double n_over_omega, double* __restrict__ out) {
+  const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (e >= NE) return;
+  const double x = E[e] / dE, scale = kpm_scale(x, dE, n_over_omega);
+  const double th = fabs(x) < 1.0 ? acos(x) : 0.0;
+  double rs, rc, acc[RB];
+  sincos(32.0 * th, &rs, &rc);
+#pragma unroll
+  for (int q = 0; q < RB; ++q) acc[q] = 0.0;
+  for (int n0 = lane; n0 < M; n0 += 512) {
+    const double a = n0 * th, da = fma((double)n0, th, -a);
+    double sn, cn;
+    sincos(a, &sn, &cn);
+    const double c0 = cn;
+    cn = fma(-da, sn, cn);
+    sn = fma(da, c0, sn);
+    const int end = min(M, n0 + 512);
+#pragma unroll 4
+    for (int n = n0; n < end; n += 32) {
+      const double wc = w[n] * cn;
+#pragma unroll
+      for (int q = 0; q < RB; ++q)
+        if (q < rows) acc[q] = fma(wc, mu[(size_t)q * M + n], acc[q]);
+      const double v = fma(cn, rc, -sn * rs);
+      sn = fma(sn, rc, cn * rs);
+      cn = v;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < RB; ++q) {
+    for (int off = 16; off > 0; off >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off);
+    if (lane == 0 && q < rows) out[(size_t)q * NE + e] = scale * acc[q];
+  }
+}
+
+// out[row][e0 + e] = energy factor x 2^(row exponent) x sum over splits of the sliced
+// product part[split][row][e]; a row with an infinity or a NaN (biased exponent 2047)
+// is NaN.
+static __global__ void k_kpm_unscale(const double* __restrict__ part, int S, int rows, const int* __restrict__ exps,
+                                     const double* __restrict__ E, int e0, int ne, int NE, double dE,
+                                     double n_over_omega, double* __restrict__ out) {
+  const size_t total = (size_t)rows * ne;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
+    const int r = (int)(t / ne), e = e0 + (int)(t % ne);
+    double v = 0.0;
+    for (int q = 0; q < S; ++q) v += part[(size_t)q * total + t];
+    const int ex = exps[r];
+    out[(size_t)r * NE + e] = kpm_scale(E[e] / dE, dE, n_over_omega) * (ex == 2047 ? CUDART_NAN : scalbn(v, ex - 1022));
+  }
 }
 
 // --------------------------------------------------------------- sigma
@@ -828,6 +884,7 @@ static __global__ void k_sigma_vac(const double* __restrict__ v, const double* _
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < NE; e += gridDim.x * blockDim.x) {
     double s = 0.0;
     out[e] = 0.0;
+#pragma unroll 8
     for (int k = 1; k < Nt; ++k) {
       s += 0.5 * dt[k - 1] * (v[(size_t)(k - 1) * NE + e] + v[(size_t)k * NE + e]);
       out[(size_t)k * NE + e] = s;
@@ -839,6 +896,7 @@ static __global__ void k_sigma_msd(const double* __restrict__ m, const double* _
                             double* __restrict__ out) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < NE; e += gridDim.x * blockDim.x) {
     double prev = 0.0;
+#pragma unroll 8
     for (int k = 0; k < Nt; ++k) {
       const double c = m[(size_t)k * NE + e];
       out[(size_t)k * NE + e] = (c - prev) / (2.0 * dt[k]);

@@ -382,6 +382,45 @@ __global__ void __launch_bounds__(128) k_slice_rows(const double* __restrict__ x
   }
 }
 
+// Slices of the Chebyshev table cos(n th_e), x_e = E_e / dE = cos th_e, rows e, n < m
+// (zeros past it, and in rows with |x_e| >= 1), scaled by 2^0: out[slice][chunk][e][16].
+// A thread runs through 64 orders of one energy by rotations of th, from a first angle
+// n0 th whose rounding is taken into account to first order.  M = 500, NE = 1001: 54 us,
+// the FP64 pipe's (4 multiply-adds an entry, an angle every 64); the table in memory, one
+// acos and cosine an entry, took 874.
+__global__ void __launch_bounds__(128) k_cos_slices(const double* __restrict__ E, int ne, double inv_dE, int m,
+                                                    int nchunk, __half* __restrict__ out) {
+  const int groups = (nchunk + 3) / 4;
+  const size_t total = (size_t)groups * ne, plane = (size_t)nchunk * ne * SG_K;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
+    const int e = (int)(t % ne), g = (int)(t / ne);
+    const double x = E[e] * inv_dE;
+    const bool in = fabs(x) < 1.0;
+    const double th = in ? acos(x) : 0.0, sx = in ? sqrt((1.0 - x) * (1.0 + x)) : 0.0;
+    const double n0 = 64.0 * g, a = n0 * th, da = fma(n0, th, -a);
+    double sn, cn;
+    sincos(a, &sn, &cn);
+    const double c0 = cn;
+    cn = fma(-da, sn, cn);
+    sn = fma(da, c0, sn);
+    for (int c = 4 * g; c < min(nchunk, 4 * g + 4); ++c)
+      for (int half = 0; half < 2; ++half) {
+        Digits d;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int n = c * SG_K + half * 8 + q;
+          d.set(q, in && n < m ? fmin(1.0, fmax(-1.0, cn)) : 0.0, 0);
+          const double v = fma(cn, x, -sn * sx);
+          sn = fma(sn, x, cn * sx);
+          cn = v;
+        }
+        __half* dst = out + ((size_t)c * ne + e) * SG_K + half * 8;
+#pragma unroll
+        for (int i = 0; i < SL; ++i) *reinterpret_cast<uint4*>(dst + i * plane) = d.slice(i);
+      }
+  }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encoder() {
   static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
     void* p = nullptr;
@@ -433,6 +472,13 @@ void launch_slice_rows(const double* x, int comp, int rows, size_t stride, size_
   else
     k_slice_rows<1><<<grid, 128, 0, st>>>(x, stride, k, k0, w, rows, nchunk, exps, (__half*)out);
   check_launch("k_slice_rows");
+}
+
+void launch_cos_slices(const double* E, int ne, double dE, int m, int nchunk, void* out, cudaStream_t st) {
+  const size_t total = (size_t)((nchunk + 3) / 4) * ne;
+  k_cos_slices<<<(int)std::min<size_t>((total + 127) / 128, (size_t)sm_count() * 32), 128, 0, st>>>(
+      E, ne, 1.0 / dE, m, nchunk, (__half*)out);
+  check_launch("k_cos_slices");
 }
 
 int slice_splits(int rows_a, int rows_b, int parts, int nchunk) {

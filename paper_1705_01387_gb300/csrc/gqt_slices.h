@@ -33,6 +33,8 @@ void launch_row_exps(const double* x, int comp, int rows, size_t stride, size_t 
 // Slices of elements [k0, k0 + 16 nchunk) of each row (zeros past k).
 void launch_slice_rows(const double* x, int comp, int rows, size_t stride, size_t k, size_t k0, const double* w,
                        int nchunk, const int* exps, void* out, cudaStream_t st);
+// Slices of cos(n acos(E_e / dE)), n < m, rows e < ne, at scale 2^0 (zeros where |E| >= dE).
+void launch_cos_slices(const double* E, int ne, double dE, int m, int nchunk, void* out, cudaStream_t st);
 int slice_splits(int rows_a, int rows_b, int parts, int nchunk);
 // out[split][part][rows_a][rows_b] (+)= the products of the scaled rows: times
 // 2^(exp_a - 1022 + exp_b - 1022) for the true values.  *err: bits 16, 32 (see above).
