@@ -175,7 +175,7 @@ void gqt::prof_end(size_t i, int cat, cudaStream_t st) {
 
 // ====================================================================== handle
 
-static bool is_pow2_r(int R) { return R == 1 || R == 2 || R == 4 || R == 8 || R == 16 || R == 32; }
+
 
 // Next-iteration prefetch of the multi-vector kernels (FP32 storage, where the
 // dependent index load bounds the iteration): needs a lane group of at least K + 1
@@ -373,27 +373,6 @@ DevBuf& gqt_ham::ws(int slot, size_t bytes) {
 // ====================================================================== dispatch helpers
 
 size_t gqt_ham::vec_bytes(int R) const { return (size_t)n * R * (prec == GQT_FP64 ? 16 : 8); }
-
-// ====================================================================== status
-
-static gqt_status finish_call(gqt_ham* h, cudaStream_t st, const char* what) {
-  int flag = 0;
-  check_cuda(cudaMemcpyAsync(h->h_flag, h->d_flag.p, sizeof(int), cudaMemcpyDeviceToHost, st), "flag readback");
-  check_cuda(cudaStreamSynchronize(st), what);
-  flag = *h->h_flag;
-  if (flag & 4) throw Error(GQT_ENAN, std::string(what) + ": NaN or Inf in a result");
-  if (flag & 2)
-    throw Error(GQT_ERANGE, std::string(what) +
-                                ": a Chebyshev moment exceeds |l||r|: the spectrum of H/dE is not inside [-1,1] "
-                                "(energy scale too small)");
-  if (flag & 8) throw Error(GQT_ENORM, std::string(what) + ": |U psi| differs from |psi| beyond tolerance");
-  if (flag & 16) throw Error(GQT_ETIMEOUT, std::string(what) + ": a bounded device wait gave up");
-  return GQT_OK;
-}
-
-static void reset_flag(gqt_ham* h, cudaStream_t st) {
-  check_cuda(cudaMemsetAsync(h->d_flag.p, 0, sizeof(int), st), "flag reset");
-}
 
 // ====================================================================== moments core
 
@@ -1197,49 +1176,6 @@ void gqt::launch_velocity(gqt_ham* h, const void* x, void* y, void* ycopy, int R
   });
 }
 
-// ====================================================================== API helpers
-
-#define API_BEGIN \
-  gqt::NvtxRange nvtx_call_(__func__); \
-  try {
-#define API_END                                        \
-  }                                                    \
-  catch (const Error& e) {                             \
-    set_error(e.what());                               \
-    return e.code;                                     \
-  }                                                    \
-  catch (const std::bad_alloc&) {                      \
-    set_error("host allocation failed");               \
-    return GQT_ENOMEM;                                 \
-  }                                                    \
-  catch (const std::exception& e) {                    \
-    set_error(std::string("internal error: ") + e.what()); \
-    return GQT_EINVAL;                                 \
-  }                                                    \
-  return GQT_OK;
-
-static void require(bool c, const std::string& msg) {
-  if (!c) throw Error(GQT_EINVAL, msg);
-}
-
-static bool is_host_ptr(const void* p) {
-  cudaPointerAttributes a;
-  cudaError_t e = cudaPointerGetAttributes(&a, p);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return true;
-  }
-  return a.type == cudaMemoryTypeUnregistered || a.type == cudaMemoryTypeHost;
-}
-
-static void check_common(gqt_ham* h, int R) {
-  require(h != nullptr, "null handle");
-  require(is_pow2_r(R), "R must be 1, 2, 4, 8, 16 or 32");
-  int dev = -1;
-  check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
-  require(dev == h->device, "the current CUDA device is not the handle's device");
-}
-
 // Copy a device result to the caller's pointer (host or device).
 static void deliver(const void* dsrc, double* dst, size_t bytes, cudaStream_t st) {
   if (is_host_ptr(dst))
@@ -1280,12 +1216,6 @@ static void stage_out(const StagedPair& s, cudaStream_t st) {
   if (!s.hx) return;
   check_cuda(cudaMemcpyAsync(s.hx, s.x, s.bytes, cudaMemcpyDeviceToHost, st), "state download");
   check_cuda(cudaMemcpyAsync(s.hy, s.y, s.bytes, cudaMemcpyDeviceToHost, st), "state download");
-}
-
-static int resolve_np(gqt_ham* h, double dt, int Np) {
-  require(std::isfinite(dt) && dt >= 0.0, "time step must be finite and >= 0");
-  if (Np > 0) return Np;
-  return np_rule_lib(h->dE * dt, 4096);
 }
 
 // ====================================================================== C ABI
@@ -1735,191 +1665,6 @@ gqt_status gqt_sigma_msd(const double* d_msd, const double* dt, int Nt, int NE, 
 }
 
 }  // extern "C"
-
-// ====================================================================== adjoint (K9)
-
-namespace {
-
-// Adds to (gdiag, gslot) the gradient of J = Re sum_{m<P} coef_m <lam|T_m(H~)|r>
-// and writes rbar = sum_m conj(coef_m) T_m lam (dJ = Re <rbar|dr>).  If lbar is
-// non-null it receives sum_m coef_m T_m r (FP64).  u_m = T_m r is recomputed
-// from checkpoint pairs (u_c, u_{c+1}) taken every `stride` orders.
-template <class HT>
-void poly_adjoint(gqt_ham* h, const HT& H, const void* r, const void* lam, const std::vector<double2>& coef,
-                  int stride, void* rbar, double2* lbar, double* gdiag, double2* gslot, cudaStream_t st) {
-  using Tr = EllTraits<HT>;
-  using V = typename Tr::V;
-  const int P = (int)coef.size();
-  const BlockTable& T = h->table(1);
-  const int nb = T.nblocks;
-  const int* blk = (const int*)T.d_blk.p;
-  const size_t vb = h->vec_bytes(1);
-  const int s = std::max(2, stride);
-  const int nck = (P + s - 1) / s;
-  char* ck = (char*)h->ws(WS_ADJ0, (size_t)2 * nck * vb).p;
-  char* seg = (char*)h->ws(WS_ADJ0 + 1, (size_t)s * vb).p;
-  V* WA = (V*)h->ws(WS_ADJ0 + 2, vb).p;
-  V* WB = (V*)h->ws(WS_ADJ0 + 3, vb).p;
-  auto ckp = [&](int j, int q) { return (V*)(ck + ((size_t)2 * j + q) * vb); };
-  const double2 z = make_double2(0.0, 0.0);
-  const int thr = h->threads;
-  std::vector<double> cdata(2 * coef.size());
-  for (size_t q = 0; q < coef.size(); ++q) {
-    cdata[2 * q] = coef[q].x;
-    cdata[2 * q + 1] = coef[q].y;
-  }
-  const std::string key = key_of("padj", {r, lam, rbar, lbar, gdiag, gslot, ck, seg, WA, WB, blk},
-                                 {(double)P, (double)s, (double)thr});
-  run_graph(h, key, st, [&](cudaStream_t s2) {
-    // forward pass: checkpoints (and lbar)
-    check_cuda(cudaMemcpyAsync(ckp(0, 0), r, vb, cudaMemcpyDeviceToDevice, s2), "checkpoint");
-    if (P > 1) {
-      k_recur<Tr::fp64, Tr::ch><<<nb, thr, 0, s2>>>(H, blk, (const V*)r, nullptr, WA, lbar, coef[0], coef[1], 1);
-      check_launch("k_recur(first)");
-      if (1 % s == 1) check_cuda(cudaMemcpyAsync(ckp(0, 1), WA, vb, cudaMemcpyDeviceToDevice, s2), "checkpoint");
-    } else if (lbar) {
-      k_recur<Tr::fp64, Tr::ch><<<nb, thr, 0, s2>>>(H, blk, (const V*)r, nullptr, WA, lbar, coef[0], z, 1);
-      check_launch("k_recur(first)");
-    }
-    const V* um2 = (const V*)r;
-    V* um1 = WA;
-    for (int m = 2; m < P; ++m) {
-      V* out = (m == 2) ? WB : const_cast<V*>(um2);
-      k_recur<Tr::fp64, Tr::ch><<<nb, thr, 0, s2>>>(H, blk, um1, um2, out, lbar, z, coef[m], 0);
-      check_launch("k_recur");
-      if (m % s == 0) check_cuda(cudaMemcpyAsync(ckp(m / s, 0), out, vb, cudaMemcpyDeviceToDevice, s2), "checkpoint");
-      if (m % s == 1) check_cuda(cudaMemcpyAsync(ckp(m / s, 1), out, vb, cudaMemcpyDeviceToDevice, s2), "checkpoint");
-      um2 = um1;
-      um1 = out;
-    }
-    // backward pass
-    check_cuda(cudaMemsetAsync(WA, 0, vb, s2), "memset");
-    check_cuda(cudaMemsetAsync(WB, 0, vb, s2), "memset");
-    V* X = WA;  // w_{m+1}
-    V* Y = WB;  // w_{m+2} -> w_m
-    for (int j = nck - 1; j >= 0; --j) {
-      const int c = j * s;
-      const int len = std::min(s, P - c);
-      std::vector<const V*> useg(len);
-      for (int q = 0; q < len; ++q) {
-        if (q < 2) {
-          useg[q] = ckp(j, q);
-        } else {
-          V* o = (V*)(seg + (size_t)q * vb);
-          k_recur<Tr::fp64, Tr::ch><<<nb, thr, 0, s2>>>(H, blk, useg[q - 1], useg[q - 2], o, nullptr, z, z, 0);
-          check_launch("k_recur(segment)");
-          useg[q] = o;
-        }
-      }
-      for (int m = std::min(c + len, P - 1); m >= c + 1; --m) {
-        const double2 lc = make_double2(coef[m].x, -coef[m].y);
-        const double f = (m == 1 ? 1.0 : 2.0) / h->dE;
-        k_adj_step<Tr::fp64, Tr::ch><<<nb, thr, 0, s2>>>(H, blk, X, Y, (const V*)lam, lc, useg[m - 1 - c], f, gdiag,
-                                                           gslot);
-        check_launch("k_adj_step");
-        std::swap(X, Y);
-      }
-    }
-    const double2 lc0 = make_double2(coef[0].x, -coef[0].y);
-    k_adj_final<Tr::fp64, Tr::ch><<<nb, thr, 0, s2>>>(H, blk, P > 1 ? X : nullptr, Y, (const V*)lam, lc0, (V*)rbar);
-    check_launch("k_adj_final");
-  }, &cdata);
-}
-
-}  // namespace
-
-extern "C" gqt_status gqt_vac_loss_grad(gqt_ham* h, const void* d_phi, const double* dt, const int* Np, int Nt,
-                                        int M, const double* beta, int stride, double* loss, double* d_g_onsite,
-                                        double* d_g_slot, void* stream) {
-  API_BEGIN
-  check_common(h, 1);
-  require(d_phi && dt && beta && loss && d_g_onsite && d_g_slot && Nt >= 1 && M >= 1, "gqt_vac_loss_grad: bad argument");
-  require(h->nseg == 1, "gqt_vac_loss_grad: single-segment handles only");
-  cudaStream_t st = (cudaStream_t)stream;
-  reset_flag(h, st);
-  const int64_t n = h->n;
-  const int K = h->K;
-  const size_t vb = h->vec_bytes(1);
-  const BlockTable& T = h->table(1);
-  const int nb = T.nblocks;
-  const int* blk = (const int*)T.d_blk.p;
-  const int thr = h->threads;
-  if (stride <= 0) stride = (int)std::ceil(std::sqrt((double)M));
-  std::vector<double> hbeta;
-  if (!is_host_ptr(beta)) {  // device weights: one copy to the host (they become kernel arguments)
-    hbeta.resize((size_t)Nt * M);
-    check_cuda(cudaMemcpy(hbeta.data(), beta, hbeta.size() * sizeof(double), cudaMemcpyDeviceToHost), "beta");
-    beta = hbeta.data();
-  }
-  char* A = (char*)h->ws(WS_ADJ0 + 4, (size_t)Nt * vb).p;
-  char* B = (char*)h->ws(WS_ADJ0 + 5, (size_t)Nt * vb).p;
-  double* gdiag = (double*)h->ws(WS_ADJ0 + 6, (size_t)n * sizeof(double)).p;
-  double2* gslot = (double2*)h->ws(WS_ADJ0 + 7, (size_t)n * K * sizeof(double2)).p;
-  void* abar = h->ws(WS_ADJ0 + 8, vb).p;
-  void* bbar = h->ws(WS_ADJ0 + 9, vb).p;
-  double2* LB = (double2*)h->ws(WS_ADJ0 + 10, (size_t)n * sizeof(double2)).p;
-  void* tmp = h->ws(WS_ADJ0 + 11, vb).p;
-  void* l = h->ws(WS_L, vb).p;
-  double* dpart = (double*)h->ws(WS_ADJ0 + 12, (size_t)Nt * nb * sizeof(double)).p;  // loss partials per row
-  auto Ak = [&](int k) { return (void*)(A + (size_t)k * vb); };
-  auto Bk = [&](int k) { return (void*)(B + (size_t)k * vb); };
-  // forward states a_k = U(-t_k) phi, b_k = U(-t_k) V phi
-  launch_velocity(h, d_phi, Bk(0), Ak(0), 1, st);
-  std::vector<int> nps(Nt);
-  for (int k = 0; k < Nt; ++k) nps[k] = resolve_np(h, dt[k], Np ? Np[k] : 0);
-  for (int k = 0; k + 1 < Nt; ++k) {
-    check_cuda(cudaMemcpyAsync(Ak(k + 1), Ak(k), vb, cudaMemcpyDeviceToDevice, st), "copy");
-    check_cuda(cudaMemcpyAsync(Bk(k + 1), Bk(k), vb, cudaMemcpyDeviceToDevice, st), "copy");
-    void* sets[2] = {Ak(k + 1), Bk(k + 1)};
-    launch_evolve_sets<2>(h, sets, 1, evolve_coefs(h->dE * dt[k], -1, nps[k]), st, nullptr);
-  }
-  check_cuda(cudaMemsetAsync(gdiag, 0, (size_t)n * sizeof(double), st), "memset");
-  check_cuda(cudaMemsetAsync(gslot, 0, (size_t)n * K * sizeof(double2), st), "memset");
-  check_cuda(cudaMemsetAsync(abar, 0, vb, st), "memset");
-  check_cuda(cudaMemsetAsync(bbar, 0, vb, st), "memset");
-  std::vector<double> hpart((size_t)Nt * nb);
-  double total = 0.0;
-  dispatch(h, [&](auto H) {
-    using Tr = EllTraits<decltype(H)>;
-    using V = typename Tr::V;
-    for (int k = Nt - 1; k >= 0; --k) {
-      if (k + 1 < Nt) {
-        const auto c = evolve_coefs(h->dE * dt[k], -1, nps[k]);
-        poly_adjoint(h, H, Ak(k), abar, c, std::max(2, (int)std::ceil(std::sqrt((double)c.size()))), tmp, nullptr,
-                     gdiag, gslot, st);
-        std::swap(abar, tmp);
-        poly_adjoint(h, H, Bk(k), bbar, c, std::max(2, (int)std::ceil(std::sqrt((double)c.size()))), tmp, nullptr,
-                     gdiag, gslot, st);
-        std::swap(bbar, tmp);
-      }
-      launch_velocity(h, Ak(k), l, nullptr, 1, st);
-      std::vector<double2> bc(M);
-      for (int m = 0; m < M; ++m) bc[m] = make_double2(beta[(size_t)k * M + m], 0.0);
-      poly_adjoint(h, H, Bk(k), l, bc, stride, tmp, LB, gdiag, gslot, st);
-      k_axpy<V><<<nb, thr, 0, st>>>(blk, (V*)bbar, (const V*)tmp);
-      check_launch("k_axpy");
-      k_dot_re<V><<<nb, thr, 0, st>>>(blk, (const V*)l, LB, dpart + (size_t)k * nb);
-      check_launch("k_dot_re");
-      k_vel_adj<Tr::fp64, Tr::ch, double2><<<nb, thr, 0, st>>>(H, blk, LB, (const V*)Ak(k), gslot);
-      check_launch("k_vel_adj");
-      k_vel_acc<Tr::fp64, Tr::ch><<<nb, thr, 0, st>>>(H, blk, 0.5 * h->dE, LB, (V*)abar);
-      check_launch("k_vel_acc");
-    }
-    k_vel_adj<Tr::fp64, Tr::ch, V><<<nb, thr, 0, st>>>(H, blk, (const V*)bbar, (const V*)d_phi, gslot);
-    check_launch("k_vel_adj");
-  });
-  const size_t tot = (size_t)n * K;
-  k_grad_out<<<(int)std::min<size_t>((tot + 255) / 256, 8192), 256, 0, st>>>((int)n, K, gslot, gdiag,
-                                                                            (double2*)d_g_slot, d_g_onsite);
-  check_launch("k_grad_out");
-  check_cuda(cudaMemcpyAsync(hpart.data(), dpart, hpart.size() * sizeof(double), cudaMemcpyDeviceToHost, st), "loss");
-  check_cuda(cudaStreamSynchronize(st), "loss");
-  for (int k = Nt - 1; k >= 0; --k)  // the order the rows were summed before: last row first
-    for (int b = 0; b < nb; ++b) total += hpart[(size_t)k * nb + b];
-  *loss = total;
-  return finish_call(h, st, "gqt_vac_loss_grad");
-  API_END
-}
 
 extern "C" gqt_status gqt_kpm_weights(int M, const double* d_E, int NE, const double* d_w, double energy_scale,
                                       double n_over_omega, int kernel, double* d_beta, void* stream) {

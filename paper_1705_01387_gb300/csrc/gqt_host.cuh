@@ -22,6 +22,9 @@ namespace gqt {
 extern std::atomic<uint64_t> g_launches;
 bool prof_on();
 
+// (2 - delta_m0) (-sign i)^m J_m(x), m < Np (Eq. 17).
+std::vector<double2> evolve_coefs(double x, int sign, int Np);
+
 // 2H~, 2U/dE (and 2[X,H~]) of an FP64 handle as pairs of FP32 numbers, split on first
 // use and after an update, on the call's stream and before any capture.
 void ensure_df(gqt_ham* h, cudaStream_t st);
@@ -225,6 +228,78 @@ inline void launch_split(void* const* in, float4* const* out, size_t n, cudaStre
   }
   k_split_vec<NV><<<(int)std::min<size_t>((n + 255) / 256, (size_t)sm_count() * 8), 256, 0, st>>>(A, n);
   check_launch("k_split_vec");
+}
+
+inline bool is_pow2_r(int R) { return R == 1 || R == 2 || R == 4 || R == 8 || R == 16 || R == 32; }
+
+// ---------------------------------------------------------------- status
+
+inline gqt_status finish_call(gqt_ham* h, cudaStream_t st, const char* what) {
+  int flag = 0;
+  check_cuda(cudaMemcpyAsync(h->h_flag, h->d_flag.p, sizeof(int), cudaMemcpyDeviceToHost, st), "flag readback");
+  check_cuda(cudaStreamSynchronize(st), what);
+  flag = *h->h_flag;
+  if (flag & 4) throw Error(GQT_ENAN, std::string(what) + ": NaN or Inf in a result");
+  if (flag & 2)
+    throw Error(GQT_ERANGE, std::string(what) +
+                                ": a Chebyshev moment exceeds |l||r|: the spectrum of H/dE is not inside [-1,1] "
+                                "(energy scale too small)");
+  if (flag & 8) throw Error(GQT_ENORM, std::string(what) + ": |U psi| differs from |psi| beyond tolerance");
+  if (flag & 16) throw Error(GQT_ETIMEOUT, std::string(what) + ": a bounded device wait gave up");
+  return GQT_OK;
+}
+
+inline void reset_flag(gqt_ham* h, cudaStream_t st) {
+  check_cuda(cudaMemsetAsync(h->d_flag.p, 0, sizeof(int), st), "flag reset");
+}
+
+// ---------------------------------------------------------------- API helpers
+
+#define API_BEGIN \
+  gqt::NvtxRange nvtx_call_(__func__); \
+  try {
+#define API_END                                        \
+  }                                                    \
+  catch (const Error& e) {                             \
+    set_error(e.what());                               \
+    return e.code;                                     \
+  }                                                    \
+  catch (const std::bad_alloc&) {                      \
+    set_error("host allocation failed");               \
+    return GQT_ENOMEM;                                 \
+  }                                                    \
+  catch (const std::exception& e) {                    \
+    set_error(std::string("internal error: ") + e.what()); \
+    return GQT_EINVAL;                                 \
+  }                                                    \
+  return GQT_OK;
+
+inline void require(bool c, const std::string& msg) {
+  if (!c) throw Error(GQT_EINVAL, msg);
+}
+
+inline bool is_host_ptr(const void* p) {
+  cudaPointerAttributes a;
+  cudaError_t e = cudaPointerGetAttributes(&a, p);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return a.type == cudaMemoryTypeUnregistered || a.type == cudaMemoryTypeHost;
+}
+
+inline void check_common(gqt_ham* h, int R) {
+  require(h != nullptr, "null handle");
+  require(is_pow2_r(R), "R must be 1, 2, 4, 8, 16 or 32");
+  int dev = -1;
+  check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
+  require(dev == h->device, "the current CUDA device is not the handle's device");
+}
+
+inline int resolve_np(gqt_ham* h, double dt, int Np) {
+  require(std::isfinite(dt) && dt >= 0.0, "time step must be finite and >= 0");
+  if (Np > 0) return Np;
+  return np_rule_lib(h->dE * dt, 4096);
 }
 
 }  // namespace gqt

@@ -937,194 +937,6 @@ __global__ void k_random_phase(int n, int R, const uint64_t* __restrict__ keys, 
 }  // namespace gqt
 
 namespace gqt {
-
-// ------------------------------------------------------------ K9: adjoint
-//
-// Reverse-mode derivative of J = Re sum_{m<P} coef_m <lam| T_m(H~) |r> with
-// u_m = T_m r (not in the paper; it differentiates Eqs. 17, 21 and 29).  The
-// adjoint vectors obey the transposed recurrence
-//   w_m = conj(coef_m) lam + 2 H~ w_{m+1} - w_{m+2},   w_P = w_{P+1} = 0,
-// and dJ = Re sum_ij conj(G_ij) dH~_ij with G = w_1 u_0^+ + 2 sum_{m>=2} w_m u_{m-1}^+,
-// needed only on the diagonal and the ELL slots.
-
-// Plain recurrence step: out = 2H~ t1 - t2 (first: out = H~ t1); if acc != null,
-// first: acc = cA t1 + cB out, else acc += cB out.
-template <bool FP64, bool CH>
-__global__ void k_recur(Ell<FP64, CH> H, const int* __restrict__ blk, const typename Prec<FP64>::V* __restrict__ t1,
-                        const typename Prec<FP64>::V* t2, typename Prec<FP64>::V* out, double2* __restrict__ acc,
-                        double2 cA, double2 cB, int first) {
-  using V = typename Prec<FP64>::V;
-  using S = typename Prec<FP64>::S;
-  const int b = blockIdx.x;
-  for (int i = blk[b] + threadIdx.x; i < blk[b + 1]; i += blockDim.x) {
-    V y;
-    if (first) {
-      V zero;
-      zero.x = 0;
-      zero.y = 0;
-      y = cscale(apply2h<FP64, CH>(H, t1, i, 0, 0, zero), (S)0.5);
-    } else {
-      y = apply2h<FP64, CH>(H, t1, i, 0, 0, cneg(t2[i]));
-    }
-    out[i] = y;
-    if (acc) {
-      if (first)
-        acc[i] = cfma_d(cfma_d(make_double2(0.0, 0.0), cA, __ldg(t1 + i)), cB, y);
-      else
-        acc[i] = cfma_d(acc[i], cB, y);
-    }
-  }
-}
-
-// One adjoint order m: w_m = lc lam + 2H~ w1 - w2 (w1 = w_{m+1}, w2 = w_{m+2},
-// w_m overwrites w2) and G += f w_m conj(u_{m-1}) on the diagonal (gdiag, real
-// part) and on the slots (gslot [K][n]).  f = (m == 1 ? 1 : 2) / dE.
-template <bool FP64, bool CH>
-__global__ void k_adj_step(Ell<FP64, CH> H, const int* __restrict__ blk, const typename Prec<FP64>::V* __restrict__ w1,
-                           typename Prec<FP64>::V* w2, const typename Prec<FP64>::V* __restrict__ lam, double2 lc,
-                           const typename Prec<FP64>::V* __restrict__ u, double f, double* __restrict__ gdiag,
-                           double2* __restrict__ gslot) {
-  using V = typename Prec<FP64>::V;
-  const int b = blockIdx.x;
-  for (int i = blk[b] + threadIdx.x; i < blk[b + 1]; i += blockDim.x) {
-    V y = apply2h<FP64, CH>(H, w1, i, 0, 0, cneg(w2[i]));
-    double2 wd = cfma_d(to_d2(y), lc, __ldg(lam + i));
-    const V w = from_d2<V>(wd);
-    w2[i] = w;
-    wd = to_d2(w);
-    const double2 ui = to_d2(__ldg(u + i));
-    gdiag[i] += f * (wd.x * ui.x + wd.y * ui.y);
-    for (int k = 0; k < H.K; ++k) {
-      const size_t s = (size_t)k * H.n + i;
-      const double2 uj = to_d2(__ldg(u + __ldg(H.idx + s)));
-      double2 g = gslot[s];
-      // w * conj(uj)
-      g.x += f * (wd.x * uj.x + wd.y * uj.y);
-      g.y += f * (wd.y * uj.x - wd.x * uj.y);
-      gslot[s] = g;
-    }
-  }
-}
-
-// rbar = lc0 lam + H~ w1 - w2 (Clenshaw end, = sum_m conj(coef_m) T_m lam); w1 may be null (P = 1).
-template <bool FP64, bool CH>
-__global__ void k_adj_final(Ell<FP64, CH> H, const int* __restrict__ blk, const typename Prec<FP64>::V* __restrict__ w1,
-                            const typename Prec<FP64>::V* __restrict__ w2, const typename Prec<FP64>::V* __restrict__ lam,
-                            double2 lc0, typename Prec<FP64>::V* __restrict__ rbar) {
-  using V = typename Prec<FP64>::V;
-  using S = typename Prec<FP64>::S;
-  const int b = blockIdx.x;
-  for (int i = blk[b] + threadIdx.x; i < blk[b + 1]; i += blockDim.x) {
-    double2 acc = cfma_d(make_double2(0.0, 0.0), lc0, __ldg(lam + i));
-    if (w1) {
-      V zero;
-      zero.x = 0;
-      zero.y = 0;
-      V y = cscale(apply2h<FP64, CH>(H, w1, i, 0, 0, zero), (S)0.5);
-      const double2 yd = to_d2(y), w2d = to_d2(__ldg(w2 + i));
-      acc.x += yd.x - w2d.x;
-      acc.y += yd.y - w2d.y;
-    }
-    rbar[i] = from_d2<V>(acc);
-  }
-}
-
-__device__ __forceinline__ double2 hop_d(double2 h) { return h; }
-__device__ __forceinline__ double2 hop_d(float2 h) { return to_d2(h); }
-__device__ __forceinline__ double hop_d(double h) { return h; }
-__device__ __forceinline__ double hop_d(float h) { return (double)h; }
-
-// Velocity part of the gradient: l = V x with V_ij = i dx_ij H_ij (unscaled H), so
-// G_ij += lbar_i (-i dx_ij) conj(x_j) (slots only; V has no diagonal).
-template <bool FP64, bool CH, class LB>
-__global__ void k_vel_adj(Ell<FP64, CH> H, const int* __restrict__ blk, const LB* __restrict__ lbar,
-                          const typename Prec<FP64>::V* __restrict__ x, double2* __restrict__ gslot) {
-  const int b = blockIdx.x;
-  for (int i = blk[b] + threadIdx.x; i < blk[b + 1]; i += blockDim.x) {
-    const double2 lb = to_d2(lbar[i]);
-    for (int k = 0; k < H.K; ++k) {
-      const size_t s = (size_t)k * H.n + i;
-      const double2 xj = to_d2(__ldg(x + __ldg(H.idx + s)));
-      const double d = (double)__ldg(H.dx + s);
-      // lbar * (-i d) * conj(xj) = -i d (lb.x + i lb.y)(xj.x - i xj.y)
-      const double re = lb.x * xj.x + lb.y * xj.y, im = lb.y * xj.x - lb.x * xj.y;
-      double2 g = gslot[s];
-      g.x += d * im;
-      g.y += -d * re;
-      gslot[s] = g;
-    }
-  }
-}
-
-// y += V x for a double2 accumulator y (x storage precision), V = i dE sum dx H~.
-template <bool FP64, bool CH>
-__global__ void k_vel_acc(Ell<FP64, CH> H, const int* __restrict__ blk, double half_dE,
-                          const double2* __restrict__ x, typename Prec<FP64>::V* __restrict__ y) {
-  using V = typename Prec<FP64>::V;
-  const int b = blockIdx.x;
-  for (int i = blk[b] + threadIdx.x; i < blk[b + 1]; i += blockDim.x) {
-    double2 a = make_double2(0.0, 0.0);
-    for (int k = 0; k < H.K; ++k) {
-      const size_t s = (size_t)k * H.n + i;
-      const int j = __ldg(H.idx + s);
-      const double d = (double)__ldg(H.dx + s);
-      a = cmul_acc(a, hop_d(__ldg(H.hop2 + s)), cscale(x[j], d));
-    }
-    double2 yo = to_d2(y[i]);
-    yo.x += -a.y * half_dE;
-    yo.y += a.x * half_dE;
-    y[i] = from_d2<V>(yo);
-  }
-}
-
-// Re <l|x> partial sums per CTA (x double2).
-template <class V>
-__global__ void k_dot_re(const int* __restrict__ blk, const V* __restrict__ l, const double2* __restrict__ x,
-                         double* __restrict__ partial) {
-  __shared__ double sh[32];
-  const int b = blockIdx.x;
-  double s = 0.0;
-  for (int i = blk[b] + threadIdx.x; i < blk[b + 1]; i += blockDim.x) {
-    const double2 lv = to_d2(l[i]);
-    const double2 xv = x[i];
-    s += lv.x * xv.x + lv.y * xv.y;
-  }
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-    partial[b] = t;
-  }
-}
-
-// y += x (storage precision).
-template <class V>
-__global__ void k_axpy(const int* __restrict__ blk, V* __restrict__ y, const V* __restrict__ x) {
-  const int b = blockIdx.x;
-  for (int i = blk[b] + threadIdx.x; i < blk[b + 1]; i += blockDim.x) {
-    V a = y[i];
-    const V c = x[i];
-    a.x += c.x;
-    a.y += c.y;
-    y[i] = a;
-  }
-}
-
-// Slot-major [K][n] double2 -> row-major [n][K] double2; diagonal copied.
-static __global__ void k_grad_out(int n, int K, const double2* __restrict__ gslot, const double* __restrict__ gdiag,
-                           double2* __restrict__ out_slot, double* __restrict__ out_diag) {
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)n * K; t += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t / K), k = (int)(t % K);
-    out_slot[t] = gslot[(size_t)k * n + i];
-    if (k == 0) out_diag[i] = gdiag[i];
-  }
-}
-
-}  // namespace gqt
-
-namespace gqt {
 // beta[n] = sum_e w[e] tab[n][e]: the transpose of the reconstruction (the weight
 // each moment carries in a weighted sum of reconstructed values).  NaN entries of
 // the table (|E| >= dE) must carry zero weight and are skipped when w[e] == 0.
