@@ -8,6 +8,7 @@
 #include <cmath>
 #include <complex>
 #include <cstring>
+#include <map>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -313,6 +314,43 @@ static int64_t detect_honeycomb(const HostModel& m, int (&type)[2][3]) {
   return 0;
 }
 
+// Row classes of a model (gqt_ham::d_cls): the distinct offset vectors of its rows in
+// order of appearance, and each row's class.  False for an irregular model (more than
+// ROW_CLASSES of them) or more than 8 slots.
+constexpr int ROW_CLASSES = 4096;
+static bool row_classes(const HostModel& m, std::vector<uint16_t>& cls, std::vector<int32_t>& off) {
+  const int K = m.K;
+  if (K > 8) return false;
+  cls.resize(m.n);
+  std::map<std::vector<int32_t>, int> known;
+  std::vector<int32_t> o(K);
+  auto same = [&](int64_t i, int c) {
+    for (int k = 0; k < K; ++k)
+      if (m.idx[i * K + k] - (int32_t)i != off[8 * c + k]) return false;
+    return true;
+  };
+  for (int64_t i = 0; i < m.n; ++i) {
+    int c = -1;
+    for (int64_t b = 1; b <= 2 && c < 0 && i >= b; ++b)  // most rows repeat one of the two before
+      if (same(i, cls[i - b])) c = cls[i - b];
+    if (c < 0) {
+      for (int k = 0; k < K; ++k) o[k] = m.idx[i * K + k] - (int32_t)i;
+      auto it = known.find(o);
+      if (it != known.end()) {
+        c = it->second;
+      } else {
+        c = (int)known.size();
+        if (c == ROW_CLASSES) return false;
+        known.emplace(o, c);
+        off.insert(off.end(), o.begin(), o.end());
+        off.resize((size_t)8 * (c + 1), 0);
+      }
+    }
+    cls[i] = (uint16_t)c;
+  }
+  return true;
+}
+
 extern "C" gqt_status gqt_build_hamiltonian(const gqt_lattice* lattice, double energy_scale, gqt_precision precision,
                                             const int64_t* seg_offsets, int nseg, gqt_ham** out) {
   gqt::NvtxRange nvtx_call_(__func__);
@@ -422,6 +460,8 @@ extern "C" gqt_status gqt_build_hamiltonian(const gqt_lattice* lattice, double e
       upload(h->d_hop, hop.data(), hop.size() * 4);
       upload(h->d_diag, dg.data(), dg.size() * 4);
       upload(h->d_dx, dxv.data(), dxv.size() * 4);
+      h->hop_uniform32 = hop_real && std::all_of(hop.begin(), hop.end(), [&](float v) { return v == hop[0]; });
+      h->hop0f = h->hop_uniform32 ? hop[0] : 0.f;
     }
     // y displacements (FP64, slot-major) for the Hall moments
     h->has_dy = m.has_dy;
@@ -447,6 +487,15 @@ extern "C" gqt_status gqt_build_hamiltonian(const gqt_lattice* lattice, double e
       int sh = 0;
       while ((int64_t(1) << sh) < L) ++sh;
       if (L >= 64 && (int64_t(1) << sh) == L) h->row_shift = sh;
+    }
+    {
+      std::vector<uint16_t> cls;
+      std::vector<int32_t> off;
+      if (row_classes(m, cls, off)) {
+        upload(h->d_cls, cls.data(), cls.size() * 2);
+        upload(h->d_cls_off, off.data(), off.size() * 4);
+        h->has_cls = true;
+      }
     }
     if (nseg == 1) {
       h->honey_L1 = (int)detect_honeycomb(m, h->honey_type);
@@ -581,6 +630,15 @@ extern "C" gqt_status gqt_update_hamiltonian(gqt_ham* h, const double* onsite, c
       }
       put(h->d_hop, hop.data(), hop.size() * 4);
       put(h->d_diag, dg.data(), dg.size() * 4);
+      const bool uni = hw == 1 && std::all_of(hop.begin(), hop.end(), [&](float v) { return v == hop[0]; });
+      const float h0 = uni ? hop[0] : 0.f;
+      if (uni != h->hop_uniform32 || h0 != h->hop0f) {  // a kernel argument of the captured graphs
+        for (auto& gr : h->graphs) cudaGraphExecDestroy(gr.second);
+        h->graphs.clear();
+        h->graph_data.clear();
+      }
+      h->hop_uniform32 = uni;
+      h->hop0f = h0;
     }
     return GQT_OK;
   } catch (const Error& e) {

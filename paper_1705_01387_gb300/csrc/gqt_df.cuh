@@ -49,6 +49,8 @@ struct DfEll {
   const int* idx = nullptr;                    // [K][n]
   const typename DfHop<CH>::T* hop = nullptr;  // [K][n]
   const float2* diag = nullptr;                // [n]
+  const uint16_t* cls = nullptr;    // row classes (row_neighbours)
+  const int* cls_off = nullptr;
   const typename DfHop<CH>::T* xhop = nullptr;  // [K][n] 2[X,H~]_ij = -dx_ij 2H~_ij (commutator orders)
   float2 h0 = {0.f, 0.f};  // the common 2H~_ij of handles whose slots all hold one real hopping
 };
@@ -325,7 +327,7 @@ __device__ __forceinline__ float4 df_step_any(const DfEll<CH>& H, const typename
 // Re <A_{m-1}|B_{m-1}> (moment slot 2m-2) and Re <A_{m-1}|B_m> (slot 2m-1); the
 // first step also adds |l|^2 and |r|^2 (slot_norm).  l and r are split before it
 // (k_split_vec).  R = 1, wavefront CTA order, one element per thread.
-template <bool CH, int KK, bool FIRST>
+template <bool CH, int KK, bool FIRST, bool UH>
 __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4* __restrict__ tab,
                                                          const float4* __restrict__ am1,
                                                          const float4* __restrict__ bm1, const float4* am2,
@@ -343,12 +345,10 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
     const int i = (int)e;
     int idx[KK];
     HT hv[KK];
+    row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, row_class(H.cls, i), idx);
+    if (!UH)
 #pragma unroll
-    for (int k = 0; k < KK; ++k) {
-      const size_t s = (size_t)k * H.n + i;
-      idx[k] = __ldg(H.idx + s);
-      hv[k] = __ldg(H.hop + s);
-    }
+      for (int k = 0; k < KK; ++k) hv[k] = __ldg(H.hop + (size_t)k * H.n + i);
     const float2 dg = __ldg(H.diag + i);
     const float4 ao = __ldg(am1 + e), bo = __ldg(bm1 + e);
     float4 a2 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = a2;
@@ -362,8 +362,8 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
       na[k] = __ldg(am1 + idx[k]);
       nbv[k] = __ldg(bm1 + idx[k]);
     }
-    const float4 a = df_step<CH, KK, FIRST>(hv, dg, ao, na, a2);
-    const float4 bb = df_step<CH, KK, FIRST>(hv, dg, bo, nbv, b2);
+    const float4 a = df_step_any<CH, KK, FIRST, UH>(H, hv, dg, ao, na, a2);
+    const float4 bb = df_step_any<CH, KK, FIRST, UH>(H, hv, dg, bo, nbv, b2);
     aout[e] = a;
     bout[e] = bb;
     d0.add_re(ao, bo);
@@ -396,8 +396,8 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
 // k_cheb_dbl_w): step m writes u_m and adds <u_{m-1}|u_{m-1}> (slot 2m-2) and
 // Re <u_m|u_{m-1}> (slot 2m-1).  R = 1, wavefront CTA order, U elements in flight
 // per thread.
-template <bool CH, int KK, int U, bool FIRST>
-__global__ void __launch_bounds__(256, 3) k_cheb_dbl_df(DfEll<CH> H, const int4* __restrict__ tab,
+template <bool CH, int KK, int U, bool FIRST, bool UH>
+__global__ void __launch_bounds__(256, U == 1 && UH ? 4 : 3) k_cheb_dbl_df(DfEll<CH> H, const int4* __restrict__ tab,
                                                         const float4* __restrict__ tm1, const float4* tm2,
                                                         float4* tout, double2* __restrict__ partial, int nblocks,
                                                         int m) {
@@ -408,7 +408,13 @@ __global__ void __launch_bounds__(256, 3) k_cheb_dbl_df(DfEll<CH> H, const int4*
   const size_t segb = (size_t)tb.x, sege = (size_t)tb.y;
   const size_t step = (size_t)tb.w * blockDim.x;
   DfDot a0, a1;
-  for (size_t e0 = segb + (size_t)tb.z * blockDim.x + threadIdx.x; e0 < sege; e0 += (size_t)U * step) {
+  // a row's class is asked for one iteration ahead (as the index array would be by U = 2
+  // elements in flight): the neighbours' addresses then depend on no load from memory
+  const size_t first_e = segb + (size_t)tb.z * blockDim.x + threadIdx.x;
+  int cl[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) cl[u] = first_e + u * step < sege ? row_class(H.cls, (int)(first_e + u * step)) : 0;
+  for (size_t e0 = first_e; e0 < sege; e0 += (size_t)U * step) {
     int idx[U][KK];
     HT hv[U][KK];
     float2 dg[U];
@@ -420,24 +426,25 @@ __global__ void __launch_bounds__(256, 3) k_cheb_dbl_df(DfEll<CH> H, const int4*
       ok[u] = e < sege;
       const size_t ee = ok[u] ? e : e0;
       const int i = (int)ee;
+      row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, ok[u] ? cl[u] : cl[0], idx[u]);
+      if (!UH)
 #pragma unroll
-      for (int k = 0; k < KK; ++k) {
-        const size_t s = (size_t)k * H.n + i;
-        idx[u][k] = __ldg(H.idx + s);
-        hv[u][k] = __ldg(H.hop + s);
-      }
+        for (int k = 0; k < KK; ++k) hv[u][k] = __ldg(H.hop + (size_t)k * H.n + i);
       dg[u] = __ldg(H.diag + i);
       own[u] = __ldg(tm1 + ee);
       t2[u] = FIRST ? make_float4(0.f, 0.f, 0.f, 0.f) : tm2[ee];
     }
     float4 nb[U][KK];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+    for (int u = 0; u < U; ++u) {
 #pragma unroll
       for (int k = 0; k < KK; ++k) nb[u][k] = __ldg(tm1 + idx[u][k]);
+      const size_t en = e0 + (size_t)(U + u) * step;
+      cl[u] = en < sege ? row_class(H.cls, (int)en) : 0;
+    }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float4 a = df_step<CH, KK, FIRST>(hv[u], dg[u], own[u], nb[u], t2[u]);
+      const float4 a = df_step_any<CH, KK, FIRST, UH>(H, hv[u], dg[u], own[u], nb[u], t2[u]);
       if (ok[u]) {
         const size_t e = e0 + u * step;
         tout[e] = a;

@@ -58,15 +58,21 @@ struct DfEvo {
 
 __device__ __forceinline__ double2 df_to_d2(float4 f) { return make_double2(df_value(f.x, f.z), df_value(f.y, f.w)); }
 
-template <bool CH, int KK, bool UH = false>
+// CLS: neighbours by the row's class.  The commutator orders, which stream six vectors a
+// site, lose more by its second dependent load (31 -> 34 us at N = 1M, K = 4) than the
+// index array costs them.
+template <bool CH, int KK, bool UH, bool CLS>
 __device__ __forceinline__ void df_row_ops(const DfEll<CH>& H, int i, int (&idx)[KK],
                                            typename DfHop<CH>::T (&hv)[KK], float2& dg) {
+  if (CLS) {
+    row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, row_class(H.cls, i), idx);
+  } else {
 #pragma unroll
-  for (int k = 0; k < KK; ++k) {
-    const size_t s = (size_t)k * H.n + i;
-    idx[k] = __ldg(H.idx + s);
-    if (!UH) hv[k] = __ldg(H.hop + s);
+    for (int k = 0; k < KK; ++k) idx[k] = __ldg(H.idx + (size_t)k * H.n + i);
   }
+  if (!UH)
+#pragma unroll
+    for (int k = 0; k < KK; ++k) hv[k] = __ldg(H.hop + (size_t)k * H.n + i);
   dg = __ldg(H.diag + i);
 }
 
@@ -113,7 +119,7 @@ __global__ void __launch_bounds__(256) k_evolve_df(DfEll<CH> H, const int4* __re
     int idx[KK];
     HT hv[KK];
     float2 dg;
-    df_row_ops<CH, KK, UH>(H, i, idx, hv, dg);
+    df_row_ops<CH, KK, UH, true>(H, i, idx, hv, dg);
 #pragma unroll
     for (int q = 0; q < NSET; ++q) {
       const float4 own = __ldg(A.t1[q] + e);
@@ -188,7 +194,7 @@ __global__ void __launch_bounds__(256) k_msd_evolve_df(DfEll<CH> H, const int4* 
     int idx[KK];
     HT hv[KK];
     float2 dg;
-    df_row_ops<CH, KK, UH>(H, i, idx, hv, dg);
+    df_row_ops<CH, KK, UH, false>(H, i, idx, hv, dg);
     const float4 u_own = __ldg(B.u1 + e), z_own = __ldg(B.z1 + e);
     float4 un[KK];
 #pragma unroll
@@ -329,12 +335,9 @@ struct EvoRow {
   typename E::HT hv[KK];
   typename E::S dg;
   __device__ __forceinline__ EvoRow(const E& H, int i) {
+    row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, row_class(H.cls, i), idx);
 #pragma unroll
-    for (int k = 0; k < KK; ++k) {
-      const size_t s = (size_t)k * H.n + i;
-      idx[k] = __ldg(H.idx + s);
-      hv[k] = __ldg(H.hop2 + s);
-    }
+    for (int k = 0; k < KK; ++k) hv[k] = hop_of(H, k, i);
     dg = __ldg(H.diag2 + i);
   }
 };

@@ -615,11 +615,16 @@ void gqt::ensure_df_x(gqt_ham* h, cudaStream_t st) {
 
 // elements in flight per thread in the l = r rows (two, within 85 registers, up
 // to four neighbour slots)
-constexpr int df_u(int KK) { return KK <= 4 ? 2 : 1; }
+constexpr int df_u(int KK, bool uh = false) { return KK <= 4 && !uh ? 2 : 1; }
 
 template <bool CH, int KK>
-static int df_occupancy_k(bool pair, int threads) {
-  const void* f = pair ? (const void*)k_cheb_pair_df<CH, KK, false> : (const void*)k_cheb_dbl_df<CH, KK, df_u(KK), false>;
+static int df_occupancy_k(bool pair, bool uh, int threads) {
+  const void* f = pair ? (const void*)k_cheb_pair_df<CH, KK, false, false>
+                       : (const void*)k_cheb_dbl_df<CH, KK, df_u(KK), false, false>;
+  if constexpr (!CH)
+    if (uh)
+      f = pair ? (const void*)k_cheb_pair_df<CH, KK, false, true>
+               : (const void*)k_cheb_dbl_df<CH, KK, df_u(KK, true), false, true>;
   int n = 0;
   const size_t smem = (size_t)3 * (threads / 32) * sizeof(double2);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, smem) != cudaSuccess) {
@@ -630,12 +635,12 @@ static int df_occupancy_k(bool pair, int threads) {
 }
 
 template <bool CH>
-static int df_occupancy(int K, bool pair, int threads) {
+static int df_occupancy(int K, bool pair, bool uh, int threads) {
   switch (K) {
-    case 2: return df_occupancy_k<CH, 2>(pair, threads);
-    case 3: return df_occupancy_k<CH, 3>(pair, threads);
-    case 4: return df_occupancy_k<CH, 4>(pair, threads);
-    default: return df_occupancy_k<CH, 6>(pair, threads);
+    case 2: return df_occupancy_k<CH, 2>(pair, uh, threads);
+    case 3: return df_occupancy_k<CH, 3>(pair, uh, threads);
+    case 4: return df_occupancy_k<CH, 4>(pair, uh, threads);
+    default: return df_occupancy_k<CH, 6>(pair, uh, threads);
   }
 }
 
@@ -738,6 +743,16 @@ static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const
   const int4* tab = (const int4*)T.d_tab4.p;
   const int nb = T.nblocks;
   const size_t sm = smem_bytes(h, 1, 3);
+  const bool uni = !CH && h->hop_uniform;  // one common hopping: no hop array is read
+  auto with_uh = [&](auto&& f) {
+    if constexpr (!CH) {
+      if (uni) {
+        f(std::true_type());
+        return;
+      }
+    }
+    f(std::false_type());
+  };
   int cur = 0, prv = 1;
   for (int m = 1; m <= std::max(steps, 1);) {
     size_t pe = prof_begin(s2);
@@ -746,12 +761,17 @@ static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const
         void* in[2] = {const_cast<void*>(l), const_cast<void*>(r)};
         float4* t0[2] = {A[1], B[1]};
         launch_split<2>(in, t0, (size_t)h->n, s2);
-        k_cheb_pair_df<CH, KK, true><<<nb, h->threads, sm, s2>>>(H, tab, A[1], B[1], nullptr, nullptr, A[0], B[0],
-                                                                 partial, nb, 1, 2 * steps);
+        with_uh([&](auto uh) {
+          k_cheb_pair_df<CH, KK, true, decltype(uh)::value><<<nb, h->threads, sm, s2>>>(
+              H, tab, A[1], B[1], nullptr, nullptr, A[0], B[0], partial, nb, 1, 2 * steps);
+        });
       } else {
         void* in[1] = {const_cast<void*>(r)};
         launch_split<1>(in, &B[1], (size_t)h->n, s2);
-        k_cheb_dbl_df<CH, KK, df_u(KK), true><<<nb, h->threads, sm, s2>>>(H, tab, B[1], nullptr, B[0], partial, nb, 1);
+        with_uh([&](auto uh) {
+          k_cheb_dbl_df<CH, KK, df_u(KK, decltype(uh)::value), true, decltype(uh)::value><<<nb, h->threads, sm, s2>>>(
+              H, tab, B[1], nullptr, B[0], partial, nb, 1);
+        });
       }
       check_launch(pair ? "k_cheb_pair_df(first)" : "k_cheb_dbl_df(first)");
       prof_end(pe, 0, s2);
@@ -795,12 +815,15 @@ static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const
         continue;
       }
     }
-    if (pair)
-      k_cheb_pair_df<CH, KK, false><<<nb, h->threads, sm, s2>>>(H, tab, A[cur], B[cur], A[prv], B[prv], A[prv],
-                                                                B[prv], partial, nb, m, 2 * steps);
-    else
-      k_cheb_dbl_df<CH, KK, df_u(KK), false><<<nb, h->threads, sm, s2>>>(H, tab, B[cur], B[prv], B[prv], partial, nb,
-                                                                         m);
+    with_uh([&](auto uh) {
+      constexpr bool UH = decltype(uh)::value;
+      if (pair)
+        k_cheb_pair_df<CH, KK, false, UH><<<nb, h->threads, sm, s2>>>(H, tab, A[cur], B[cur], A[prv], B[prv], A[prv],
+                                                                      B[prv], partial, nb, m, 2 * steps);
+      else
+        k_cheb_dbl_df<CH, KK, df_u(KK, UH), false, UH><<<nb, h->threads, sm, s2>>>(H, tab, B[cur], B[prv], B[prv], partial,
+                                                                               nb, m);
+    });
     check_launch(pair ? "k_cheb_pair_df" : "k_cheb_dbl_df");
     prof_end(pe, pair ? 6 : 5, s2);
     std::swap(cur, prv);
@@ -815,8 +838,8 @@ static void launch_moments_df(gqt_ham* h, const void* l, const void* r, int M, v
   ensure_df(h, st);
   const bool pair = kind == 1;
   const int occ = h->blocks_per_sm > 0 ? h->blocks_per_sm
-                                       : (h->hop_real ? df_occupancy<false>(h->K, pair, h->threads)
-                                                      : df_occupancy<true>(h->K, pair, h->threads));
+                                       : (h->hop_real ? df_occupancy<false>(h->K, pair, h->hop_uniform, h->threads)
+                                                      : df_occupancy<true>(h->K, pair, false, h->threads));
   const BlockTable& T = h->table(1, occ);
   const int nb = T.nblocks;
   const size_t vb = h->vec_bytes(1);

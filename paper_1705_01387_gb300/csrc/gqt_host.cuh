@@ -164,6 +164,10 @@ inline Ell<FP64, CH> ell_of(const gqt_ham* h) {
   e.hop2 = (const typename Ell<FP64, CH>::HT*)h->d_hop.p;
   e.diag2 = (const typename Ell<FP64, CH>::S*)h->d_diag.p;
   e.dx = (const typename Ell<FP64, CH>::S*)h->d_dx.p;
+  e.cls = h->has_cls ? (const uint16_t*)h->d_cls.p : nullptr;
+  e.cls_off = (const int*)h->d_cls_off.p;
+  e.uni = !FP64 && h->hop_uniform32;
+  e.h0 = (typename Ell<FP64, CH>::S)h->hop0f;
   e.row_shift = (h->use_sweep_order && h->row_shift > 0) ? h->row_shift : 0;
   return e;
 }
@@ -209,6 +213,8 @@ inline DfEll<CH> df_ell_of(const gqt_ham* h) {
   e.idx = (const int*)h->d_idx.p;
   e.hop = (const typename DfHop<CH>::T*)h->d_hop_df.p;
   e.diag = (const float2*)h->d_diag_df.p;
+  e.cls = h->has_cls ? (const uint16_t*)h->d_cls.p : nullptr;
+  e.cls_off = (const int*)h->d_cls_off.p;
   e.xhop = (const typename DfHop<CH>::T*)h->d_xhop_df.p;
   if (h->hop_uniform) {
     const float a = (float)h->hop0;

@@ -103,6 +103,15 @@ struct gqt_ham {
   int nseg = 1;
   std::vector<int64_t> seg;  // nseg + 1 offsets
   gqt::DevBuf d_idx, d_hop, d_diag, d_dx, d_site_seg, d_flag;
+  // Row classes: rows with the same neighbour offsets idx - i share a class, so that the
+  // wavefront kernels read two bytes per row instead of K indices (on the built-in
+  // lattices the rows fall into a few classes, one or two of them away from the edges).
+  // Absent for models with more than ROW_CLASSES distinct rows or 8 slots.
+  gqt::DevBuf d_cls, d_cls_off;  // [n] uint16, [classes][8] offsets
+  bool has_cls = false;
+  // FP32 handles: every ELL slot holds this one real 2H~ value
+  bool hop_uniform32 = false;
+  float hop0f = 0.f;
   gqt::DevBuf d_dy;     // FP64 slot-major y displacements (Hall moments), when the model defines them
   int row_shift = 0;       // blocked sweep order (built-in cubic lattices): log2 of the side, 0 = off
   bool use_sweep_order = true;

@@ -63,6 +63,12 @@ struct Ell {
   const HT* __restrict__ hop2;
   const S* __restrict__ diag2;
   const S* __restrict__ dx;
+  // row classes (null: every row reads its indices), see row_neighbours
+  const uint16_t* __restrict__ cls;
+  const int* __restrict__ cls_off;
+  // every slot holds the real value h0 (FP32 storage): the hop array is not read
+  int uni;
+  S h0;
   // optional blocked sweep order of the multi-vector kernels for a simple-cubic
   // lattice of side L = 2^row_shift (0: sites in index order), see site_of
   int row_shift;
@@ -78,6 +84,44 @@ __device__ __forceinline__ int site_of(const E& H, int w) {
   const int m = (1 << lx) - 1;
   const int r = w >> lx, t = r >> 5;
   return (w & m) | ((((t >> lx) << 5) | (r & 31)) << lx) | ((t & m) << (2 * lx));
+}
+
+// Class of row i (0 where the handle has none).
+__device__ __forceinline__ int row_class(const uint16_t* __restrict__ cls, int i) { return cls ? __ldg(cls + i) : 0; }
+
+// Neighbours of row i of class c.  The class names the row's K offsets idx - i in a table
+// that stays in L1; a handle without classes reads the index array.  At K = 6 that is 2
+// instead of 24 bytes a row: FP32 l = r orders of 1.9M sites, with one common hopping not
+// read either, 23.2 -> 14.6 us (L2 bound: 29 instead of 76 bytes a site); paired-FP32
+// orders of 1M sites, K = 4, 15.0 -> 13.0.  The multi-vector kernels that prefetch the next
+// site's row keep the index array: behind a class the prefetched neighbours come one
+// load later (318 -> 367 us an order at 67M elements).
+template <int KK>
+__device__ __forceinline__ void row_neighbours(const int* __restrict__ idx, const uint16_t* __restrict__ cls,
+                                               const int* __restrict__ cls_off, int n, int i, int c, int (&j)[KK]) {
+  if (cls) {
+    const int4 a = __ldg(reinterpret_cast<const int4*>(cls_off) + 2 * c);
+    j[0] = i + a.x;
+    j[1] = i + a.y;
+    if (KK > 2) j[KK > 2 ? 2 : 0] = i + a.z;
+    if (KK > 3) j[KK > 3 ? 3 : 0] = i + a.w;
+    if (KK > 4) {
+      const int2 b = __ldg(reinterpret_cast<const int2*>(cls_off) + 4 * c + 2);
+      j[KK > 4 ? 4 : 0] = i + b.x;
+      j[KK > 5 ? 5 : 0] = i + b.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < KK; ++k) j[k] = __ldg(idx + (size_t)k * n + i);
+  }
+}
+
+// 2H~ of slot k of row i.
+template <bool FP64, bool CH>
+__device__ __forceinline__ typename Ell<FP64, CH>::HT hop_of(const Ell<FP64, CH>& H, int k, int i) {
+  if constexpr (!FP64 && !CH)
+    if (H.uni) return H.h0;
+  return __ldg(H.hop2 + (size_t)k * H.n + i);
 }
 
 // ---------------------------------------------------------------- arithmetic
@@ -1010,13 +1054,9 @@ __device__ __forceinline__ void cheb_wave_body(const Ell<FP64, CH>& H, int4 tb, 
           acc[u] = cneg(tm2[ee]);
         }
       }
+      row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, row_class(H.cls, i), idx[u]);
 #pragma unroll
-      for (int k = 0; k < KMAX; ++k)
-        if (k < K) {
-          const size_t s = (size_t)k * H.n + i;
-          idx[u][k] = __ldg(H.idx + s);
-          hv[u][k] = __ldg(H.hop2 + s);
-        }
+      for (int k = 0; k < KMAX; ++k) hv[u][k] = hop_of(H, k, i);
     }
     V nbv[U][KMAX];
 #pragma unroll
@@ -1133,12 +1173,9 @@ __device__ __forceinline__ void cheb_pair_body(const Ell<FP64, CH>& H, int4 tb, 
     const int i = (int)(e >> rs);
     int idx[KK];
     HT hv[KK];
+    row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, row_class(H.cls, i), idx);
 #pragma unroll
-    for (int k = 0; k < KK; ++k) {
-      const size_t s = (size_t)k * H.n + i;
-      idx[k] = __ldg(H.idx + s);
-      hv[k] = __ldg(H.hop2 + s);
-    }
+    for (int k = 0; k < KK; ++k) hv[k] = hop_of(H, k, i);
     const S dg = __ldg(H.diag2 + i);
     const V ao = __ldg(am1 + e), bo = __ldg(bm1 + e);
     V a, b;
@@ -1380,12 +1417,9 @@ __device__ __forceinline__ void cheb_wave_vpt(const Ell<FP64, CH>& H, int4 tb, i
     const size_t base = (size_t)i * R + r0;
     V own[VPT], acc[VPT], lv[VPT];
     if constexpr (!PF) {
+      row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, row_class(H.cls, i), idx);
 #pragma unroll
-      for (int k = 0; k < KK; ++k) {
-        const size_t s = (size_t)k * H.n + i;
-        idx[k] = __ldg(H.idx + s);
-        hv[k] = __ldg(H.hop2 + s);
-      }
+      for (int k = 0; k < KK; ++k) hv[k] = hop_of(H, k, i);
       dg = __ldg(H.diag2 + i);
     }
     ldg_v<VPT>(own, tm1 + base, G);
@@ -1558,12 +1592,9 @@ __device__ __forceinline__ void cheb_pair_vpt(const Ell<FP64, CH>& H, int4 tb, i
     const int r0 = lane_offset<FP64>(lg);
     const size_t base = (size_t)i * R + r0;
     if constexpr (!PF) {
+      row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, row_class(H.cls, i), idx);
 #pragma unroll
-      for (int k = 0; k < KK; ++k) {
-        const size_t s = (size_t)k * H.n + i;
-        idx[k] = __ldg(H.idx + s);
-        hv[k] = __ldg(H.hop2 + s);
-      }
+      for (int k = 0; k < KK; ++k) hv[k] = hop_of(H, k, i);
       dg = __ldg(H.diag2 + i);
     }
     V ao[VPT], bo[VPT], a[VPT], b[VPT];

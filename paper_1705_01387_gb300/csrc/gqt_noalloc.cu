@@ -124,6 +124,10 @@ Ell<FP64, CH> ell_view(const gqt_ham* h) {
   e.hop2 = (const typename Ell<FP64, CH>::HT*)h->d_hop.p;
   e.diag2 = (const typename Ell<FP64, CH>::S*)h->d_diag.p;
   e.dx = (const typename Ell<FP64, CH>::S*)h->d_dx.p;
+  e.cls = nullptr;
+  e.cls_off = nullptr;
+  e.uni = 0;
+  e.h0 = 0;
   e.row_shift = 0;
   return e;
 }
