@@ -329,8 +329,8 @@ __device__ __forceinline__ float4 df_step_any(const DfEll<CH>& H, const typename
 // (k_split_vec).  R = 1, wavefront CTA order, one element per thread.
 template <bool CH, int KK, bool FIRST, bool UH>
 __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4* __restrict__ tab,
-                                                         const float4* __restrict__ am1,
-                                                         const float4* __restrict__ bm1, const float4* am2,
+                                                         const float4* am1,
+                                                         const float4* bm1, const float4* am2,
                                                          const float4* bm2, float4* aout, float4* bout,
                                                          double2* __restrict__ partial, int nblocks, int m,
                                                          int slot_norm) {
@@ -338,6 +338,7 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
   double2* smem = dyn_smem();
   const int b = blockIdx.x;
   const int4 tb = tab[b];
+  chain_wait();
   const size_t segb = (size_t)tb.x, sege = (size_t)tb.y;
   const size_t step = (size_t)tb.w * blockDim.x;
   DfDot d0, d1, nl, nr;
@@ -350,7 +351,7 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
 #pragma unroll
       for (int k = 0; k < KK; ++k) hv[k] = __ldg(H.hop + (size_t)k * H.n + i);
     const float2 dg = __ldg(H.diag + i);
-    const float4 ao = __ldg(am1 + e), bo = __ldg(bm1 + e);
+    const float4 ao = am1[e], bo = bm1[e];
     float4 a2 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = a2;
     if (!FIRST) {
       a2 = am2[e];
@@ -359,8 +360,8 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
     float4 na[KK], nbv[KK];
 #pragma unroll
     for (int k = 0; k < KK; ++k) {
-      na[k] = __ldg(am1 + idx[k]);
-      nbv[k] = __ldg(bm1 + idx[k]);
+      na[k] = am1[idx[k]];
+      nbv[k] = bm1[idx[k]];
     }
     const float4 a = df_step_any<CH, KK, FIRST, UH>(H, hv, dg, ao, na, a2);
     const float4 bb = df_step_any<CH, KK, FIRST, UH>(H, hv, dg, bo, nbv, b2);
@@ -398,13 +399,14 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_df(DfEll<CH> H, const int4
 // per thread.
 template <bool CH, int KK, int U, bool FIRST, bool UH>
 __global__ void __launch_bounds__(256, U == 1 && UH ? 4 : 3) k_cheb_dbl_df(DfEll<CH> H, const int4* __restrict__ tab,
-                                                        const float4* __restrict__ tm1, const float4* tm2,
+                                                        const float4* tm1, const float4* tm2,
                                                         float4* tout, double2* __restrict__ partial, int nblocks,
                                                         int m) {
   using HT = typename DfHop<CH>::T;
   double2* smem = dyn_smem();
   const int b = blockIdx.x;
   const int4 tb = tab[b];
+  chain_wait();
   const size_t segb = (size_t)tb.x, sege = (size_t)tb.y;
   const size_t step = (size_t)tb.w * blockDim.x;
   DfDot a0, a1;
@@ -431,14 +433,14 @@ __global__ void __launch_bounds__(256, U == 1 && UH ? 4 : 3) k_cheb_dbl_df(DfEll
 #pragma unroll
         for (int k = 0; k < KK; ++k) hv[u][k] = __ldg(H.hop + (size_t)k * H.n + i);
       dg[u] = __ldg(H.diag + i);
-      own[u] = __ldg(tm1 + ee);
+      own[u] = tm1[ee];
       t2[u] = FIRST ? make_float4(0.f, 0.f, 0.f, 0.f) : tm2[ee];
     }
     float4 nb[U][KK];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
 #pragma unroll
-      for (int k = 0; k < KK; ++k) nb[u][k] = __ldg(tm1 + idx[u][k]);
+      for (int k = 0; k < KK; ++k) nb[u][k] = tm1[idx[u][k]];
       const size_t en = e0 + (size_t)(U + u) * step;
       cl[u] = en < sege ? row_class(H.cls, (int)en) : 0;
     }

@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(256) k_evolve_df(DfEll<CH> H, const int4* __re
   using HT = typename DfHop<CH>::T;
   const int4 tb = tab[blockIdx.x];
   const size_t sege = (size_t)tb.y, step = (size_t)tb.w * blockDim.x;
+  chain_wait();
   DfDot nrm[NSET];
   for (size_t e = (size_t)tb.x + (size_t)tb.z * blockDim.x + threadIdx.x; e < sege; e += step) {
     const int i = (int)e;
@@ -122,10 +123,10 @@ __global__ void __launch_bounds__(256) k_evolve_df(DfEll<CH> H, const int4* __re
     df_row_ops<CH, KK, UH, true>(H, i, idx, hv, dg);
 #pragma unroll
     for (int q = 0; q < NSET; ++q) {
-      const float4 own = __ldg(A.t1[q] + e);
+      const float4 own = A.t1[q][e];
       float4 nb[KK];
 #pragma unroll
-      for (int k = 0; k < KK; ++k) nb[k] = __ldg(A.t1[q] + idx[k]);
+      for (int k = 0; k < KK; ++k) nb[k] = A.t1[q][idx[k]];
       const float4 t2 = PH == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : A.t2[q][e];
       const float4 y = df_step_any<CH, KK, PH == 0, UH>(H, hv, dg, own, nb, t2);
       if (PH != 2) A.out[q][e] = y;
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(256) k_msd_evolve_df(DfEll<CH> H, const int4* 
   using HT = typename DfHop<CH>::T;
   const int4 tb = tab[blockIdx.x];
   const size_t sege = (size_t)tb.y, step = (size_t)tb.w * blockDim.x;
+  chain_wait();
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   DfDot n0, n1;
   for (size_t e = (size_t)tb.x + (size_t)tb.z * blockDim.x + threadIdx.x; e < sege; e += step) {
@@ -195,16 +197,16 @@ __global__ void __launch_bounds__(256) k_msd_evolve_df(DfEll<CH> H, const int4* 
     HT hv[KK];
     float2 dg;
     df_row_ops<CH, KK, UH, false>(H, i, idx, hv, dg);
-    const float4 u_own = __ldg(B.u1 + e), z_own = __ldg(B.z1 + e);
+    const float4 u_own = B.u1[e], z_own = B.z1[e];
     float4 un[KK];
 #pragma unroll
-    for (int k = 0; k < KK; ++k) un[k] = __ldg(B.u1 + idx[k]);
+    for (int k = 0; k < KK; ++k) un[k] = B.u1[idx[k]];
     const float4 u2 = PH == 0 ? zero : B.u2[e], z2 = PH == 0 ? zero : B.z2[e];
     const float4 uo = df_step_any<CH, KK, PH == 0, UH>(H, hv, dg, u_own, un, u2);
     DfC a = df_start<PH == 0>(dg, z_own, z2);
     float4 zn[KK];
 #pragma unroll
-    for (int k = 0; k < KK; ++k) zn[k] = __ldg(B.z1 + idx[k]);
+    for (int k = 0; k < KK; ++k) zn[k] = B.z1[idx[k]];
     if constexpr (UH) {
       dfc_mac_sum<KK>(a, H.h0, zn);
     } else {
@@ -693,10 +695,10 @@ void launch_evolve_df(gqt_ham* h, void* const* psi, const std::vector<double2>& 
           }
           size_t pe = prof_begin(s2);
           if (m == Np - 1)
-            k_evolve_df<CH, KK, NSET, 2, UH><<<nb, h->threads, smem, s2>>>(H, tab, A, terms_of<float2>(c, m), partial,
+            launch_chain(true, k_evolve_df<CH, KK, NSET, 2, UH>, nb, h->threads, smem, s2, H, tab, A, terms_of<float2>(c, m), partial,
                                                                            nb, NSET);
           else
-            k_evolve_df<CH, KK, NSET, 1, UH><<<nb, h->threads, smem, s2>>>(H, tab, A, terms_of<float2>(c, m), partial,
+            launch_chain(true, k_evolve_df<CH, KK, NSET, 1, UH>, nb, h->threads, smem, s2, H, tab, A, terms_of<float2>(c, m), partial,
                                                                            nb, NSET);
           check_launch("k_evolve_df");
           prof_end(pe, 1 + NSET, s2);
@@ -773,10 +775,10 @@ void launch_msd_df(gqt_ham* h, void* p, void* px, const std::vector<double2>& c,
           B.z2 = B.zo;
           size_t pe = prof_begin(s2);
           if (m == Np - 1)
-            k_msd_evolve_df<CH, KK, 2, UH><<<nb, h->threads, smem, s2>>>(H, tab, B, terms_of<float2>(c, m), partial,
+            launch_chain(true, k_msd_evolve_df<CH, KK, 2, UH>, nb, h->threads, smem, s2, H, tab, B, terms_of<float2>(c, m), partial,
                                                                          nb, 2);
           else
-            k_msd_evolve_df<CH, KK, 1, UH><<<nb, h->threads, smem, s2>>>(H, tab, B, terms_of<float2>(c, m), partial,
+            launch_chain(true, k_msd_evolve_df<CH, KK, 1, UH>, nb, h->threads, smem, s2, H, tab, B, terms_of<float2>(c, m), partial,
                                                                          nb, 2);
           check_launch("k_msd_evolve_df");
           prof_end(pe, 4, s2);

@@ -33,6 +33,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "gqt_chain.cuh"
 #include "gqt_internal.h"
 #include "gqt_slices.h"
 
@@ -173,16 +174,17 @@ __global__ void k_kb_vhop(HallEll<F64, CH> H, const D* __restrict__ d, typename 
 template <bool F64, bool CH>
 __global__ void __launch_bounds__(256) k_kb_step(HallEll<F64, CH> H,
                                                  const typename HallEll<F64, CH>::HT* __restrict__ vh, int R,
-                                                 size_t total, const typename HallEll<F64, CH>::V* __restrict__ pk,
-                                                 const typename HallEll<F64, CH>::V* __restrict__ pkm1,
-                                                 typename HallEll<F64, CH>::V* __restrict__ pout,
-                                                 const typename HallEll<F64, CH>::V* __restrict__ qk,
-                                                 const typename HallEll<F64, CH>::V* __restrict__ qkm1,
-                                                 typename HallEll<F64, CH>::V* __restrict__ qout,
-                                                 typename HallEll<F64, CH>::V* __restrict__ bout, int first, int last,
+                                                 size_t total, const typename HallEll<F64, CH>::V* pk,
+                                                 const typename HallEll<F64, CH>::V* pkm1,
+                                                 typename HallEll<F64, CH>::V* pout,
+                                                 const typename HallEll<F64, CH>::V* qk,
+                                                 const typename HallEll<F64, CH>::V* qkm1,
+                                                 typename HallEll<F64, CH>::V* qout,
+                                                 typename HallEll<F64, CH>::V* bout, int first, int last,
                                                  TcPlanes ps, TcPlanes bs) {
   using V = typename HallEll<F64, CH>::V;
   using S = typename HallEll<F64, CH>::S;
+  chain_wait();
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const size_t i = e / R;
     const int r = (int)(e - i * R);
@@ -743,7 +745,7 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
       const V* qk = k == 0 ? r : qbuf(k);
       const V* qkm1 = k == 0 ? nullptr : (k == 1 ? r : qbuf(k - 1));
       const size_t pe = prof_begin(st);
-      k_kb_step<F64, CH><<<gs, ct, 0, st>>>(H, vh, R, total, Pst + (size_t)k * total,
+      launch_chain(k > 0, k_kb_step<F64, CH>, gs, ct, 0, st, H, vh, R, total, Pst + (size_t)k * total,
                                         k == 0 ? nullptr : Pst + (size_t)(k - 1) * total,
                                         last ? nullptr : Pst + (size_t)(k + 1) * total, qk, qkm1,
                                         last ? nullptr : qbuf(k + 1), Bst + (size_t)k * total, k == 0, last, none,
@@ -821,7 +823,7 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
     const V* qk = k == 0 ? r : qbuf(k);
     const V* qkm1 = k == 0 ? nullptr : (k == 1 ? r : qbuf(k - 1));
     const size_t pe = prof_begin(st);
-    k_kb_step<F64, CH><<<gs, ct, 0, st>>>(H, vh, R, total, pbuf(k), k == 0 ? nullptr : pbuf(k - 1),
+    launch_chain(k > 0, k_kb_step<F64, CH>, gs, ct, 0, st, H, vh, R, total, pbuf(k), k == 0 ? nullptr : pbuf(k - 1),
                                       last ? nullptr : pbuf(k + 1), qk, qkm1, last ? nullptr : qbuf(k + 1), nullptr,
                                       k == 0, last, last ? none : planes(0, k + 1), planes(4, k));
     check_launch("k_kb_step");

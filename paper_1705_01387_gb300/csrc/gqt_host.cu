@@ -393,10 +393,10 @@ static bool launch_wave_re(gqt_ham* h, const Ell<FP64, CH>& H, const BlockTable&
     k_cheb_re_wv<FP64, CH, 2, KK><<<T.nblocks, h->threads, sm, st>>>(H, tab, R, rs - 1, tm1, tm2, tout, l,       \
                                                                      partial, T.nblocks, slot0, slot_norm, first); \
   else if (h->variant == 1)                                                                                      \
-    k_cheb_re_w<FP64, CH, 1, KK><<<T.nblocks, h->threads, sm, st>>>(H, tab, R, rs, tm1, tm2, tout, l, partial, \
+    launch_chain(!first, k_cheb_re_w<FP64, CH, 1, KK>, T.nblocks, h->threads, sm, st, H, tab, R, rs, tm1, tm2, tout, l, partial, \
                                                                     T.nblocks, slot0, slot_norm, first);       \
   else                                                                                                           \
-    k_cheb_re_w<FP64, CH, 2, KK><<<T.nblocks, h->threads, sm, st>>>(H, tab, R, rs, tm1, tm2, tout, l, partial, \
+    launch_chain(!first, k_cheb_re_w<FP64, CH, 2, KK>, T.nblocks, h->threads, sm, st, H, tab, R, rs, tm1, tm2, tout, l, partial, \
                                                                     T.nblocks, slot0, slot_norm, first);       \
   return true;
   switch (H.K) {
@@ -432,10 +432,10 @@ static bool launch_wave_dbl(gqt_ham* h, const Ell<FP64, CH>& H, const BlockTable
     k_cheb_dbl_wv<FP64, CH, 2, KK><<<T.nblocks, h->threads, sm, st>>>(H, tab, R, rs - 1, tm1, tm2, tout, partial, \
                                                                       T.nblocks, m);                              \
   else if (h->variant == 1)                                                                                        \
-    k_cheb_dbl_w<FP64, CH, 1, KK><<<T.nblocks, h->threads, sm, st>>>(H, tab, R, rs, tm1, tm2, tout, partial,     \
+    launch_chain(m > 1, k_cheb_dbl_w<FP64, CH, 1, KK>, T.nblocks, h->threads, sm, st, H, tab, R, rs, tm1, tm2, tout, partial,     \
                                                                      T.nblocks, m);                               \
   else                                                                                                             \
-    k_cheb_dbl_w<FP64, CH, 2, KK><<<T.nblocks, h->threads, sm, st>>>(H, tab, R, rs, tm1, tm2, tout, partial,     \
+    launch_chain(m > 1, k_cheb_dbl_w<FP64, CH, 2, KK>, T.nblocks, h->threads, sm, st, H, tab, R, rs, tm1, tm2, tout, partial,     \
                                                                      T.nblocks, m);                               \
   return true;
   switch (H.K) {
@@ -553,7 +553,7 @@ static void launch_wave_pair(gqt_ham* h, const Ell<FP64, CH>& H, const BlockTabl
                                                                        aout, bout, partial, T.nblocks, m,        \
                                                                        slot_norm);                               \
   else                                                                                                           \
-    k_cheb_pair_w<FP64, CH, KK><<<T.nblocks, h->threads, sm, st>>>(H, tab, R, rs, am1, bm1, am2, bm2, aout, bout, \
+    launch_chain(m > 1, k_cheb_pair_w<FP64, CH, KK>, T.nblocks, h->threads, sm, st, H, tab, R, rs, am1, bm1, am2, bm2, aout, bout, \
                                                                    partial, T.nblocks, m, slot_norm);            \
   break;
   switch (H.K) {
@@ -818,10 +818,10 @@ static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const
     with_uh([&](auto uh) {
       constexpr bool UH = decltype(uh)::value;
       if (pair)
-        k_cheb_pair_df<CH, KK, false, UH><<<nb, h->threads, sm, s2>>>(H, tab, A[cur], B[cur], A[prv], B[prv], A[prv],
+        launch_chain(true, k_cheb_pair_df<CH, KK, false, UH>, nb, h->threads, sm, s2, H, tab, A[cur], B[cur], A[prv], B[prv], A[prv],
                                                                       B[prv], partial, nb, m, 2 * steps);
       else
-        k_cheb_dbl_df<CH, KK, df_u(KK, UH), false, UH><<<nb, h->threads, sm, s2>>>(H, tab, B[cur], B[prv], B[prv], partial,
+        launch_chain(true, k_cheb_dbl_df<CH, KK, df_u(KK, UH), false, UH>, nb, h->threads, sm, s2, H, tab, B[cur], B[prv], B[prv], partial,
                                                                                nb, m);
     });
     check_launch(pair ? "k_cheb_pair_df" : "k_cheb_dbl_df");

@@ -25,6 +25,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 #include <stdint.h>
+
+#include "gqt_chain.cuh"
 #endif
 
 namespace gqt {
@@ -1011,9 +1013,9 @@ namespace gqt {
 
 template <bool FP64, bool CH, int U, bool DBL, int KK, bool first>
 __device__ __forceinline__ void cheb_wave_body(const Ell<FP64, CH>& H, int4 tb, int R, int rs,
-                                               const typename Prec<FP64>::V* __restrict__ tm1,
+                                               const typename Prec<FP64>::V* tm1,
                                                const typename Prec<FP64>::V* tm2, typename Prec<FP64>::V* tout,
-                                               const typename Prec<FP64>::V* __restrict__ l,
+                                               const typename Prec<FP64>::V* l,
                                                DotAcc<typename Prec<FP64>::V>& d0, DotAcc<typename Prec<FP64>::V>& d1,
                                                DotAcc<typename Prec<FP64>::V>& nl, DotAcc<typename Prec<FP64>::V>& nr) {
   using V = typename Prec<FP64>::V;
@@ -1036,7 +1038,7 @@ __device__ __forceinline__ void cheb_wave_body(const Ell<FP64, CH>& H, int4 tb, 
       ok[u] = e < sege;
       const size_t ee = ok[u] ? e : e0;
       const int i = (int)(ee >> rs);
-      own[u] = __ldg(tm1 + ee);
+      own[u] = tm1[ee];
       dg[u] = __ldg(H.diag2 + i);
       if (DBL) {
         if (first) {
@@ -1046,7 +1048,7 @@ __device__ __forceinline__ void cheb_wave_body(const Ell<FP64, CH>& H, int4 tb, 
           acc[u] = cneg(tm2[ee]);
         }
       } else {
-        lv[u] = __ldg(l + ee);
+        lv[u] = l[ee];
         if (first) {
           acc[u].x = 0;
           acc[u].y = 0;
@@ -1063,7 +1065,7 @@ __device__ __forceinline__ void cheb_wave_body(const Ell<FP64, CH>& H, int4 tb, 
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int k = 0; k < KMAX; ++k)
-        if (k < K) nbv[u][k] = __ldg(tm1 + (((size_t)idx[u][k] << rs) + r));
+        if (k < K) nbv[u][k] = tm1[(((size_t)idx[u][k] << rs) + r)];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       V a = first ? cscale(own[u], dg[u]) : cmul_acc(acc[u], dg[u], own[u]);
@@ -1092,9 +1094,9 @@ __device__ __forceinline__ void cheb_wave_body(const Ell<FP64, CH>& H, int4 tb, 
 // Re <l|T_m|r> orders (VAC rows) in wavefront order; slots as k_cheb_re.
 template <bool FP64, bool CH, int U, int KK>
 __global__ void __launch_bounds__(256, (U == 1 ? 4 : 2)) k_cheb_re_w(Ell<FP64, CH> H, const int4* __restrict__ tab, int R, int rs,
-                                                   const typename Prec<FP64>::V* __restrict__ tm1,
+                                                   const typename Prec<FP64>::V* tm1,
                                                    const typename Prec<FP64>::V* tm2, typename Prec<FP64>::V* tout,
-                                                   const typename Prec<FP64>::V* __restrict__ l,
+                                                   const typename Prec<FP64>::V* l,
                                                    double2* __restrict__ partial, int nblocks, int slot0, int slot_norm,
                                                    int first) {
   using V = typename Prec<FP64>::V;
@@ -1103,6 +1105,7 @@ __global__ void __launch_bounds__(256, (U == 1 ? 4 : 2)) k_cheb_re_w(Ell<FP64, C
   DotAcc<V> d0, d1, nl, nr;
   // the first order (no T_{m-2}) is a separate instantiation of the loop body, so the
   // other orders fold -T_{m-2} into the first fused multiply-add
+  chain_wait();
   if (first)
     cheb_wave_body<FP64, CH, U, false, KK, true>(H, tab[b], R, rs, tm1, tm2, tout, l, d0, d1, nl, nr);
   else
@@ -1125,13 +1128,14 @@ __global__ void __launch_bounds__(256, (U == 1 ? 4 : 2)) k_cheb_re_w(Ell<FP64, C
 // l = r doubling orders (DOS, MSD rows) in wavefront order; slots as k_cheb_dbl.
 template <bool FP64, bool CH, int U, int KK>
 __global__ void __launch_bounds__(256, (U == 1 ? 4 : 2)) k_cheb_dbl_w(Ell<FP64, CH> H, const int4* __restrict__ tab, int R, int rs,
-                                                    const typename Prec<FP64>::V* __restrict__ tm1,
+                                                    const typename Prec<FP64>::V* tm1,
                                                     const typename Prec<FP64>::V* tm2, typename Prec<FP64>::V* tout,
                                                     double2* __restrict__ partial, int nblocks, int m) {
   using V = typename Prec<FP64>::V;
   double2* smem = dyn_smem();
   const int b = blockIdx.x;
   DotAcc<V> a0, a1, u0, u1;
+  chain_wait();
   if (m == 1)
     cheb_wave_body<FP64, CH, U, true, KK, true>(H, tab[b], R, rs, tm1, tm2, tout, nullptr, a0, a1, u0, u1);
   else
@@ -1157,8 +1161,8 @@ __global__ void __launch_bounds__(256, (U == 1 ? 4 : 2)) k_cheb_dbl_w(Ell<FP64, 
 // (slot_norm) for the moment bound.  Wavefront order, one element per thread.
 template <bool FP64, bool CH, int KK, bool first>
 __device__ __forceinline__ void cheb_pair_body(const Ell<FP64, CH>& H, int4 tb, int R, int rs,
-                                               const typename Prec<FP64>::V* __restrict__ am1,
-                                               const typename Prec<FP64>::V* __restrict__ bm1,
+                                               const typename Prec<FP64>::V* am1,
+                                               const typename Prec<FP64>::V* bm1,
                                                const typename Prec<FP64>::V* am2, const typename Prec<FP64>::V* bm2,
                                                typename Prec<FP64>::V* aout, typename Prec<FP64>::V* bout,
                                                DotAcc<typename Prec<FP64>::V>& d0, DotAcc<typename Prec<FP64>::V>& d1,
@@ -1177,7 +1181,7 @@ __device__ __forceinline__ void cheb_pair_body(const Ell<FP64, CH>& H, int4 tb, 
 #pragma unroll
     for (int k = 0; k < KK; ++k) hv[k] = hop_of(H, k, i);
     const S dg = __ldg(H.diag2 + i);
-    const V ao = __ldg(am1 + e), bo = __ldg(bm1 + e);
+    const V ao = am1[e], bo = bm1[e];
     V a, b;
     if (first) {
       a = cscale(ao, dg);
@@ -1190,8 +1194,8 @@ __device__ __forceinline__ void cheb_pair_body(const Ell<FP64, CH>& H, int4 tb, 
 #pragma unroll
     for (int k = 0; k < KK; ++k) {
       const size_t j = ((size_t)idx[k] << rs) + r;
-      na[k] = __ldg(am1 + j);
-      nb[k] = __ldg(bm1 + j);
+      na[k] = am1[j];
+      nb[k] = bm1[j];
     }
 #pragma unroll
     for (int k = 0; k < KK; ++k) {
@@ -1215,8 +1219,8 @@ __device__ __forceinline__ void cheb_pair_body(const Ell<FP64, CH>& H, int4 tb, 
 
 template <bool FP64, bool CH, int KK>
 __global__ void __launch_bounds__(256, 3) k_cheb_pair_w(Ell<FP64, CH> H, const int4* __restrict__ tab, int R, int rs,
-                                                       const typename Prec<FP64>::V* __restrict__ am1,
-                                                       const typename Prec<FP64>::V* __restrict__ bm1,
+                                                       const typename Prec<FP64>::V* am1,
+                                                       const typename Prec<FP64>::V* bm1,
                                                        const typename Prec<FP64>::V* am2,
                                                        const typename Prec<FP64>::V* bm2,
                                                        typename Prec<FP64>::V* aout, typename Prec<FP64>::V* bout,
@@ -1226,6 +1230,7 @@ __global__ void __launch_bounds__(256, 3) k_cheb_pair_w(Ell<FP64, CH> H, const i
   double2* smem = dyn_smem();
   const int b = blockIdx.x;
   DotAcc<V> d0, d1, nl, nr;
+  chain_wait();
   if (m == 1)
     cheb_pair_body<FP64, CH, KK, true>(H, tab[b], R, rs, am1, bm1, am2, bm2, aout, bout, d0, d1, nl, nr);
   else

@@ -20,6 +20,7 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include "gqt_chain.cuh"
 #include "gqt_internal.h"
 
 // The kernel templates are compiled into this translation unit under their own
@@ -29,6 +30,9 @@
 // needs and this file lacks is a compile error rather than a silent rebinding.
 #define GQT_KERNELS_NO_SYSTEM_INCLUDES 1
 namespace gqt_na {
+namespace gqt {
+using ::gqt::chain_wait;
+}  // namespace gqt
 #include "gqt_kernels.cuh"
 }
 #undef GQT_KERNELS_NO_SYSTEM_INCLUDES
