@@ -590,12 +590,15 @@ def run_ours(args):
     df = args.fp64_arith == 1
     sfx = "_df" if df else ""
     uniform = bool(ham.forms & g.GQT_FORM_UNIFORM_HOP)
+    # the single-order kernels read a row's class (2 bytes) instead of its indices and, in
+    # paired arithmetic with one common hopping, no hoppings
+    row = 0 if R > 1 else 2 - 3 * 4 - (3 * 8 if df and uniform else 0)
     fam = {1: ("k_cheb_re (VAC row: fused SpMV + three-term recurrence + Re <l|T_m|r>)",
-               bytes_per_orbital_cheb(3, True, ham.hop_real, R), "re", 1),
+               bytes_per_orbital_cheb(3, True, ham.hop_real, R) + row, "re", 1),
            5: (f"k_cheb_dbl{sfx} (MSD row: fused SpMV + recurrence + <u_n|u_n>, <u_n+1|u_n>)",
-               bytes_per_orbital_cheb(3, True, ham.hop_real, R) - 16 * R, "dbl", 1),
+               bytes_per_orbital_cheb(3, True, ham.hop_real, R) - 16 * R + row, "dbl", 1),
            6: (f"k_cheb_pair{sfx} (VAC row: two fused SpMV + recurrences, T_k l and T_k r, + Re <A_k|B_k>, "
-               "Re <A_k|B_k+1>)", bytes_per_orbital_pair(3, ham.hop_real, R), "pair", 1),
+               "Re <A_k|B_k+1>)", bytes_per_orbital_pair(3, ham.hop_real, R) + row, "pair", 1),
            10: ("k_cheb2_honey_df_pair (VAC row, temporally blocked: two steps of both recurrences per launch, "
                 "the second from the first's rows in shared memory" + (", one common hopping" if uniform else "") + ")",
                 bytes_per_orbital_tiled(3, ham.hop_real, True, uniform), "pair", 2),
@@ -639,7 +642,7 @@ def run_ours(args):
         if nsteps == 2:
             # the two single-step launches this one replaces would move these bytes
             eq = 2 * (bytes_per_orbital_pair(3, ham.hop_real, R) if fkind == "pair"
-                      else bytes_per_orbital_cheb(3, True, ham.hop_real, R) - 16 * R)
+                      else bytes_per_orbital_cheb(3, True, ham.hop_real, R) - 16 * R) + 2 * row
             roof["steps_per_launch"] = 2
             roof["single_step_equivalent"] = {"bytes_per_orbital": eq, "achieved": N * eq / avg_s / 1e9,
                                               "frac": N * eq / avg_s / 1e9 / hbm, "unit": "GB/s"}
