@@ -988,18 +988,6 @@ static const double* kb_integrand_dev(int M, const double* d_E, int NE, double e
   return F;
 }
 
-// Stream-ordered scratch of one call, given back on every way out.
-struct StreamBuf {
-  double* p = nullptr;
-  cudaStream_t st;
-  StreamBuf(size_t doubles, cudaStream_t s) : st(s) {
-    check_cuda(cudaMallocAsync((void**)&p, doubles * sizeof(double), st), "cudaMallocAsync");
-  }
-  ~StreamBuf() { cudaFreeAsync(p, st); }
-  StreamBuf(const StreamBuf&) = delete;
-  StreamBuf& operator=(const StreamBuf&) = delete;
-};
-
 static std::vector<double> check_energies(const double* d_E, int NE, double energy_scale, cudaStream_t st) {
   std::vector<double> hE(NE);
   check_cuda(cudaMemcpyAsync(hE.data(), d_E, NE * sizeof(double), cudaMemcpyDeviceToHost, st), "energies");
@@ -1020,9 +1008,10 @@ extern "C" gqt_status gqt_kubo_bastin(const double* d_lambda, int M, const doubl
       throw Error(GQT_EINVAL, "gqt_kubo_bastin: bad argument");
     cudaStream_t st = (cudaStream_t)stream;
     check_energies(d_E, NE, energy_scale, st);
-    StreamBuf buf(kb_scratch(M, NE), st);
-    kb_collapse(d_lambda, M, kernel, buf.p, st);
-    const double* F = kb_integrand_dev(M, d_E, NE, energy_scale, buf.p, st);
+    StreamScratch scratch(kb_scratch(M, NE) * sizeof(double), st);
+    double* buf = (double*)scratch.p;
+    kb_collapse(d_lambda, M, kernel, buf, st);
+    const double* F = kb_integrand_dev(M, d_E, NE, energy_scale, buf, st);
     k_kb_scan<<<1, 1024, 0, st>>>(F, d_E, NE, 1.0 / energy_scale, 2.0 / area, d_sigma);
     check_launch("k_kb_scan");
     check_cuda(cudaStreamSynchronize(st), "gqt_kubo_bastin");
@@ -1049,9 +1038,10 @@ extern "C" gqt_status gqt_kubo_bastin_fermi(const double* d_lambda, int M, const
       throw Error(GQT_EINVAL, "gqt_kubo_bastin_fermi: bad argument");
     cudaStream_t st = (cudaStream_t)stream;
     check_energies(d_E, NE, energy_scale, st);
-    StreamBuf buf(kb_scratch(M, NE), st);
-    kb_collapse(d_lambda, M, kernel, buf.p, st);
-    const double* F = kb_integrand_dev(M, d_E, NE, energy_scale, buf.p, st);
+    StreamScratch scratch(kb_scratch(M, NE) * sizeof(double), st);
+    double* buf = (double*)scratch.p;
+    kb_collapse(d_lambda, M, kernel, buf, st);
+    const double* F = kb_integrand_dev(M, d_E, NE, energy_scale, buf, st);
     k_kb_fermi<<<(Nmu + 127) / 128, 128, 0, st>>>(F, d_E, NE, 1.0 / energy_scale, d_mu, Nmu, kT, 2.0 / area, d_sigma);
     check_launch("k_kb_fermi");
     check_cuda(cudaStreamSynchronize(st), "gqt_kubo_bastin_fermi");

@@ -16,6 +16,7 @@
 #include <cstring>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <stdexcept>
 #include <string>
 #include <tuple>
@@ -61,6 +62,59 @@ void check_launch(const char* what) {
   if (e != cudaSuccess) throw Error(GQT_ECUDA, std::string("launch ") + what + ": " + cudaGetErrorString(e));
 }
 
+// The calls without a handle (reconstruction, sigma, Kubo-Bastin sums) take their scratch
+// from a memory pool of the library, one per device, which keeps up to SCRATCH_KEEP
+// between calls: the device's default pool gives everything back at each
+// synchronisation, and mapping it anew costs 0.1 ms a call.  The pool is stream-ordered
+// and shared by all threads; an allocation that fails for want of memory, here or in
+// DevBuf, empties it and tries again.
+constexpr size_t SCRATCH_KEEP = (size_t)128 << 20;
+constexpr int MAX_DEVICES = 64;
+static std::mutex g_pool_mu;
+static cudaMemPool_t g_pools[MAX_DEVICES] = {};
+
+static cudaMemPool_t scratch_pool() {
+  int dev = 0;
+  check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
+  if (dev >= MAX_DEVICES) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!g_pools[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    unsigned long long keep = SCRATCH_KEEP;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      if (pool) cudaMemPoolDestroy(pool);
+      return nullptr;
+    }
+    g_pools[dev] = pool;
+  }
+  return g_pools[dev];
+}
+
+// Gives back what the current device's pool holds unused.
+static void trim_scratch() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= MAX_DEVICES) return;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (g_pools[dev]) cudaMemPoolTrimTo(g_pools[dev], 0);
+}
+
+StreamScratch::StreamScratch(size_t bytes, cudaStream_t s) : st(s) {
+  cudaMemPool_t pool = scratch_pool();
+  if (pool) {
+    if (cudaMallocFromPoolAsync((void**)&p, bytes, pool, st) == cudaSuccess) return;
+    cudaGetLastError();
+    trim_scratch();
+  }
+  check_cuda(cudaMallocAsync((void**)&p, bytes, st), "cudaMallocAsync");
+}
+StreamScratch::~StreamScratch() { cudaFreeAsync(p, st); }
+
 DevBuf::~DevBuf() {
   if (p) cudaFree(p);
 }
@@ -70,6 +124,11 @@ void DevBuf::ensure(size_t n) {
   p = nullptr;
   bytes = 0;
   cudaError_t e = cudaMalloc(&p, n);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    trim_scratch();
+    e = cudaMalloc(&p, n);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     p = nullptr;
@@ -1243,18 +1302,6 @@ static void stage_out(const StagedPair& s, cudaStream_t st) {
 
 // ====================================================================== C ABI
 
-// Stream-ordered scratch of one call, given back on every way out.
-struct StreamScratch {
-  char* p = nullptr;
-  cudaStream_t st;
-  StreamScratch(size_t bytes, cudaStream_t s) : st(s) {
-    check_cuda(cudaMallocAsync((void**)&p, bytes, st), "cudaMallocAsync");
-  }
-  ~StreamScratch() { cudaFreeAsync(p, st); }
-  StreamScratch(const StreamScratch&) = delete;
-  StreamScratch& operator=(const StreamScratch&) = delete;
-};
-
 extern "C" {
 
 const char* gqt_last_error(void) { return g_last_error.c_str(); }
@@ -1661,8 +1708,8 @@ static gqt_status sigma_common(const double* d_in, const double* dt, int Nt, int
   if (Nt == 0 || NE == 0) return GQT_OK;
   for (int k = 0; k < Nt; ++k) require(std::isfinite(dt[k]) && dt[k] > 0, "time steps must be positive");
   cudaStream_t st = (cudaStream_t)stream;
-  double* ddt = nullptr;
-  check_cuda(cudaMallocAsync((void**)&ddt, Nt * sizeof(double), st), "cudaMallocAsync");
+  StreamScratch buf(Nt * sizeof(double), st);
+  double* ddt = (double*)buf.p;
   check_cuda(cudaMemcpyAsync(ddt, dt, Nt * sizeof(double), cudaMemcpyHostToDevice, st), "dt copy");
   const int nbk = std::max(1, std::min(1024, (NE + 127) / 128));
   if (vac)
@@ -1670,7 +1717,6 @@ static gqt_status sigma_common(const double* d_in, const double* dt, int Nt, int
   else
     k_sigma_msd<<<nbk, 128, 0, st>>>(d_in, ddt, Nt, NE, d_out);
   check_launch("k_sigma");
-  check_cuda(cudaFreeAsync(ddt, st), "cudaFreeAsync");
   check_cuda(cudaStreamSynchronize(st), "gqt_sigma");
   return GQT_OK;
 }
@@ -1695,9 +1741,8 @@ extern "C" gqt_status gqt_kpm_weights(int M, const double* d_E, int NE, const do
   require(d_E && d_w && d_beta && M >= 1 && NE >= 0 && energy_scale > 0 && (kernel == 0 || kernel == 1),
           "gqt_kpm_weights: bad argument");
   cudaStream_t st = (cudaStream_t)stream;
-  double* tab = nullptr;
-  check_cuda(cudaMallocAsync((void**)&tab, std::max<size_t>(1, (size_t)M * NE) * sizeof(double), st),
-             "cudaMallocAsync");
+  StreamScratch buf(std::max<size_t>(1, (size_t)M * NE) * sizeof(double), st);
+  double* tab = (double*)buf.p;
   const size_t total = (size_t)M * NE;
   if (total) {
     k_kpm_table<<<(int)std::min<size_t>((total + 255) / 256, 8192), 256, 0, st>>>(M, d_E, NE, energy_scale,
@@ -1706,7 +1751,6 @@ extern "C" gqt_status gqt_kpm_weights(int M, const double* d_E, int NE, const do
   }
   k_kpm_weights<<<(M + 127) / 128, 128, 0, st>>>(tab, M, NE, d_w, d_beta);
   check_launch("k_kpm_weights");
-  check_cuda(cudaFreeAsync(tab, st), "cudaFreeAsync");
   check_cuda(cudaStreamSynchronize(st), "gqt_kpm_weights");
   API_END
 }
@@ -1829,18 +1873,14 @@ extern "C" gqt_status gqt_sigma_vac_loss_weights(int M, const double* d_E, int N
     c[k] += 0.5 * dt[k];
     c[k + 1] += 0.5 * dt[k];
   }
-  double* buf = nullptr;
-  check_cuda(cudaMallocAsync((void**)&buf, (size_t)(M + K + 1) * sizeof(double), st), "cudaMallocAsync");
+  StreamScratch scratch((size_t)(M + K + 1) * sizeof(double), st);
+  double* buf = (double*)scratch.p;
   check_cuda(cudaMemcpyAsync(buf + M, c.data(), c.size() * sizeof(double), cudaMemcpyHostToDevice, st), "copy");
   gqt_status s = gqt_kpm_weights(M, d_E, NE, d_w, energy_scale, n_over_omega, kernel, buf, stream);
-  if (s != GQT_OK) {
-    cudaFreeAsync(buf, st);
-    return s;
-  }
+  if (s != GQT_OK) return s;
   const size_t total = (size_t)(K + 1) * M;
   k_trapezoid_outer<<<(int)std::min<size_t>((total + 255) / 256, 4096), 256, 0, st>>>(buf + M, K + 1, buf, M, d_beta);
   check_launch("k_trapezoid_outer");
-  check_cuda(cudaFreeAsync(buf, st), "cudaFreeAsync");
   check_cuda(cudaStreamSynchronize(st), "gqt_sigma_vac_loss_weights");
   API_END
 }

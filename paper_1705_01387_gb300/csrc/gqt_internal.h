@@ -40,6 +40,17 @@ void check_cuda(cudaError_t e, const char* what);
 void check_launch(const char* what);
 int sm_count();
 
+// Stream-ordered scratch of one call, given back on every way out (scratch pool of the
+// current device, gqt_host.cu).
+struct StreamScratch {
+  char* p = nullptr;
+  cudaStream_t st;
+  StreamScratch(size_t bytes, cudaStream_t s);
+  ~StreamScratch();
+  StreamScratch(const StreamScratch&) = delete;
+  StreamScratch& operator=(const StreamScratch&) = delete;
+};
+
 // Device allocation owned by its holder, grown on demand (contents not kept).
 struct DevBuf {
   void* p = nullptr;
