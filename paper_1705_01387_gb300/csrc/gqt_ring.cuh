@@ -24,7 +24,7 @@
 // 0.75 of HBM), 520 with T_{m+1} staged through L2 instead of shared memory; an l = r
 // pass at N = 4.2M 73.4 us (0.61), 79 before.  With the scalar operations the VAC pass is
 // at 484, with a band width read at run time at 460, with bands of 64 at 494; of the
-// instructions issued per site a third are not arithmetic.
+// 320 instructions per site of an l = r pass (450 of a VAC pass) 152 are arithmetic.
 //
 // Ring rows hold the cells B1 - 1 .. B1 + BW (entry 0: sublattice A of the left halo
 // cell).  T_{m+1} at the two halo sites that T_{m+2} needs (A left, B right) is computed
