@@ -862,13 +862,14 @@ int wave_grid(const gqt_ham* h, K kern, size_t smem) {
   return std::min(16, occupancy_of((const void*)kern, h->threads, smem));
 }
 
-// Vectors per lane: two FP32 ones (one 16-byte load) for R >= 2.
+// Vectors per lane: two FP32 ones (one 16-byte load) for R >= 2, where the caller's
+// vectors are 16-byte aligned.
 template <class F>
-void with_width(const gqt_ham* h, int R, F&& f) {
+void with_width(const gqt_ham* h, int R, bool aligned, F&& f) {
   dispatch(h, [&](auto H) {
     using Tr = EllTraits<decltype(H)>;
     if constexpr (!Tr::fp64) {
-      if (R >= 2) {
+      if (R >= 2 && aligned) {
         f(H, std::integral_constant<int, 2>());
         return;
       }
@@ -889,10 +890,12 @@ void gqt::launch_evolve_sets(gqt_ham* h, void* const* psi, int R, const std::vec
   }
   const int Np = (int)c.size();
   const bool wave = wave_evo_applies(h);
+  bool aligned = true;
+  for (int q = 0; q < NSET; ++q) aligned = aligned && (uintptr_t)psi[q] % 16 == 0;
   const size_t smem = smem_bytes(h, R, 4);
   int occ = 0;
   if (wave)
-    with_width(h, R, [&](auto H, auto vw) {
+    with_width(h, R, aligned, [&](auto H, auto vw) {
       using Tr = EllTraits<decltype(H)>;
       with_K(h->K, [&](auto kk) {
         occ = wave_grid(h, k_evolve_w<NSET, Tr::fp64, Tr::ch, decltype(vw)::value, decltype(kk)::value>, smem);
@@ -914,7 +917,7 @@ void gqt::launch_evolve_sets(gqt_ham* h, void* const* psi, int R, const std::vec
                                  {(double)NSET, (double)R, (double)Np, (double)h->threads, (double)wave, (double)nb}) +
                           coef_bits(c);
   run_graph(h, key, st, [&](cudaStream_t s2) {
-    with_width(h, R, [&](auto H, auto vw) {
+    with_width(h, R, aligned, [&](auto H, auto vw) {
       using Tr = EllTraits<decltype(H)>;
       using V = typename Tr::V;
       constexpr int VW = decltype(vw)::value;
@@ -983,10 +986,11 @@ void gqt::launch_msd_step(gqt_ham* h, void* p, void* px, int R, const std::vecto
   }
   const int Np = (int)c.size();
   const bool wave = wave_evo_applies(h);
+  const bool aligned = ((uintptr_t)p | (uintptr_t)px) % 16 == 0;
   const size_t smem = smem_bytes(h, R, 4);
   int occ = 0;
   if (wave)
-    with_width(h, R, [&](auto H, auto vw) {
+    with_width(h, R, aligned, [&](auto H, auto vw) {
       using Tr = EllTraits<decltype(H)>;
       with_K(h->K, [&](auto kk) {
         occ = wave_grid(h, k_msd_evolve_w<Tr::fp64, Tr::ch, decltype(vw)::value, decltype(kk)::value>, smem);
@@ -1005,7 +1009,7 @@ void gqt::launch_msd_step(gqt_ham* h, void* p, void* px, int R, const std::vecto
   const std::string key = key_of("msd", {p, px, U1, Z1, AP, AX, partial, T.d_blk.p},
                                  {(double)R, (double)Np, (double)h->threads, (double)wave, (double)nb}) + coef_bits(c);
   run_graph(h, key, st, [&](cudaStream_t s2) {
-    with_width(h, R, [&](auto H, auto vw) {
+    with_width(h, R, aligned, [&](auto H, auto vw) {
       using Tr = EllTraits<decltype(H)>;
       using V = typename Tr::V;
       constexpr int VW = decltype(vw)::value;
