@@ -11,6 +11,8 @@
 #include <map>
 #include <numeric>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "gqt_internal.h"
@@ -316,38 +318,93 @@ static int64_t detect_honeycomb(const HostModel& m, int (&type)[2][3]) {
 
 // Row classes of a model (gqt_ham::d_cls): the distinct offset vectors of its rows in
 // order of appearance, and each row's class.  False for an irregular model (more than
-// ROW_CLASSES of them) or more than 8 slots.
+// ROW_CLASSES of them) or more than 8 slots.  Ranges of rows are scanned by a few
+// threads, each with classes of its own, which are then numbered in common: a row costs
+// 5 ns, 5.5 of the 60 ms in which a lattice of a million sites is built.
 constexpr int ROW_CLASSES = 4096;
-static bool row_classes(const HostModel& m, std::vector<uint16_t>& cls, std::vector<int32_t>& off) {
-  const int K = m.K;
-  if (K > 8) return false;
-  cls.resize(m.n);
+struct ClassScan {
   std::map<std::vector<int32_t>, int> known;
-  std::vector<int32_t> o(K);
-  auto same = [&](int64_t i, int c) {
-    for (int k = 0; k < K; ++k)
-      if (m.idx[i * K + k] - (int32_t)i != off[8 * c + k]) return false;
-    return true;
-  };
-  for (int64_t i = 0; i < m.n; ++i) {
-    int c = -1;
-    for (int64_t b = 1; b <= 2 && c < 0 && i >= b; ++b)  // most rows repeat one of the two before
-      if (same(i, cls[i - b])) c = cls[i - b];
-    if (c < 0) {
-      for (int k = 0; k < K; ++k) o[k] = m.idx[i * K + k] - (int32_t)i;
-      auto it = known.find(o);
-      if (it != known.end()) {
-        c = it->second;
-      } else {
-        c = (int)known.size();
-        if (c == ROW_CLASSES) return false;
-        known.emplace(o, c);
-        off.insert(off.end(), o.begin(), o.end());
-        off.resize((size_t)8 * (c + 1), 0);
+  std::vector<int32_t> off;  // [classes][8]
+  bool regular = true;
+  // class of the offsets o, a new one if need be; -1: too many
+  int find(const std::vector<int32_t>& o) {
+    auto it = known.find(o);
+    if (it != known.end()) return it->second;
+    const int c = (int)known.size();
+    if (c == ROW_CLASSES) return -1;
+    known.emplace(o, c);
+    off.insert(off.end(), o.begin(), o.end());
+    off.resize((size_t)8 * (c + 1), 0);
+    return c;
+  }
+  void rows(const HostModel& m, int64_t beg, int64_t end, uint16_t* cls) {
+    const int K = m.K;
+    std::vector<int32_t> o(K);
+    auto same = [&](int64_t i, int c) {
+      for (int k = 0; k < K; ++k)
+        if (m.idx[i * K + k] - (int32_t)i != off[8 * c + k]) return false;
+      return true;
+    };
+    for (int64_t i = beg; i < end; ++i) {
+      int c = -1;
+      for (int64_t b = 1; b <= 2 && c < 0 && i - b >= beg; ++b)  // most rows repeat one of the two before
+        if (same(i, cls[i - b])) c = cls[i - b];
+      if (c < 0) {
+        for (int k = 0; k < K; ++k) o[k] = m.idx[i * K + k] - (int32_t)i;
+        c = find(o);
+        if (c < 0) {
+          regular = false;
+          return;
+        }
+      }
+      cls[i] = (uint16_t)c;
+    }
+  }
+};
+
+static bool row_classes(const HostModel& m, std::vector<uint16_t>& cls, std::vector<int32_t>& off) {
+  if (m.K > 8) return false;
+  cls.resize(m.n);
+  const int T = m.n < 65536 ? 1 : (int)std::min(8u, std::max(1u, std::thread::hardware_concurrency()));
+  auto first = [&](int t) { return m.n * t / T; };
+  // work(t) for every range, on threads of their own where they can be had
+  auto ranges = [&](auto&& work) {
+    std::vector<std::thread> th;
+    th.reserve(T);
+    for (int t = 1; t < T; ++t) {
+      try {
+        th.emplace_back(work, t);
+      } catch (const std::system_error&) {
+        work(t);
       }
     }
-    cls[i] = (uint16_t)c;
-  }
+    work(0);
+    for (auto& t : th) t.join();
+  };
+  std::vector<ClassScan> part(T);
+  ranges([&](int t) {
+    try {
+      part[t].rows(m, first(t), first(t + 1), cls.data());
+    } catch (const std::exception&) {  // out of memory: no classes
+      part[t].regular = false;
+    }
+  });
+  for (const auto& p : part)
+    if (!p.regular) return false;
+  ClassScan all;
+  std::vector<std::vector<uint16_t>> number(T);
+  for (int t = 0; t < T; ++t)
+    for (size_t c = 0; 8 * c < part[t].off.size(); ++c) {
+      const auto o = part[t].off.begin() + 8 * c;
+      const int g = all.find(std::vector<int32_t>(o, o + m.K));
+      if (g < 0) return false;
+      number[t].push_back((uint16_t)g);
+    }
+  ranges([&](int t) {
+    if (t == 0) return;  // numbered as they stand
+    for (int64_t i = first(t); i < first(t + 1); ++i) cls[i] = number[t][cls[i]];
+  });
+  off = std::move(all.off);
   return true;
 }
 

@@ -85,3 +85,28 @@ def test_common_hopping_of_fp32_handles_follows_updates():
             for _ in range(2):  # the second call replays the captured graph
                 g.gqt_dos_moments(h, r, 1, M, m)
         assert np.array_equal(mu[0], mu[1])
+
+
+@pytest.mark.parametrize("what", ["regular", "too many in one range", "too many together"])
+def test_classes_of_large_models(what):
+    """Models whose rows are scanned in ranges by several threads (65536 sites and more):
+    one whose classes agree across ranges, one range with more than 4096, and ranges with
+    fewer each that have more together."""
+    lat = S.square(331, 257, -1.0, 1.0, seed=3)
+    n = lat.n
+    p = np.arange(n)
+    rng = np.random.default_rng(1)
+    if what == "too many in one range":
+        p[40000:48000] = rng.permutation(p[40000:48000])
+    elif what == "too many together":
+        for a in range(0, n - 3000, 10000):
+            p[a:a + 700] = rng.permutation(p[a:a + 700])
+    q = np.argsort(p)
+    other = dataclasses.replace(lat, nb_count=lat.nb_count[q], nb_idx=p[lat.nb_idx[q]].astype(np.int32), hop=lat.hop[q],
+                                onsite=lat.onsite[q], dx=lat.dx[q], dy=None)
+    dE = S.energy_scale_rule(4, -1.0, 1.0)
+    vecs = [S.random_phase(n, 1, seed=s) for s in (1, 2, 3, 4)]
+    x = _rows(lat, dE, g.GQT_FP64, 1, True, vecs, M=11)
+    y = _rows(other, dE, g.GQT_FP64, 1, True, [v[q] for v in vecs], M=11)
+    for u, v in zip(x, y):
+        assert np.all(np.abs(u - v) < 1e-13 * max(1.0, np.abs(u).max()))
