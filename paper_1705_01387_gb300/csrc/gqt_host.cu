@@ -1252,9 +1252,30 @@ void gqt::launch_velocity(gqt_ham* h, const void* x, void* y, void* ycopy, int R
   dispatch(h, [&](auto H) {
     using Tr = EllTraits<decltype(H)>;
     using V = typename Tr::V;
-    k_velocity<Tr::fp64, Tr::ch><<<nb, h->threads, smem_bytes(h, R, 3), st>>>(H, (const int*)T.d_blk.p, R, rs, 0.5 * h->dE, (const V*)x,
-                                                             (V*)y, (V*)ycopy);
-    check_launch("k_velocity");
+    auto unrolled = [&](auto kk, auto vw) {
+      constexpr int VW = decltype(vw)::value;
+      const size_t total = (size_t)h->n * R / VW;
+      k_velocity_w<Tr::fp64, Tr::ch, decltype(kk)::value, VW><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
+          H, total, rs - (VW - 1), R, 0.5 * h->dE, (const V*)x, (V*)y, (V*)ycopy);
+      check_launch("k_velocity_w");
+    };
+    const bool two = R >= 2 && ((uintptr_t)x | (uintptr_t)y | (uintptr_t)ycopy) % 16 == 0;
+    auto by_width = [&](auto kk) {
+      if (two)
+        unrolled(kk, std::integral_constant<int, 2>());
+      else
+        unrolled(kk, std::integral_constant<int, 1>());
+    };
+    switch ((size_t)h->n * R < ((size_t)1 << 38) ? h->K : 0) {  // at most 2^31 - 1 CTAs
+      case 2: by_width(std::integral_constant<int, 2>()); break;
+      case 3: by_width(std::integral_constant<int, 3>()); break;
+      case 4: by_width(std::integral_constant<int, 4>()); break;
+      case 6: by_width(std::integral_constant<int, 6>()); break;
+      default:
+        k_velocity<Tr::fp64, Tr::ch><<<nb, h->threads, smem_bytes(h, R, 3), st>>>(
+            H, (const int*)T.d_blk.p, R, rs, 0.5 * h->dE, (const V*)x, (V*)y, (V*)ycopy);
+        check_launch("k_velocity");
+    }
   });
 }
 

@@ -825,6 +825,83 @@ __global__ void k_velocity(Ell<FP64, CH> H, const int* __restrict__ blk, int R, 
   }
 }
 
+// VW adjacent vectors of a site as one load or store (VW = 2: 16-byte aligned FP32, 32
+// bytes of FP64 in two halves).
+template <int VW, class V>
+__device__ __forceinline__ void vel_ld(V (&d)[VW], const V* __restrict__ p) {
+  if constexpr (VW == 2 && sizeof(V) == 8) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    d[0].x = t.x;
+    d[0].y = t.y;
+    d[1].x = t.z;
+    d[1].y = t.w;
+  } else {
+#pragma unroll
+    for (int w = 0; w < VW; ++w) d[w] = __ldg(p + w);
+  }
+}
+template <int VW, class V>
+__device__ __forceinline__ void vel_st(V* __restrict__ p, const V (&d)[VW]) {
+  if constexpr (VW == 2 && sizeof(V) == 8) {
+    *reinterpret_cast<float4*>(p) = make_float4(d[0].x, d[0].y, d[1].x, d[1].y);
+  } else {
+#pragma unroll
+    for (int w = 0; w < VW; ++w) p[w] = d[w];
+  }
+}
+
+// k_velocity for 2, 3, 4 and 6 slots: a row's displacements, hoppings and neighbours are
+// in flight at once, VW vectors of a site per thread (2 from R = 2 on, where the vectors
+// are 16-byte aligned).  Real FP64 hoppings are multiplied by the displacement first: 11
+// instead of 14 FP64 operations at three slots, the bound of the FP64 form; FP32 keeps
+// its order of operations.  16.8M sites, FP64, K = 3: 460 -> 343 us (FP64 pipe 294); 2.1M
+// sites, FP32, R = 8: 234 -> 72 us; 2048 sites: 4.4 -> 2.3 us.
+template <bool FP64, bool CH, int KK, int VW>
+__global__ void __launch_bounds__(256) k_velocity_w(Ell<FP64, CH> H, size_t total, int gs, int R, double half_dE,
+                                                    const typename Prec<FP64>::V* __restrict__ x,
+                                                    typename Prec<FP64>::V* __restrict__ y,
+                                                    typename Prec<FP64>::V* __restrict__ y2) {
+  using V = typename Prec<FP64>::V;
+  using S = typename Prec<FP64>::S;
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t >= total) return;
+  const int i = (int)(t >> gs), off = VW * (int)(t & (((size_t)1 << gs) - 1));
+  const size_t e = (size_t)i * R + off;
+  int idx[KK];
+  S dx[KK];
+  typename Ell<FP64, CH>::HT hv[KK];
+  row_neighbours<KK>(H.idx, H.cls, H.cls_off, H.n, i, row_class(H.cls, i), idx);
+#pragma unroll
+  for (int k = 0; k < KK; ++k) {
+    hv[k] = hop_of(H, k, i);
+    dx[k] = __ldg(H.dx + (size_t)k * H.n + i);
+  }
+  V nb[KK][VW];
+#pragma unroll
+  for (int k = 0; k < KK; ++k) vel_ld<VW>(nb[k], x + (size_t)idx[k] * R + off);
+  V o[VW];
+#pragma unroll
+  for (int w = 0; w < VW; ++w) {
+    V a;
+    a.x = 0;
+    a.y = 0;
+#pragma unroll
+    for (int k = 0; k < KK; ++k) {
+      if constexpr (FP64 && !CH)
+        a = cmul_acc(a, hv[k] * dx[k], nb[k][w]);
+      else
+        a = cmul_acc(a, hv[k], cscale(nb[k][w], dx[k]));
+    }
+    o[w].x = -a.y * (S)half_dE;
+    o[w].y = a.x * (S)half_dE;
+  }
+  vel_st<VW>(y + e, o);
+  if (y2) {
+    vel_ld<VW>(o, x + e);
+    vel_st<VW>(y2 + e, o);
+  }
+}
+
 // --------------------------------------------------------------- K7: KPM
 
 // tab[n][e] = g_n (2 - delta_n0) cos(n arccos x_e) * 2 n_over_omega / (pi dE sqrt(1 - x_e^2))
