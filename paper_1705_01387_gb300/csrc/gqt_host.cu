@@ -1122,6 +1122,20 @@ void gqt::launch_moments(gqt_ham* h, const void* l, const void* r, int R, int M,
     launch_moments_df(h, l, r, M, out, kind, st);
     return;
   }
+  // The multi-vector kernels of FP32 handles read two vectors of a site in one 16-byte
+  // load.  A caller's array may start at any multiple of 8 bytes: one that is not 16-byte
+  // aligned is copied first (one pass over it, before orders that each read it or more).
+  if (h->prec != GQT_FP64 && R >= 2 && kind != 0) {
+    auto aligned = [&](const void* x, int slot) -> const void* {
+      if ((uintptr_t)x % 16 == 0) return x;
+      void* c = h->ws(slot, vb).p;
+      check_cuda(cudaMemcpyAsync(c, x, vb, cudaMemcpyDeviceToDevice, st), "aligned copy");
+      return c;
+    };
+    const bool same = l == r;
+    r = aligned(r, WS_ALIGN0);
+    l = same ? r : aligned(l, WS_ALIGN0 + 1);
+  }
   const bool pair = kind == 1 && pair_applies(h, R);
   void* wa1 = pair ? h->ws(WS_PA1, vb).p : nullptr;
   void* wa2 = pair ? h->ws(WS_PA2, vb).p : nullptr;

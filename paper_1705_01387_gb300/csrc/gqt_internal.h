@@ -88,7 +88,8 @@ enum WorkSlot {
   WS_ADJ0 = 20,  // adjoint workspace slots start here
   WS_STAGE0 = 96,  // +0, +1: host-resident VAC/MSD state staged on the device
   WS_TILE0 = 98,   // +0..+3: the third and fourth chain buffers of the tiled rows
-  WS_TILE_SCRATCH = 102  // per-CTA partial dots of a tiled grid larger than the single-order grid
+  WS_TILE_SCRATCH = 102,  // per-CTA partial dots of a tiled grid larger than the single-order grid
+  WS_ALIGN0 = 104  // +0, +1: 16-byte aligned copies of a moment row's vectors
 };
 
 uint64_t splitmix_mix(uint64_t z);
