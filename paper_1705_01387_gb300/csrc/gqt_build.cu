@@ -665,9 +665,7 @@ extern "C" gqt_status gqt_update_hamiltonian(gqt_ham* h, const double* onsite, c
       if (uni != h->hop_uniform || h0 != h->hop0) {
         // the blocked rows switch form, or their common hopping (a kernel argument
         // inside the captured graphs) changes: retire the graphs
-        for (auto& gr : h->graphs) cudaGraphExecDestroy(gr.second);
-        h->graphs.clear();
-        h->graph_data.clear();
+        h->drop_graphs();
       }
       h->hop_uniform = uni;
       h->hop0 = h0;
@@ -690,9 +688,7 @@ extern "C" gqt_status gqt_update_hamiltonian(gqt_ham* h, const double* onsite, c
       const bool uni = hw == 1 && std::all_of(hop.begin(), hop.end(), [&](float v) { return v == hop[0]; });
       const float h0 = uni ? hop[0] : 0.f;
       if (uni != h->hop_uniform32 || h0 != h->hop0f) {  // a kernel argument of the captured graphs
-        for (auto& gr : h->graphs) cudaGraphExecDestroy(gr.second);
-        h->graphs.clear();
-        h->graph_data.clear();
+        h->drop_graphs();
       }
       h->hop_uniform32 = uni;
       h->hop0f = h0;

@@ -425,8 +425,26 @@ const BlockTable& gqt_ham::table(int R, int grid_per_sm) {
 DevBuf& gqt_ham::ws(int slot, size_t bytes) {
   if ((int)work.size() <= slot) work.resize(slot + 1);
   if (!work[slot]) work[slot] = std::make_unique<DevBuf>();
-  work[slot]->ensure(bytes);
-  return *work[slot];
+  DevBuf& b = *work[slot];
+  const void* before = b.p;
+  try {
+    b.ensure(bytes);
+  } catch (...) {
+    if (before) drop_graphs();  // the growth has freed the buffer
+    throw;
+  }
+  if (before && b.p != before) drop_graphs();
+  return b;
+}
+
+// Retires the captured graphs: a setting has changed which kernels run or their
+// parameters, or a workspace has moved.  (A graph's key names some of its buffers only,
+// and a slot that a call has no key for may grow by itself: two-set evolutions at one
+// R after one-set evolutions at a larger one.)
+void gqt_ham::drop_graphs() {
+  for (auto& g : graphs) cudaGraphExecDestroy(g.second);
+  graphs.clear();
+  graph_data.clear();
 }
 
 // ====================================================================== dispatch helpers
@@ -1414,19 +1432,11 @@ gqt_status gqt_set_graphs(gqt_ham* h, int enable) {
   API_END
 }
 
-// A setting that changes which kernels run, or their parameters, retires the
-// handle's captured graphs (their launches carry the old choice).
-static void drop_graphs(gqt_ham* h) {
-  for (auto& g : h->graphs) cudaGraphExecDestroy(g.second);
-  h->graphs.clear();
-  h->graph_data.clear();
-}
-
 gqt_status gqt_set_cluster(gqt_ham* h, int enable) {
   API_BEGIN
   require(h != nullptr, "null handle");
   h->use_cluster = enable != 0;
-  drop_graphs(h);
+  h->drop_graphs();
   API_END
 }
 
@@ -1434,7 +1444,7 @@ gqt_status gqt_set_vac_pair(gqt_ham* h, int enable) {
   API_BEGIN
   require(h != nullptr, "null handle");
   h->use_pair = enable != 0;
-  drop_graphs(h);
+  h->drop_graphs();
   API_END
 }
 
@@ -1442,7 +1452,7 @@ gqt_status gqt_set_temporal_blocking(gqt_ham* h, int enable) {
   API_BEGIN
   require(h != nullptr, "null handle");
   h->use_tiling = enable != 0;
-  drop_graphs(h);
+  h->drop_graphs();
   API_END
 }
 
@@ -1450,7 +1460,7 @@ gqt_status gqt_set_fp64_arith(gqt_ham* h, int mode) {
   API_BEGIN
   require(h != nullptr && (mode == 0 || mode == 1), "gqt_set_fp64_arith: mode must be 0 or 1");
   h->fp64_arith = mode;
-  drop_graphs(h);
+  h->drop_graphs();
   API_END
 }
 
@@ -1458,7 +1468,7 @@ gqt_status gqt_set_sweep_order(gqt_ham* h, int enable) {
   API_BEGIN
   require(h != nullptr, "null handle");
   h->use_sweep_order = enable != 0;
-  drop_graphs(h);
+  h->drop_graphs();
   API_END
 }
 
@@ -1466,8 +1476,7 @@ gqt_status gqt_set_variant(gqt_ham* h, int variant) {
   API_BEGIN
   require(h != nullptr && variant >= 0 && variant <= 3, "gqt_set_variant: variant must be 0, 1, 2 or 3");
   h->variant = variant;
-  for (auto& g : h->graphs) cudaGraphExecDestroy(g.second);
-  h->graphs.clear();
+  h->drop_graphs();
   API_END
 }
 
@@ -1480,8 +1489,7 @@ gqt_status gqt_set_launch(gqt_ham* h, int threads, int blocks_per_sm) {
   h->threads = threads;
   h->blocks_per_sm = blocks_per_sm;
   h->tables.clear();
-  for (auto& g : h->graphs) cudaGraphExecDestroy(g.second);
-  h->graphs.clear();
+  h->drop_graphs();
   API_END
 }
 
@@ -1852,8 +1860,7 @@ extern "C" gqt_status gqt_autotune(gqt_ham* h, int R, int* threads, int* blocks_
   h->blocks_per_sm = bb;
   h->variant = bv;
   h->tables.clear();
-  for (auto& g : h->graphs) cudaGraphExecDestroy(g.second);
-  h->graphs.clear();
+  h->drop_graphs();
   reset_flag(h, st);
   check_cuda(cudaStreamSynchronize(st), "gqt_autotune");
   if (threads) *threads = bt;

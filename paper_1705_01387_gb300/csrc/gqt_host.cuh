@@ -84,11 +84,7 @@ inline void run_graph(gqt_ham* h, std::string key, cudaStream_t st, F&& launches
   }
   auto it = h->graphs.find(key);
   if (it == h->graphs.end()) {
-    if (h->graphs.size() >= 512) {
-      for (auto& g : h->graphs) cudaGraphExecDestroy(g.second);
-      h->graphs.clear();
-      h->graph_data.clear();
-    }
+    if (h->graphs.size() >= 512) h->drop_graphs();
     cudaGraph_t graph = nullptr;
     check_cuda(cudaStreamBeginCapture(h->gstream, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
     try {

@@ -158,6 +158,7 @@ struct gqt_ham {
 
   const gqt::BlockTable& table(int R, int grid_per_sm = 0);
   gqt::DevBuf& ws(int slot, size_t bytes);
+  void drop_graphs();
   size_t vec_bytes(int R) const;
   ~gqt_ham();
 };
