@@ -336,6 +336,20 @@ __global__ void __launch_bounds__(512) k_cheb_cluster1(Ell<FP64, CH> H, int chun
   cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
+// Allows a cluster kernel clusters of C CTAs and its largest shared memory.  The attributes
+// belong to the kernel, which all handles and threads share: they are set to the same
+// values by every call, never to what one call needs, since another thread may launch
+// between the two.
+constexpr size_t CL_SMEM = 220 * 1024;
+template <class KERN>
+inline bool cluster_attributes(KERN kern, int C) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM) == cudaSuccess &&
+      (C <= 8 || cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess))
+    return true;
+  cudaGetLastError();
+  return false;
+}
+
 // Launches one of the one-site-per-thread cluster kernels for n sites: clusters of 16
 // CTAs where the GPU allows, else 8, of a power of two of threads (the ring's parts), at
 // most 512; smem_of(chunk, threads) bytes of shared memory; f(config, chunk) launches.
@@ -348,12 +362,7 @@ inline bool cluster1_launch(KERN kern, int64_t n, cudaStream_t st, SM&& smem_of,
     while (thr < chunk && thr <= 512) thr *= 2;
     if (thr > 512) continue;
     const size_t smem = smem_of(chunk, thr);
-    if (smem > 220 * 1024) continue;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        (C > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
-      cudaGetLastError();
-      continue;
-    }
+    if (smem > CL_SMEM || !cluster_attributes(kern, C)) continue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C, 1, 1);
     cfg.blockDim = dim3(thr, 1, 1);

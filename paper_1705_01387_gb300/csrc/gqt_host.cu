@@ -538,12 +538,7 @@ static bool launch_cluster_row(gqt_ham* h, const Ell<FP64, CH>& H, const V* r, c
     const int chunk = (int)((h->n + C - 1) / C);
     const int thr = std::min(1024, std::max(32, (chunk + 31) / 32 * 32));
     const size_t smem = (size_t)chunk * per_site + 64 + cluster_red_bytes(M, slot_norm, thr / 32) + 16;
-    if (smem > 220 * 1024) continue;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        (C > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
-      cudaGetLastError();
-      continue;
-    }
+    if (smem > CL_SMEM || !cluster_attributes(kern, C)) continue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C, 1, 1);
     cfg.blockDim = dim3(thr, 1, 1);
@@ -778,7 +773,10 @@ static RingGrid ring_grid(const gqt_ham* h) {
   const size_t most = ring_smem(bw, NC, std::min(RG_ROWS, h->honey_L2));
   int n = 0;
   with_ring<NC>(h, [&](auto kern) {
-    check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most), "smem attribute");
+    // the size of the longest pieces for every handle: the attribute belongs to the kernel,
+    // and another thread's handle may set it before this one launches
+    check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)ring_smem(bw, NC, RG_ROWS)), "smem attribute");
     check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, 2 * bw, most), "occupancy");
   });
   const int res = std::max(1, n) * sm_count();
