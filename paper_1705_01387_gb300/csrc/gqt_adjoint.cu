@@ -83,14 +83,14 @@ struct AdjTerms {
 };
 
 // Order m of the forward recursion, one site per thread: out = 2H~ t1 - t2 (first: out =
-// H~ t1) and, where on, the accumulator's terms up to it.  FP64 pipe bound (8 + 2
+// H~ t1) and, where on, the accumulator's terms up to it.  t2 and out may be one buffer
+// (each element is read and written by its thread only).  FP64 pipe bound (8 + 2
 // multiply-adds per site), so the grid is as fine as the sites allow: 1024 CTAs of 128
 // at 131,072 sites leave 4% of the SM time idle, 256 of 256 with two sites a thread 16%.
 template <bool FP64, bool CH, int KK>
 __global__ void __launch_bounds__(128) k_recur(Ell<FP64, CH> H, const typename Prec<FP64>::V* __restrict__ t1,
-                                               const typename Prec<FP64>::V* __restrict__ t2,
-                                               typename Prec<FP64>::V* __restrict__ out, double2* __restrict__ acc,
-                                               AdjTerms t, int first) {
+                                               const typename Prec<FP64>::V* t2, typename Prec<FP64>::V* out,
+                                               double2* __restrict__ acc, AdjTerms t, int first) {
   using V = typename Prec<FP64>::V;
   using S = typename Prec<FP64>::S;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(128) k_recur(Ell<FP64, CH> H, const typename P
   const AdjRow<Ell<FP64, CH>, KK> row(H, i);
   V tm2, y;
   tm2.x = tm2.y = 0;
-  if (!first) tm2 = __ldg(t2 + i);
+  if (!first) tm2 = t2[i];
   y = row.apply(H, i, t1, first ? tm2 : cneg(tm2));
   if (first) y = cscale(y, (S)0.5);
   out[i] = y;
