@@ -259,15 +259,17 @@ gqt_status gqt_kb_moments(gqt_ham* ham, const void* d_r, int R, int M, int alpha
 gqt_status gqt_set_kb_contraction(gqt_ham* ham, int mode);
 
 /* Polls of each bounded device wait of the handle's kernels (default 2^24, a
- * few tenths of a second to seconds; 0 = give up at once).  The kernel that takes
- * this setting is the split-TF32 Hall contraction (gqt_set_kb_contraction mode
- * 1; the FP64 contraction's and the blocked FP64 moment rows' waits for their copies
- * always have 2^24 polls and end the same way): its single issuing thread waits on mbarriers for the bulk tensor copies of
- * each stage and for the commit of the products that read a buffer.  A wait that
- * runs out stops the pipeline; the thread then drains what is in flight (the
- * last committed products and the issued copies, 2^24 polls each, independent of
- * this setting), frees its tensor memory and the call returns GQT_ETIMEOUT; the
- * moments it wrote are not valid.  The handle stays usable.  If the drain
+ * few tenths of a second to seconds; 0 = give up at once).  The kernels that wait are
+ *  - the split-TF32 Hall contraction (gqt_set_kb_contraction mode 1), whose single
+ *    issuing thread waits on mbarriers for the bulk tensor copies of each stage and for
+ *    the commit of the products that read a buffer, and
+ *  - the blocked FP64 moment rows (gqt_set_temporal_blocking), which wait for the bulk
+ *    copies of their rows.
+ * (The FP64 Hall contraction's waits always have 2^24 polls and end the same way.)
+ * A wait that runs out is reported; what is in flight is then drained (committed
+ * products and issued copies, 2^24 polls each, independent of this setting), tensor
+ * memory is freed and the call returns GQT_ETIMEOUT; the moments it
+ * wrote are not valid.  The handle stays usable.  If the drain
  * itself gives up (the error message then says so), products or copies may still
  * be in flight when the CTA frees its tensor memory and exits: treat the CUDA
  * context as suspect and restart the process.  This is the library's failure

@@ -941,6 +941,7 @@ extern "C" gqt_status gqt_set_wait_limit(gqt_ham* h, int polls) {
     return GQT_EINVAL;
   }
   h->wait_limit = polls;
+  h->drop_graphs();  // the limit is a kernel argument
   return GQT_OK;
 }
 

@@ -795,13 +795,13 @@ static RingGrid ring_grid(const gqt_ham* h) {
 // One blocked pass; the kernels of the other hopping type are compiled but not launched.
 template <bool CK, bool CH>
 static void ring_launch(void (*kern)(DfEll<CK>, Honey, RingHop, int, int, const float4*, const float4*, const float4*,
-                                     const float4*, float4*, float4*, float4*, float4*, double2*, int, int, int*),
+                                     const float4*, float4*, float4*, float4*, float4*, double2*, int, int, int*, int),
                         const DfEll<CH>& H, const Honey& G, const RingHop& hs, const RingGrid& rg, int threads,
                         const float4* xa, const float4* ya, const float4* xb, const float4* yb, float4* za, float4* wa,
-                        float4* zb, float4* wb, double2* pout, int ostride, int nzero, int* err, cudaStream_t st) {
+                        float4* zb, float4* wb, double2* pout, int ostride, int nzero, int* err, int limit, cudaStream_t st) {
   if constexpr (CK == CH)
     kern<<<rg.grid, threads, rg.smem, st>>>(H, G, hs, rg.nseg, rg.rows, xa, ya, xb, yb, za, wa, zb, wb, pout, ostride,
-                                            nzero, err);
+                                            nzero, err, limit);
 }
 
 // The rows' chains live in rotating buffers (4 per chain when tiled, else 2):
@@ -871,12 +871,12 @@ static void df_rows(gqt_ham* h, const BlockTable& T, bool pair, int steps, const
         if (pair)
           with_ring<2>(h, [&](auto kern) {
             ring_launch(kern, H, G, hs, rg, 2 * bw, A[cur], A[prv], B[cur], B[prv], A[f[0]], A[f[1]], B[f[0]], B[f[1]],
-                        pout, ostride, nzero, (int*)h->d_flag.p, s2);
+                        pout, ostride, nzero, (int*)h->d_flag.p, h->wait_limit, s2);
           });
         else
           with_ring<1>(h, [&](auto kern) {
             ring_launch(kern, H, G, hs, rg, 2 * bw, B[cur], B[prv], nullptr, nullptr, B[f[0]], B[f[1]], nullptr,
-                        nullptr, pout, ostride, nzero, (int*)h->d_flag.p, s2);
+                        nullptr, pout, ostride, nzero, (int*)h->d_flag.p, h->wait_limit, s2);
           });
         check_launch("k_cheb2_honey_df");
         if (fold) {

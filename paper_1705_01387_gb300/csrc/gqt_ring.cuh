@@ -35,9 +35,13 @@
 // cut into gridDim.x equal ranges instead; a range that crosses a band's end, or is
 // longer than RG_ROWS, is walked in pieces.
 //
-// The waits for the copies are bounded.  A CTA whose wait runs out marks itself, goes
-// through its remaining rows without waiting, drains the copies it has in flight and
-// sets bit 16 of the status word (32 if the drain ran out too).
+// The waits for the copies are bounded (gqt_set_wait_limit).  One that runs out sets bit
+// 16 of the status word and goes on as a drain of RG_DRAIN polls: a slot may be filled
+// again only when its row has landed, and no CTA may end with a copy in flight.  If the
+// drain runs out too (bit 32), the thread that issues the copies leaves, so that none
+// follows, and the others go through the remaining rows without waiting.  All of it is in
+// the path of a poll that failed: a flag looked at before each row is asked for costs 5%
+// of an l = r pass.
 #pragma once
 
 #include "gqt_tile.cuh"
@@ -52,7 +56,7 @@ __host__ __device__ inline int tl_band_width(int L1) {
 constexpr int RG_X = 6;       // rows of T_m in shared memory: four in use, two on their way
 constexpr int RG_Z = 4;       // rows of T_{m+1}
 constexpr int RG_ROWS = 256;  // rows of a piece at most (its halo columns are kept)
-constexpr int RG_LIMIT = 1 << 24;
+constexpr int RG_DRAIN = 1 << 24;  // polls of a drain
 
 __host__ __device__ constexpr int ring_row(int bw) { return 2 * bw + 4; }  // entries of a ring row
 inline size_t ring_smem(int bw, int nc, int rows) {
@@ -69,27 +73,28 @@ __device__ __forceinline__ bool rg_poll(uint32_t bar, uint32_t parity) {
       : "memory");
   return done != 0;
 }
-// The rest of a wait whose first poll failed; a CTA marked dead waits no more.
-__device__ __noinline__ void rg_wait_slow(uint32_t bar, uint32_t parity, volatile int* dead) {
-  for (int it = 0; it < RG_LIMIT; ++it) {
-    if (*dead) return;
+// What a CTA's waits share.
+struct RingWait {
+  int* err;    // status word
+  int limit;   // polls of a wait
+  int dead;    // a drain has run out
+};
+// The rest of a wait whose first poll failed.
+__device__ __noinline__ void rg_wait_slow(uint32_t bar, uint32_t parity, volatile RingWait* w) {
+  const bool issuer = threadIdx.x == 0;
+  const int limit = w->limit;
+  for (int it = 0; it < limit; ++it) {
     if (rg_poll(bar, parity)) return;
+    if (w->dead && !issuer) return;
   }
-  *dead = 1;
-}
-// End of a CTA marked dead: the copies that had not landed when the waits ran out, and
-// the status word.  sw, pw: the slot after the last row waited for, and its parity.
-__device__ __forceinline__ void rg_finish(volatile int* dead, uint32_t bar, int sw, uint32_t pw, int* err) {
-  if (threadIdx.x != 0 || !*dead) return;
-  bool drained = true;
-  for (int q = 0; q < RG_X; ++q) {
-    // rows take the slots in turn: those before sw are one phase further
-    const uint32_t par = (q < sw ? pw : pw ^ 1u) & 1u;
-    bool ok = false;
-    for (int it = 0; it < RG_LIMIT && !ok; ++it) ok = rg_poll(bar + 8 * q, par);
-    drained = drained && ok;
+  atomicOr(w->err, 16);
+  for (int it = 0; it < RG_DRAIN; ++it) {
+    if (rg_poll(bar, parity)) return;
+    if (w->dead && !issuer) return;
   }
-  atomicOr(err, drained ? 16 : (16 | 32));
+  w->dead = 1;
+  atomicOr(w->err, 32);
+  if (issuer) asm volatile("exit;");
 }
 __device__ __forceinline__ void rg_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile(
@@ -228,7 +233,7 @@ __global__ void __launch_bounds__(2 * BW, (NC == 1 && UH ? 3 : 2) * (128 / BW)) 
     DfEll<CH> H, Honey G, RingHop hs, int nseg, int max_rows, const float4* __restrict__ xa,
     const float4* __restrict__ ya, const float4* __restrict__ xb, const float4* __restrict__ yb,
     float4* __restrict__ za, float4* __restrict__ wa, float4* __restrict__ zb, float4* __restrict__ wb,
-    double2* __restrict__ pout, int ostride, int nzero, int* __restrict__ err) {
+    double2* __restrict__ pout, int ostride, int nzero, int* __restrict__ err, int limit) {
   using HT = typename DfHop<CH>::T;
   constexpr int RW = ring_row(BW), RB = RW * 16;   // a ring row: entries, bytes
   constexpr int XCH = RG_X * RB, ZCH = RG_Z * RB;  // a chain's rings in bytes
@@ -237,14 +242,17 @@ __global__ void __launch_bounds__(2 * BW, (NC == 1 && UH ? 3 : 2) * (128 / BW)) 
   const int zs = max_rows + 2;
   float4* const zh = reinterpret_cast<float4*>(rg_sm + NC * (XCH + ZCH));  // [NC][2][max_rows + 2]
   uint64_t* const full = reinterpret_cast<uint64_t*>(zh + NC * 2 * zs);
-  volatile int* const dead = reinterpret_cast<volatile int*>(full + RG_X);
+  volatile RingWait* const rw = reinterpret_cast<volatile RingWait*>(full + RG_X);
   double* const rsm = reinterpret_cast<double*>(full + RG_X + 2);
   const uint32_t xr = rg_addr(rg_sm), zr = xr + NC * XCH, bar = rg_addr(full);
   if (tid == 0) {
     for (int q = 0; q < RG_X; ++q)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar + 8 * q), "r"(1));
     asm volatile("fence.mbarrier_init.release.cluster;");
-    *dead = 0;
+    rw->err = err;
+    rw->limit = limit;
+    rw->dead = 0;
+    if (limit == 0) atomicOr(err, 16);  // gives up whatever its first polls say
   }
   __syncthreads();
   // the thread's site and its neighbours: own entry 2 + tid, the same cell's other site
@@ -275,7 +283,7 @@ __global__ void __launch_bounds__(2 * BW, (NC == 1 && UH ? 3 : 2) * (128 / BW)) 
     p += S;
     const int B1 = band * BW;
     const int cl = B1 == 0 ? G.L1 - 1 : B1 - 1, cr = B1 + BW == G.L1 ? 0 : B1 + BW;
-    int issued = 0, si = sw, yi = y0 >= 2 ? y0 - 2 : y0 - 2 + G.L2;  // next row to ask for (thread 0)
+    int si = sw, yi = y0 >= 2 ? y0 - 2 : y0 - 2 + G.L2;  // next row to ask for (thread 0)
     auto issue = [&]() {
       const size_t b = (size_t)r2 * yi;
       const uint32_t fb = bar + 8 * si;
@@ -289,7 +297,6 @@ __global__ void __launch_bounds__(2 * BW, (NC == 1 && UH ? 3 : 2) * (128 / BW)) 
         rg_copy(d + 32, x + 2 * B1, 2 * BW * 16, fb);
         rg_copy(d + 32 + 2 * BW * 16, x + 2 * cr, 32, fb);
       }
-      ++issued;
       si = si + 1 == RG_X ? 0 : si + 1;
       yi = yi + 1 == G.L2 ? 0 : yi + 1;
     };
@@ -324,7 +331,7 @@ __global__ void __launch_bounds__(2 * BW, (NC == 1 && UH ? 3 : 2) * (128 / BW)) 
     int sx = sw;                        // ring slot of row u = t (lattice row y0 - 2 + t)
     int waited = 0;
     auto wait_row = [&]() {
-      if (!rg_poll(bar + 8 * sw, pw)) rg_wait_slow(bar + 8 * sw, pw, dead);
+      if (!rg_poll(bar + 8 * sw, pw)) rg_wait_slow(bar + 8 * sw, pw, rw);
       sw = sw + 1 == RG_X ? 0 : sw + 1;
       pw ^= sw == 0 ? 1u : 0u;
       ++waited;
@@ -427,7 +434,6 @@ __global__ void __launch_bounds__(2 * BW, (NC == 1 && UH ? 3 : 2) * (128 / BW)) 
       }
     }
   }
-  rg_finish(dead, bar, sw, pw, err);
   double r[4] = {p2_total(q0), p2_total(q1), p2_total(q2), p2_total(q3)};
   block_reduce_rx<4>(r, 1, rsm);
   if (tid == 0) {
