@@ -918,10 +918,7 @@ extern "C" gqt_status gqt_kb_moments(gqt_ham* h, const void* d_r, int R, int M, 
     int flag = 0;
     check_cuda(cudaMemcpyAsync(&flag, h->d_flag.p, sizeof(int), cudaMemcpyDeviceToHost, st), "flag readback");
     check_cuda(cudaStreamSynchronize(st), "gqt_kb_moments");
-    if (flag & 32)
-      throw Error(GQT_ETIMEOUT, "gqt_kb_moments: a bounded tensor-core wait gave up and so did the drain of the "
-                                "copies and products in flight: later results in this CUDA context are not trusted");
-    if (flag & 16) throw Error(GQT_ETIMEOUT, "gqt_kb_moments: a bounded tensor-core wait gave up");
+    gqt::check_waits(flag, "gqt_kb_moments");
     return GQT_OK;
   } catch (const Error& e) {
     set_error(e.what());

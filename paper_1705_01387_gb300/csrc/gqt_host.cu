@@ -1736,7 +1736,7 @@ gqt_status gqt_kpm_reconstruct(const double* d_mu, int rows, int M, const double
     int flag = 0;
     check_cuda(cudaMemcpyAsync(&flag, err, sizeof(int), cudaMemcpyDeviceToHost, st), "status readback");
     check_cuda(cudaStreamSynchronize(st), "gqt_kpm_reconstruct");
-    if (flag) throw Error(GQT_ETIMEOUT, "gqt_kpm_reconstruct: a bounded tensor-core wait gave up");
+    check_waits(flag, "gqt_kpm_reconstruct");
     return GQT_OK;
   }
   check_cuda(cudaStreamSynchronize(st), "gqt_kpm_reconstruct");

@@ -241,13 +241,13 @@ inline gqt_status finish_call(gqt_ham* h, cudaStream_t st, const char* what) {
   check_cuda(cudaMemcpyAsync(h->h_flag, h->d_flag.p, sizeof(int), cudaMemcpyDeviceToHost, st), "flag readback");
   check_cuda(cudaStreamSynchronize(st), what);
   flag = *h->h_flag;
+  check_waits(flag, what);  // first: what the other checks saw may be its consequence
   if (flag & 4) throw Error(GQT_ENAN, std::string(what) + ": NaN or Inf in a result");
   if (flag & 2)
     throw Error(GQT_ERANGE, std::string(what) +
                                 ": a Chebyshev moment exceeds |l||r|: the spectrum of H/dE is not inside [-1,1] "
                                 "(energy scale too small)");
   if (flag & 8) throw Error(GQT_ENORM, std::string(what) + ": |U psi| differs from |psi| beyond tolerance");
-  if (flag & 16) throw Error(GQT_ETIMEOUT, std::string(what) + ": a bounded device wait gave up");
   return GQT_OK;
 }
 

@@ -40,6 +40,16 @@ void check_cuda(cudaError_t e, const char* what);
 void check_launch(const char* what);
 int sm_count();
 
+// The error of a status word whose bit 16 (a bounded device wait gave up) or 32 (so did
+// the drain of what it had in flight) is set.
+inline void check_waits(int flag, const char* what) {
+  if (flag & 32)
+    throw Error(GQT_ETIMEOUT, std::string(what) + ": a bounded device wait gave up and so did the drain of the copies "
+                                                  "and products in flight: later results in this CUDA context are "
+                                                  "not trusted");
+  if (flag & 16) throw Error(GQT_ETIMEOUT, std::string(what) + ": a bounded device wait gave up");
+}
+
 // Stream-ordered scratch of one call, given back on every way out (scratch pool of the
 // current device, gqt_host.cu).
 struct StreamScratch {

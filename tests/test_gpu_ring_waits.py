@@ -40,3 +40,17 @@ def test_waits_that_run_out(L1, L2, graphs):
         assert "drain" not in str(ei.value)
     g.gqt_set_wait_limit(ham, 1 << 24)
     assert rows() == want
+
+
+def test_a_wait_that_ran_out_is_named_first():
+    """A row of NaN whose waits run out: the status is that of the wait, whose consequence a
+    NaN in a result may be."""
+    ham = g.gqt_build_hamiltonian(kind=g.GQT_LATTICE_HONEYCOMB, L1=64, L2=40, t=-1.0, W=1.0, seed=1,
+                                  energy_scale=S.energy_scale_rule(3, -1.0, 1.0))
+    g.gqt_set_cluster(ham, False)
+    a = torch.full((ham.n, 1), float("nan"), dtype=torch.complex128, device="cuda")
+    for limit, status in ((1 << 24, g.GQT_ENAN), (0, g.GQT_ETIMEOUT)):
+        g.gqt_set_wait_limit(ham, limit)
+        with pytest.raises(g.GqtError) as ei:
+            g.gqt_dos_moments(ham, a, 1, 12, np.empty((1, 1, 12)))
+        assert ei.value.status == status
