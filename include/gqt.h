@@ -260,12 +260,13 @@ gqt_status gqt_set_kb_contraction(gqt_ham* ham, int mode);
 
 /* Polls of each bounded device wait of the handle's kernels (default 2^24, a
  * few tenths of a second to seconds; 0 = give up at once).  The kernels that wait are
- *  - the split-TF32 Hall contraction (gqt_set_kb_contraction mode 1), whose single
- *    issuing thread waits on mbarriers for the bulk tensor copies of each stage and for
- *    the commit of the products that read a buffer, and
+ *  - the Hall contractions (gqt_set_kb_contraction), whose issuing threads wait on
+ *    mbarriers for the bulk tensor copies of each stage and for the commit of the
+ *    products that read a buffer (and, in FP64, for the accumulators to be emptied, whose
+ *    warps wait for the products), and
  *  - the blocked FP64 moment rows (gqt_set_temporal_blocking), which wait for the bulk
  *    copies of their rows.
- * (The FP64 Hall contraction's waits always have 2^24 polls and end the same way.)
+ * (gqt_kpm_reconstruct has no handle: its waits have 2^24 polls.)
  * A wait that runs out is reported; what is in flight is then drained (committed
  * products and issued copies, 2^24 polls each, independent of this setting), tensor
  * memory is freed and the call returns GQT_ETIMEOUT; the moments it

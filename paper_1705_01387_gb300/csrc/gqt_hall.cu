@@ -781,7 +781,8 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
       char* sb = sl + slice_bytes(M, 2, nc);
       launch_slice_rows((const double*)Pst, 2, M, total, total, (size_t)c0 * SLICE_K, nullptr, nc, exps, sl, st);
       launch_slice_rows((const double*)Bst, 2, M, total, total, (size_t)c0 * SLICE_K, nullptr, nc, exps + M, sb, st);
-      launch_slice_gemm({sl, M, 2}, {sb, M, 2}, parts, nc, S, part, c0 > 0, (int*)h->d_flag.p, st);
+      launch_slice_gemm({sl, M, 2}, {sb, M, 2}, parts, nc, S, part, c0 > 0, (int*)h->d_flag.p,
+                        h->wait_limit, st);
     }
     prof_end(pg, 8, st);
     k_kb_unscale<<<(int)std::min<size_t>((mm + 255) / 256, 4096), 256, 0, st>>>(part, S, M, exps, exps + M,

@@ -1727,7 +1727,7 @@ gqt_status gqt_kpm_reconstruct(const double* d_mu, int rows, int M, const double
       for (int e0 = 0; e0 < NE; e0 += eb) {
         const int ne = std::min(eb, NE - e0);
         if (r0 == 0 || eb < NE) launch_cos_slices(d_E + e0, ne, energy_scale, M, nk, buf.p + o_b, st);
-        launch_slice_gemm({buf.p + o_a, nr, 1}, {buf.p + o_b, ne, 1}, one, nk, S, part, false, err, st);
+        launch_slice_gemm({buf.p + o_a, nr, 1}, {buf.p + o_b, ne, 1}, one, nk, S, part, false, err, SLICE_WAIT, st);
         k_kpm_unscale<<<(int)std::min<size_t>(((size_t)nr * ne + 255) / 256, 4096), 256, 0, st>>>(
             part, S, nr, exps + r0, d_E, e0, ne, NE, energy_scale, n_over_omega, d_out + (size_t)r0 * NE);
         check_launch("k_kpm_unscale");

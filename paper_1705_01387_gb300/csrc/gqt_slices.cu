@@ -27,9 +27,9 @@
 // (643 TFLOP/s of digit products, 0.31 of the FP16 rate) and 0.15 ms for the slices,
 // against 8.15 ms for the same contraction on the FP64 pipe at 0.99 of its rate.
 //
-// Every wait is bounded: after LIMIT polls a role gives up, the issuing thread drains
-// what it has in flight, tensor memory is freed, and the error word gets bit 16 (32 if
-// the drain gave up as well).
+// Every wait is bounded: after `limit` polls (0: at once) a role gives up, the issuing
+// thread drains what it has in flight (SLICE_WAIT polls a wait), tensor memory is freed,
+// and the error word gets bit 16 (32 if the drain gave up as well).
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -53,7 +53,6 @@ constexpr int SG_NBUF = 5;
 constexpr int SG_GROUP = 8;  // stages per emptying of the accumulators
 constexpr int SG_THREADS = 288;
 constexpr int SG_SMEM = SG_NBUF * SG_STAGE + 1024 + 256;
-constexpr int SG_LIMIT = 1 << 24;
 
 static_assert(SL * SG_GROUP * SG_K * (1 << 14) < (1 << 24), "a level's sum must stay exact in FP32");
 
@@ -69,15 +68,15 @@ __device__ __forceinline__ bool sg_poll(uint64_t* bar, uint32_t parity) {
   return done != 0;
 }
 // Bounded wait; gives up early once another role has.
-__device__ __forceinline__ bool sg_wait(uint64_t* bar, uint32_t parity, volatile int* stop) {
-  for (int it = 0; it < SG_LIMIT; ++it) {
+__device__ __forceinline__ bool sg_wait(uint64_t* bar, uint32_t parity, int limit, volatile int* stop) {
+  for (int it = 0; it < limit; ++it) {
     if (sg_poll(bar, parity)) return true;
     if (*stop) return false;
   }
   return false;
 }
 __device__ __forceinline__ bool sg_drain(uint64_t* bar, uint32_t parity) {
-  for (int it = 0; it < SG_LIMIT; ++it)
+  for (int it = 0; it < SLICE_WAIT; ++it)
     if (sg_poll(bar, parity)) return true;
   return false;
 }
@@ -130,7 +129,7 @@ __device__ __forceinline__ void sg_tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) 
 __global__ void __launch_bounds__(SG_THREADS, 1)
     k_slice_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, SliceParts parts,
                  int rows_a, int rows_b, int nchunk, int per_split, double* __restrict__ out, int add,
-                 int* __restrict__ err) {
+                 int* __restrict__ err, int limit) {
   extern __shared__ __align__(1024) unsigned char sg_raw[];
   const uint32_t raw = sg_addr(sg_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -184,8 +183,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
       for (int s = 0; s < nst && ok; ++s) {
         const int b = s % SG_NBUF, g = s / SG_GROUP;
         const bool fresh = s % SG_GROUP == 0;
-        if (fresh && g > 0) ok = sg_wait(acc_free, (uint32_t)((g - 1) & 1), stop);
-        ok = ok && sg_wait(&full[b], (uint32_t)((s / SG_NBUF) & 1), stop);
+        if (fresh && g > 0) ok = sg_wait(acc_free, (uint32_t)((g - 1) & 1), limit, stop);
+        ok = ok && sg_wait(&full[b], (uint32_t)((s / SG_NBUF) & 1), limit, stop);
         if (!ok) break;
         landed = s + 1;
         asm volatile("tcgen05.fence::after_thread_sync;");
@@ -204,7 +203,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         // stage s run
         if (s >= 1 && issued < nst) {
           const int p = s - 1;
-          if (!sg_wait(&done[p % SG_NBUF], (uint32_t)((p / SG_NBUF) & 1), stop)) {
+          if (!sg_wait(&done[p % SG_NBUF], (uint32_t)((p / SG_NBUF) & 1), limit, stop)) {
             ok = false;
             break;
           }
@@ -232,7 +231,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
     for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
     bool ok = true;
     for (int g = 0; g < groups; ++g) {
-      ok = sg_wait(acc_full, (uint32_t)(g & 1), stop);
+      ok = sg_wait(acc_full, (uint32_t)(g & 1), limit, stop);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
@@ -499,13 +498,14 @@ int slice_splits(int rows_a, int rows_b, int parts, int nchunk) {
 }
 
 void launch_slice_gemm(const SliceOperand& a, const SliceOperand& b, const SliceParts& parts, int nchunk, int splits,
-                       double* out, bool add, int* err, cudaStream_t st) {
+                       double* out, bool add, int* err, int limit, cudaStream_t st) {
   const CUtensorMap ma = slice_map(a, nchunk, SG_M), mb = slice_map(b, nchunk, SG_N);
   check_cuda(cudaFuncSetAttribute(k_slice_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM),
              "smem attribute");
   const int per = (nchunk + splits - 1) / splits;
   const dim3 grid((a.rows + SG_M - 1) / SG_M, (unsigned)((b.rows + SG_N - 1) / SG_N) * parts.n, splits);
-  k_slice_gemm<<<grid, SG_THREADS, SG_SMEM, st>>>(ma, mb, parts, a.rows, b.rows, nchunk, per, out, add ? 1 : 0, err);
+  k_slice_gemm<<<grid, SG_THREADS, SG_SMEM, st>>>(ma, mb, parts, a.rows, b.rows, nchunk, per, out, add ? 1 : 0, err,
+                                              limit);
   check_launch("k_slice_gemm");
 }
 

@@ -10,6 +10,7 @@ namespace gqt {
 
 constexpr int SLICES = 7;     // base-256 digits of a value
 constexpr int SLICE_K = 16;   // contraction elements per chunk
+constexpr int SLICE_WAIT = 1 << 24;  // polls of a device wait where no handle sets them
 
 // A matrix of `rows` rows (K-major) in `planes` real planes, sliced:
 // [plane * SLICES + slice][chunk][row][16] FP16.
@@ -37,8 +38,9 @@ void launch_slice_rows(const double* x, int comp, int rows, size_t stride, size_
 void launch_cos_slices(const double* E, int ne, double dE, int m, int nchunk, void* out, cudaStream_t st);
 int slice_splits(int rows_a, int rows_b, int parts, int nchunk);
 // out[split][part][rows_a][rows_b] (+)= the products of the scaled rows: times
-// 2^(exp_a - 1022 + exp_b - 1022) for the true values.  *err: bits 16, 32 (see above).
+// 2^(exp_a - 1022 + exp_b - 1022) for the true values.  *err: bit 16 where a device
+// wait of `limit` polls gave up, 32 where the drain after it did.
 void launch_slice_gemm(const SliceOperand& a, const SliceOperand& b, const SliceParts& parts, int nchunk, int splits,
-                       double* out, bool add, int* err, cudaStream_t st);
+                       double* out, bool add, int* err, int limit, cudaStream_t st);
 
 }  // namespace gqt
