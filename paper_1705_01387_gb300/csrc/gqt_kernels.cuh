@@ -920,7 +920,7 @@ static __global__ void k_kpm_table(int M, const double* __restrict__ E, int NE, 
       v = CUDART_NAN;
     } else {
       const double g = jackson ? (1.0 - n * a) * cos(M_PI * n * a) + a * sin(M_PI * n * a) * cot : 1.0;
-      v = g * (n == 0 ? 1.0 : 2.0) * cos(n * acos(x)) * 2.0 * n_over_omega / (M_PI * dE * sqrt(1.0 - x * x));
+      v = g * (n == 0 ? 1.0 : 2.0) * cos(n * acos(x)) * 2.0 * n_over_omega / (M_PI * dE * sqrt((1.0 - x) * (1.0 + x)));
     }
     tab[t] = v;
   }
@@ -935,9 +935,10 @@ static __global__ void k_kpm_moment_weights(int M, int jackson, double* __restri
   }
 }
 
-// Energy factor of the reconstruction, 2 (N/Omega) / (pi dE sqrt(1 - x^2)); NaN where |x| >= 1.
+// Energy factor of the reconstruction, 2 (N/Omega) / (pi dE sqrt(1 - x^2)); NaN where |x|
+// >= 1.  (1 - x)(1 + x): the rounding of x^2 would be 1e-11 of the factor at x = 1 - 1e-6.
 __device__ __forceinline__ double kpm_scale(double x, double dE, double n_over_omega) {
-  return fabs(x) < 1.0 ? 2.0 * n_over_omega / (M_PI * dE * sqrt(1.0 - x * x)) : CUDART_NAN;
+  return fabs(x) < 1.0 ? 2.0 * n_over_omega / (M_PI * dE * sqrt((1.0 - x) * (1.0 + x))) : CUDART_NAN;
 }
 
 // A few rows (up to RB = 8) of a reconstruction: one warp per energy, lane l the orders

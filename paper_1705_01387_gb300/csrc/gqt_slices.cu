@@ -387,13 +387,13 @@ __global__ void __launch_bounds__(128) k_slice_rows(const double* __restrict__ x
 // n0 th whose rounding is taken into account to first order.  M = 500, NE = 1001: 54 us,
 // the FP64 pipe's (4 multiply-adds an entry, an angle every 64); the table in memory, one
 // acos and cosine an entry, took 874.
-__global__ void __launch_bounds__(128) k_cos_slices(const double* __restrict__ E, int ne, double inv_dE, int m,
+__global__ void __launch_bounds__(128) k_cos_slices(const double* __restrict__ E, int ne, double dE, int m,
                                                     int nchunk, __half* __restrict__ out) {
   const int groups = (nchunk + 3) / 4;
   const size_t total = (size_t)groups * ne, plane = (size_t)nchunk * ne * SG_K;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
     const int e = (int)(t % ne), g = (int)(t / ne);
-    const double x = E[e] * inv_dE;
+    const double x = E[e] / dE;  // as the energy factor has it: an ulp of x is n ulp / sin th of an angle
     const bool in = fabs(x) < 1.0;
     const double th = in ? acos(x) : 0.0, sx = in ? sqrt((1.0 - x) * (1.0 + x)) : 0.0;
     const double n0 = 64.0 * g, a = n0 * th, da = fma(n0, th, -a);
@@ -476,7 +476,7 @@ void launch_slice_rows(const double* x, int comp, int rows, size_t stride, size_
 void launch_cos_slices(const double* E, int ne, double dE, int m, int nchunk, void* out, cudaStream_t st) {
   const size_t total = (size_t)((nchunk + 3) / 4) * ne;
   k_cos_slices<<<(int)std::min<size_t>((total + 127) / 128, (size_t)sm_count() * 32), 128, 0, st>>>(
-      E, ne, 1.0 / dE, m, nchunk, (__half*)out);
+      E, ne, dE, m, nchunk, (__half*)out);
   check_launch("k_cos_slices");
 }
 
