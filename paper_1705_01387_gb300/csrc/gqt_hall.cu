@@ -604,8 +604,9 @@ __global__ void k_kb_coef(const double* __restrict__ part, int M, int S, double4
 }
 
 // F at one energy per warp: lane l takes the angles k = l, l + 32, ..; cos k th and
-// sin k th advance by a rotation of 32 th and are taken afresh every 16 rotations,
-// which keeps their error at a few roundings.
+// sin k th advance by a rotation of 32 th and are taken afresh every 16 rotations, with
+// the rounding of k th taken into account to first order: at most 40 roundings, and k
+// times that of th (k 2^-53 th, 4e-12 at M = 8192).
 __global__ void __launch_bounds__(128) k_kb_series(const double4_16a* __restrict__ coef, int nk,
                                                    const double* __restrict__ E, int NE, double inv_dE,
                                                    double* __restrict__ F) {
@@ -616,8 +617,12 @@ __global__ void __launch_bounds__(128) k_kb_series(const double4_16a* __restrict
   sincos(32.0 * th, &rs, &rc);
   double cx = 0.0, cs = 0.0;  // coefficients of x and of s
   for (int k0 = lane; k0 < nk; k0 += 512) {
+    const double a = k0 * th, da = fma((double)k0, th, -a);
     double sn, cn;
-    sincos((double)k0 * th, &sn, &cn);
+    sincos(a, &sn, &cn);
+    const double c0 = cn;
+    cn = fma(-da, sn, cn);
+    sn = fma(da, c0, sn);
     const int kend = min(nk, k0 + 512);
 #pragma unroll 4
     for (int k = k0; k < kend; k += 32) {
@@ -633,7 +638,7 @@ __global__ void __launch_bounds__(128) k_kb_series(const double4_16a* __restrict
     cx += __shfl_xor_sync(0xffffffffu, cx, off);
     cs += __shfl_xor_sync(0xffffffffu, cs, off);
   }
-  if (lane == 0) F[e] = (x * cx + s * cs) / ((1.0 - x * x) * (1.0 - x * x));
+  if (lane == 0) F[e] = (x * cx + s * cs) / (s * s * s * s);
 }
 
 // sigma_j = pref * sum_{k<j} (x_{k+1} - x_k)(F_k + F_{k+1})/2: one CTA, each thread a
