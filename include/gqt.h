@@ -248,7 +248,11 @@ gqt_status gqt_kb_moments(gqt_ham* ham, const void* d_r, int R, int M, int alpha
 /* How gqt_kb_moments contracts the two stacks (default 0):
  * 0 = FP64 (Lambda to FP64 rounding): every stack row is scaled by a power of two and
  *     cut into seven 8-bit digits, whose products the tcgen05 tensor cores sum exactly
- *     (levels down to 2^-56 of the rows' largest elements);
+ *     down to 2^-56 of the rows' largest elements: an error of at most 2^-53 N R
+ *     max|P_m| max|B_n|, typically 2^-56 sqrt(N R) max|P_m| max|B_n|.  Entries of rows so
+ *     uneven that FP64 multiply-adds (which round by 2^-54 of their partial sums)
+ *     are the more exact are summed by those, 64 x 64 entries at a time, as are rows
+ *     with infinities, NaNs or nothing but denormals;
  * 1 = split TF32 on the tcgen05 tensor cores: both stacks are rounded to pairs of
  *     TF32 numbers (hi + lo, about 22 bits), each product is hi*hi + hi*lo + lo*hi,
  *     accumulated in FP32 over splits of at most 8192 sites and summed in FP64

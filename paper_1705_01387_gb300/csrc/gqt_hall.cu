@@ -15,9 +15,10 @@
 // order and applies v~_b to T_k r from the same neighbour gathers, writing the
 // stacks P (M vectors) and B (M vectors).  The M x M inner products <P_m|B_n> are a
 // dense complex contraction over N*R (4 M^2 N R FP64 FMAs), the dominant cost: the
-// default runs it to FP64 rounding on the tcgen05 tensor cores by exact integer slices
-// (gqt_slices.cu; k_kb_unscale sums its splits in order), k_kb_gemm_tma in split TF32,
-// its operands brought in by TMA.
+// default runs it on the tcgen05 tensor cores by exact integer slices (gqt_slices.cu;
+// k_kb_unscale sums its splits in order) where these are as exact as FP64 multiply-adds,
+// and by those (k_kb_gemm) where rows are too uneven; k_kb_gemm_tma runs it in split
+// TF32, its operands brought in by TMA.
 // k_kb_collapse turns the double sum over the moments into a series of 2M - 1 angles,
 // k_kb_series evaluates it on an energy grid, and k_kb_scan integrates it.
 
@@ -254,6 +255,78 @@ __global__ void __launch_bounds__(256) k_kb_step(HallEll<F64, CH> H,
   }
 }
 
+// part[s][m][n] = sum_{k in split s} conj(P[m][k]) B[n][k] by FP64 multiply-adds, P and B
+// row-major [M][Kt], for the entries that the slices hold less exactly: tiles of 64 x 64
+// in which no two spreads (launch_row_spreads) multiply to more than SLICE_SPREAD are
+// left out.  4 x 4 complex outputs per thread (rows tm + 16 i, columns tn + 16 j),
+// contraction chunks of 16 staged in shared memory (columns padded by one element
+// against bank conflicts).  Bound: the FP64 pipe (0.99 of its rate; M = 256, N R = 18432
+// with every tile 8.15 ms, with none 4 us).
+constexpr int KB_TM = 64, KB_TK = 16;
+
+__global__ void __launch_bounds__(256, 2) k_kb_gemm(const double2* __restrict__ P, const double2* __restrict__ B, int M,
+                                                    size_t Kt, size_t kchunk, const float* __restrict__ spread_p,
+                                                    const float* __restrict__ spread_b, double2* __restrict__ part) {
+  __shared__ double2 Ps[KB_TK][KB_TM + 1];
+  __shared__ double2 Bs[KB_TK][KB_TM + 1];
+  __shared__ unsigned top[2];
+  const int m0 = blockIdx.x * KB_TM, n0 = blockIdx.y * KB_TM;
+  const int tid = threadIdx.x, tm = tid & 15, tn = tid >> 4;
+  if (tid < 2) top[tid] = 0;
+  __syncthreads();
+  if (tid < 2 * KB_TM) {  // positive floats are ordered as their bits
+    const int row = (tid < KB_TM ? m0 : n0) + tid % KB_TM;
+    if (row < M) atomicMax(&top[tid / KB_TM], __float_as_uint((tid < KB_TM ? spread_p : spread_b)[row]));
+  }
+  __syncthreads();
+  if (!(__uint_as_float(top[0]) * __uint_as_float(top[1]) > SLICE_SPREAD)) return;
+  const size_t kb = (size_t)blockIdx.z * kchunk;
+  const size_t ke = (kb + kchunk < Kt) ? kb + kchunk : Kt;
+  double2 acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[a][c] = make_double2(0.0, 0.0);
+  for (size_t k0 = kb; k0 < ke; k0 += KB_TK) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const int q = tid + 256 * p;
+      const int row = q >> 4, kk = q & 15;
+      const size_t k = k0 + kk;
+      const bool kin = k < ke;
+      Ps[kk][row] = (kin && m0 + row < M) ? P[(size_t)(m0 + row) * Kt + k] : make_double2(0.0, 0.0);
+      Bs[kk][row] = (kin && n0 + row < M) ? B[(size_t)(n0 + row) * Kt + k] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < KB_TK; ++kk) {
+      double2 a[4], b[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        a[u] = Ps[kk][tm + 16 * u];
+        b[u] = Bs[kk][tn + 16 * u];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          acc[u][v].x = fma(a[u].x, b[v].x, acc[u][v].x);
+          acc[u][v].x = fma(a[u].y, b[v].y, acc[u][v].x);
+          acc[u][v].y = fma(a[u].x, b[v].y, acc[u][v].y);
+          acc[u][v].y = fma(-a[u].y, b[v].x, acc[u][v].y);
+        }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int m = m0 + tm + 16 * u, nn = n0 + tn + 16 * v;
+      if (m < M && nn < M) part[((size_t)blockIdx.z * M + m) * M + nn] = acc[u][v];
+    }
+}
+
 // ------------------------------------------------------------ tensor-core contraction
 // The same contraction on the tcgen05 tensor cores in split TF32 (three products
 // hi*hi + hi*lo + lo*hi per pair, FP32 accumulation in tensor memory over one
@@ -486,24 +559,31 @@ __global__ void __launch_bounds__(TM_THREADS, 1) k_kb_gemm_tma(const __grid_cons
 
 // lam[m][n] = scale * 2^(e_m + e_n) * sum_s part[s][m][n] from the sliced products
 // (part: [S][re, im][M][M] of rows scaled to below 1, exponents ep and eb of the P and
-// B rows), splits summed in order.  A row that holds an infinity or a NaN (biased
-// exponent 2047) makes its entries NaN.
+// B rows), or scale * sum_s pipe[s][m][n] from k_kb_gemm where the rows' spreads say so;
+// splits summed in order.
 __global__ void k_kb_unscale(const double* __restrict__ part, int S, int M, const int* __restrict__ ep,
-                             const int* __restrict__ eb, double scale, double2* __restrict__ lam) {
+                             const int* __restrict__ eb, const double2* __restrict__ pipe, int Sp,
+                             const float* __restrict__ spread_p, const float* __restrict__ spread_b, double scale,
+                             double2* __restrict__ lam) {
   const size_t total = (size_t)M * M;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
+    const size_t m = t / M, n = t % M;
     double re = 0.0, im = 0.0;
-    for (int q = 0; q < S; ++q) {
-      re += part[(2 * (size_t)q) * total + t];
-      im += part[(2 * (size_t)q + 1) * total + t];
-    }
-    const int xm = ep[t / M], xn = eb[t % M];
-    if (xm == 2047 || xn == 2047) {
-      lam[t] = make_double2(CUDART_NAN, CUDART_NAN);
+    int e = 0;
+    if (spread_p[m] * spread_b[n] > SLICE_SPREAD) {
+      for (int q = 0; q < Sp; ++q) {
+        const double2 v = pipe[(size_t)q * total + t];
+        re += v.x;
+        im += v.y;
+      }
     } else {
-      const int e = (xm - 1022) + (xn - 1022);
-      lam[t] = make_double2(scale * scalbn(re, e), scale * scalbn(im, e));
+      for (int q = 0; q < S; ++q) {
+        re += part[(2 * (size_t)q) * total + t];
+        im += part[(2 * (size_t)q + 1) * total + t];
+      }
+      e = (ep[m] - 1022) + (eb[n] - 1022);
     }
+    lam[t] = make_double2(scale * scalbn(re, e), scale * scalbn(im, e));
   }
 }
 
@@ -758,12 +838,21 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
       check_launch("k_kb_step");
       prof_end(pe, 7, st);
     }
+    // the FP64 multiply-adds' split of the contraction: about eight waves of two resident
+    // CTAs per SM, at least 512 contraction elements per split
+    const int tiles = (M + KB_TM - 1) / KB_TM;
+    const long long slots = 2LL * gqt::sm_count();
+    long long Sp = std::max<long long>(1, (8 * slots + (long long)tiles * tiles - 1) / ((long long)tiles * tiles));
+    Sp = std::min<long long>(Sp, std::max<long long>(1, (long long)(total / 512)));
+    int* exps = (int*)h->ws(WS_HALL_F, (size_t)4 * M * sizeof(int) + row_spread_bytes(M, total)).p;
+    float* spread = (float*)(exps + 2 * M);
+    void* scratch = exps + 4 * M;  // 16-byte aligned
+    for (int q = 0; q < 2; ++q)
+      launch_row_spreads((const double*)(q ? Bst : Pst), M, total, total, (double)total / Sp, scratch, exps + q * M,
+                         spread + q * M, st);
     // Lambda by exact slices of the stacks on the tensor cores: the contraction in
     // blocks of sites whose slices take at most 1 GiB (and half of the free memory, so
     // that stacks that fill the device still go through), later blocks added to the first
-    int* exps = (int*)h->ws(WS_HALL_F, (size_t)2 * M * sizeof(int)).p;
-    launch_row_exps((const double*)Pst, 2, M, total, total, nullptr, exps, st);
-    launch_row_exps((const double*)Bst, 2, M, total, total, nullptr, exps + M, st);
     const int nk = (int)((total + SLICE_K - 1) / SLICE_K);
     const size_t per_chunk = slice_bytes(M, 4, 1);
     size_t cap = (size_t)1 << 30;
@@ -774,7 +863,7 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
       cap = std::min(cap, std::max(held, free_b / 2));
     }
     const int blk = (int)std::min<size_t>(nk, std::max<size_t>(64, cap / per_chunk));
-    char* sl = (char*)h->ws(WS_HALL_S, per_chunk * blk).p;
+    char* sl = (char*)h->ws(WS_HALL_S, std::max(per_chunk * blk, mm * sizeof(double2))).p;
     const int S = slice_splits(M, M, 2, blk);
     double* part = (double*)h->ws(WS_HALL_PART, (size_t)S * 2 * mm * sizeof(double)).p;
     check_cuda(cudaMemsetAsync(h->d_flag.p, 0, sizeof(int), st), "flag reset");
@@ -789,9 +878,16 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
       launch_slice_gemm({sl, M, 2}, {sb, M, 2}, parts, nc, S, part, c0 > 0, (int*)h->d_flag.p,
                         h->wait_limit, st);
     }
+    // the uneven rows' entries, summed into the slices' buffer (as many splits as fit it)
+    Sp = std::min<long long>(Sp, (long long)(h->ws(WS_HALL_S, 0).bytes / (mm * sizeof(double2))));
+    const size_t kchunk = ((total + Sp - 1) / Sp + KB_TK - 1) / KB_TK * KB_TK;
+    Sp = (long long)((total + kchunk - 1) / kchunk);
+    double2* pipe = (double2*)sl;
+    k_kb_gemm<<<dim3(tiles, tiles, (unsigned)Sp), 256, 0, st>>>(Pst, Bst, M, total, kchunk, spread, spread + M, pipe);
+    check_launch("k_kb_gemm");
     prof_end(pg, 8, st);
-    k_kb_unscale<<<(int)std::min<size_t>((mm + 255) / 256, 4096), 256, 0, st>>>(part, S, M, exps, exps + M,
-                                                                                (double)h->n / R, lam);
+    k_kb_unscale<<<(int)std::min<size_t>((mm + 255) / 256, 4096), 256, 0, st>>>(
+        part, S, M, exps, exps + M, pipe, (int)Sp, spread, spread + M, (double)h->n / R, lam);
     check_launch("k_kb_unscale");
     return;
   }

@@ -13,10 +13,19 @@
 // such a sum rounds at 2^-53 of its partial sums.  |d_i d_j| <= 2^14 and at most 7
 // pairs share a level, so 8 stages of 16 elements stay below 2^24 and accumulate
 // without rounding in the FP32 accumulators of tensor memory; they are then added up
-// as 64-bit integers.  Errors against 64 bits are at or below those of the FP64 pipe's
-// fused multiply-adds: whole Lambda (chains in 64 bits) against 80-bit arithmetic,
-// sums of squares, 2.5e-16 at M = 12 and N R = 24 (3.0e-16 on the FP64 pipe), 8e-16 at
-// M = 100 and N R = 800 (1.4e-15), 8e-16 at M = 120 and N R = 1600 (1.0e-15).
+// as 64-bit integers.
+//
+// What is left out is at most 2^-53 of the product of the rows' largest elements for
+// every element of the contraction (six digit pairs of the first level left out and two
+// remainders, 2^-56 each), typically 2^-56 times the root of their number; a chain of
+// FP64 multiply-adds rounds by 2^-54 of its partial sums.  For rows of about even
+// magnitude the slices are the more exact of the two: simulated for normal values with the
+// largest at 2^e, 512 complex elements a chain, their error is 0.3, 0.6, 1.2 and 4 times
+// the multiply-adds' at 2^e = 6, 8, 12 and 24 standard deviations (2048 elements: 0.3,
+// 0.3, 0.7 and 3.9), which is the bound SLICE_SPREAD on the rows' spreads.  Whole Lambda
+// (chains in 64 bits) of random vectors against 80-bit arithmetic, sums of squares:
+// 2.5e-16 at M = 12 and N R = 24 (3.0e-16 on the FP64 pipe), 8e-16 at M = 100 and N R =
+// 800 (1.4e-15), 8e-16 at M = 120 and N R = 1600 (1.0e-15).
 //
 // One CTA: a 128 x 64 tile of one product, seven accumulators of 64 columns.  Stages of
 // 16 contraction elements (7 slices of both operands, 42 KB) come in by two bulk tensor
@@ -35,6 +44,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <math_constants.h>
 
 #include <algorithm>
 #include <string>
@@ -345,6 +355,96 @@ __global__ void __launch_bounds__(256) k_row_exps(const double* __restrict__ x, 
   if ((threadIdx.x & 31) == 0 && top > 0) atomicMax(exps + blockIdx.x, top);
 }
 
+// What k_row_spreads knows of a part of a row: its largest biased exponent, how many values
+// are not zero (nor denormal), and the sum of the squares of their leading 16 bits at the
+// scale of 2^(top - 1022) (a value v adds (2^16 v)^2 < 2^32).  Integers, so that the sum
+// does not load the FP64 pipe and, in a fixed tree, has the same bits each time.
+struct RowSpread {
+  unsigned long long sum;
+  unsigned int count;
+  int top;
+  __device__ __forceinline__ void rescale(int to) {
+    const int d = 2 * (to - top);
+    sum = d < 64 ? sum >> d : 0;
+    top = to;
+  }
+  __device__ __forceinline__ void add(RowSpread o) {
+    const int t = max(top, o.top);
+    rescale(t);
+    o.rescale(t);
+    sum += o.sum;
+    count += o.count;
+  }
+  __device__ __forceinline__ void warp() {
+    for (int off = 16; off > 0; off >>= 1) {
+      RowSpread o;
+      o.sum = __shfl_down_sync(0xffffffffu, sum, off);
+      o.count = __shfl_down_sync(0xffffffffu, count, off);
+      o.top = __shfl_down_sync(0xffffffffu, top, off);
+      add(o);
+    }
+  }
+};
+
+// Elements [blockIdx.y * span, ..) of row blockIdx.x (two doubles an element) into
+// part[row][blockIdx.y].  A value of nothing but denormals has top 0 and, if not zero, a
+// count of 1.
+__global__ void __launch_bounds__(256) k_row_spreads(const double* __restrict__ x, size_t stride, size_t k, size_t span,
+                                                     RowSpread* __restrict__ part) {
+  __shared__ RowSpread sh[8];
+  const double2* row = reinterpret_cast<const double2*>(x) + (size_t)blockIdx.x * stride;
+  const size_t e0 = (size_t)blockIdx.y * span, e1 = min(k, e0 + span);
+  RowSpread a = {0, 0, 0};
+  bool tiny = false;
+  auto add = [&](double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v) & 0x7FFFFFFFu;
+    const int ex = (int)(hi >> 20);
+    if (ex > a.top) a.rescale(ex);
+    if (ex == 0) {
+      tiny = tiny || v != 0.0;
+      return;
+    }
+    const uint32_t m = (((hi & 0xFFFFFu) | 0x100000u) >> 5) >> min(31, a.top - ex);
+    a.sum += (unsigned long long)m * m;
+    ++a.count;
+  };
+#pragma unroll 4
+  for (size_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+    const double2 v = row[e];
+    add(v.x);
+    add(v.y);
+  }
+  if (a.top == 0) a.count = tiny;
+  a.warp();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) a.add(sh[w]);
+    part[(size_t)blockIdx.x * gridDim.y + blockIdx.y] = a;
+  }
+}
+
+// One warp a row: its parts in a fixed tree, its exponent and its spread.
+__global__ void __launch_bounds__(128) k_row_spread_of(const RowSpread* __restrict__ part, int rows, int ny, size_t k,
+                                                       double chunk, int* __restrict__ exps,
+                                                       float* __restrict__ spread) {
+  const int r = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (r >= rows) return;
+  RowSpread a = {0, 0, 0};
+  for (int y = lane; y < ny; y += 32) a.add(part[(size_t)r * ny + y]);
+  a.warp();
+  if (lane != 0) return;
+  exps[r] = a.top;
+  float g = 1e-30f;  // a row of zeros: exact in any way
+  if (a.top == 2047 || (a.top == 0 && a.count > 0)) {
+    g = CUDART_INF_F;
+  } else if (a.count > 0) {
+    const double n = fmax(1.0, chunk * (double)a.count / (2.0 * (double)k));
+    g = (float)(65536.0 * sqrt((double)a.count / fmax(1.0, (double)a.sum) / sqrt(n)));
+  }
+  spread[r] = g;
+}
+
 // Slices of elements [k0, k0 + 16 nchunk) of every row (zeros past k), COMP planes:
 // out[plane * SL + slice][chunk][row][16].  Two threads a chunk and row, eight elements
 // each, rows fastest, so that a warp's stores are contiguous.
@@ -460,6 +560,22 @@ void launch_row_exps(const double* x, int comp, int rows, size_t stride, size_t 
   else
     k_row_exps<1><<<grid, 256, 0, st>>>(x, stride, k, w, span, exps);
   check_launch("k_row_exps");
+}
+
+// CTAs a row: a few per SM in all, at least 4096 elements each
+static size_t row_parts(int rows, size_t k) {
+  const size_t want = std::max<size_t>(1, (size_t)sm_count() * 8 / rows);
+  return std::min<size_t>(want, (k + 4095) / 4096);
+}
+size_t row_spread_bytes(int rows, size_t k) { return (size_t)rows * row_parts(rows, k) * sizeof(RowSpread); }
+
+void launch_row_spreads(const double* x, int rows, size_t stride, size_t k, double chunk, void* scratch, int* exps,
+                        float* spread, cudaStream_t st) {
+  const size_t ny = row_parts(rows, k), span = (k + ny - 1) / ny;
+  k_row_spreads<<<dim3(rows, (unsigned)ny), 256, 0, st>>>(x, stride, k, span, (RowSpread*)scratch);
+  check_launch("k_row_spreads");
+  k_row_spread_of<<<(rows + 3) / 4, 128, 0, st>>>((const RowSpread*)scratch, rows, (int)ny, k, chunk, exps, spread);
+  check_launch("k_row_spread_of");
 }
 
 void launch_slice_rows(const double* x, int comp, int rows, size_t stride, size_t k, size_t k0, const double* w,
