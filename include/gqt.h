@@ -197,7 +197,10 @@ gqt_status gqt_msd_moments(gqt_ham* ham, void* d_p, void* d_px, int R, const dou
  * x = E[e]/dE, g_n = (1 - n a) cos(pi n a) + a sin(pi n a) cot(pi a), a = 1/(M+1).
  * n_over_omega = N/Omega (sites per volume).  |x| >= 1 gives NaN.  kernel: 0 =
  * Jackson, 1 = none (g_n = 1).  d_mu [rows][M], d_E [NE], d_out [rows][NE]:
- * device FP64. */
+ * device FP64.  Up to 8 rows: FP64 multiply-adds.  More: by the exact digit products of
+ * gqt_set_kb_contraction's mode 0, with an error of at most 2^-53 M, typically 2^-56
+ * sqrt(M), of a row's largest weighted moment before the factor in front (rounding an
+ * angle n acos x is 2^-53 n acos x of the moment it belongs to in either form). */
 gqt_status gqt_kpm_reconstruct(const double* d_mu, int rows, int M, const double* d_E, int NE, double energy_scale,
                                double n_over_omega, int kernel, double* d_out, void* stream);
 

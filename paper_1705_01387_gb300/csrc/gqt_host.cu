@@ -1718,7 +1718,7 @@ gqt_status gqt_kpm_reconstruct(const double* d_mu, int rows, int M, const double
     int* exps = (int*)(buf.p + o_exp);
     int* err = (int*)(buf.p + o_err);
     check_cuda(cudaMemsetAsync(err, 0, sizeof(int), st), "status reset");
-    launch_row_exps(d_mu, 1, rows, M, M, w, exps, st);
+    launch_row_exps(d_mu, rows, M, w, exps, st);
     const SliceParts one = {1, 1, {{0, 0}, {0, 0}}, {{0, 0}, {0, 0}}, {{0, 0}, {0, 0}}};
     double* part = (double*)(buf.p + o_p);
     for (int r0 = 0; r0 < rows; r0 += rb) {
@@ -1729,7 +1729,7 @@ gqt_status gqt_kpm_reconstruct(const double* d_mu, int rows, int M, const double
         if (r0 == 0 || eb < NE) launch_cos_slices(d_E + e0, ne, energy_scale, M, nk, buf.p + o_b, st);
         launch_slice_gemm({buf.p + o_a, nr, 1}, {buf.p + o_b, ne, 1}, one, nk, S, part, false, err, SLICE_WAIT, st);
         k_kpm_unscale<<<(int)std::min<size_t>(((size_t)nr * ne + 255) / 256, 4096), 256, 0, st>>>(
-            part, S, nr, exps + r0, d_E, e0, ne, NE, energy_scale, n_over_omega, d_out + (size_t)r0 * NE);
+            part, S, nr, exps + r0, d_mu + (size_t)r0 * M, w, M, d_E, e0, ne, NE, energy_scale, n_over_omega, d_out + (size_t)r0 * NE);
         check_launch("k_kpm_unscale");
       }
     }

@@ -985,10 +985,24 @@ __global__ void __launch_bounds__(128) k_kpm_rows(const double* __restrict__ mu,
   }
 }
 
+// The moment sum of a row that has no scale to be sliced at (an infinity, a NaN, nothing
+// but zeros and denormals), term by term.
+static __device__ __noinline__ double kpm_sum(const double* __restrict__ mu, const double* __restrict__ w, int M,
+                                              double x) {
+  const double th = fabs(x) < 1.0 ? acos(x) : 0.0;
+  double acc = 0.0;
+  for (int n = 0; n < M; ++n) {
+    const double v = mu[n] * w[n];
+    if (v != 0.0) acc = fma(v, cos(n * th), acc);
+  }
+  return acc;
+}
+
 // out[row][e0 + e] = energy factor x 2^(row exponent) x sum over splits of the sliced
-// product part[split][row][e]; a row with an infinity or a NaN (biased exponent 2047)
-// is NaN.
+// product part[split][row][e], or x the sum itself where the row's largest biased
+// exponent is 0 or 2047.
 static __global__ void k_kpm_unscale(const double* __restrict__ part, int S, int rows, const int* __restrict__ exps,
+                                     const double* __restrict__ mu, const double* __restrict__ w, int M,
                                      const double* __restrict__ E, int e0, int ne, int NE, double dE,
                                      double n_over_omega, double* __restrict__ out) {
   const size_t total = (size_t)rows * ne;
@@ -997,7 +1011,9 @@ static __global__ void k_kpm_unscale(const double* __restrict__ part, int S, int
     double v = 0.0;
     for (int q = 0; q < S; ++q) v += part[(size_t)q * total + t];
     const int ex = exps[r];
-    out[(size_t)r * NE + e] = kpm_scale(E[e] / dE, dE, n_over_omega) * (ex == 2047 ? CUDART_NAN : scalbn(v, ex - 1022));
+    const double x = E[e] / dE;
+    v = ex == 0 || ex == 2047 ? kpm_sum(mu + (size_t)r * M, w, M, x) : scalbn(v, ex - 1022);
+    out[(size_t)r * NE + e] = kpm_scale(x, dE, n_over_omega) * v;
   }
 }
 

@@ -336,21 +336,16 @@ struct Digits {
   }
 };
 
-// Largest biased exponent of each row of x [rows][k] (COMP doubles an element) over
-// elements [blockIdx.y * span, ..), times the weights w [k] if given; 2047 (infinity or
-// NaN) stays and marks the row.  exps must hold zeros.
-template <int COMP>
-__global__ void __launch_bounds__(256) k_row_exps(const double* __restrict__ x, size_t stride, size_t k,
-                                                  const double* __restrict__ w, size_t span, int* __restrict__ exps) {
-  const double* row = x + (size_t)blockIdx.x * stride * COMP;
+// Largest biased exponent of each row of x [rows][k] times the weights w [k] over elements
+// [blockIdx.y * span, ..); 2047 (infinity or NaN) stays and marks the row.  exps must hold
+// zeros.
+__global__ void __launch_bounds__(256) k_row_exps(const double* __restrict__ x, size_t k, const double* __restrict__ w,
+                                                  size_t span, int* __restrict__ exps) {
+  const double* row = x + (size_t)blockIdx.x * k;
   const size_t e0 = (size_t)blockIdx.y * span, e1 = min(k, e0 + span);
   int top = 0;
-  for (size_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const double ww = w ? w[e] : 1.0;
-#pragma unroll
-    for (int c = 0; c < COMP; ++c)
-      top = max(top, (int)((__double_as_longlong(w ? row[e * COMP + c] * ww : row[e * COMP + c]) >> 52) & 0x7FF));
-  }
+  for (size_t e = e0 + threadIdx.x; e < e1; e += blockDim.x)
+    top = max(top, (int)((__double_as_longlong(row[e] * w[e]) >> 52) & 0x7FF));
   top = __reduce_max_sync(0xffffffffu, top);
   if ((threadIdx.x & 31) == 0 && top > 0) atomicMax(exps + blockIdx.x, top);
 }
@@ -548,25 +543,18 @@ CUtensorMap slice_map(const SliceOperand& o, int nchunk, int box_rows) {
 
 size_t slice_bytes(int rows, int planes, int nchunk) { return (size_t)planes * SL * nchunk * rows * SG_K * 2; }
 
-void launch_row_exps(const double* x, int comp, int rows, size_t stride, size_t k, const double* w, int* exps,
-                     cudaStream_t st) {
-  check_cuda(cudaMemsetAsync(exps, 0, (size_t)rows * sizeof(int), st), "row exponents");
-  // a few CTAs per SM in all, at least 4096 elements each
-  const size_t want = std::max<size_t>(1, (size_t)sm_count() * 8 / rows);
-  const size_t ny = std::min<size_t>(want, (k + 4095) / 4096), span = (k + ny - 1) / ny;
-  const dim3 grid(rows, (unsigned)ny);
-  if (comp == 2)
-    k_row_exps<2><<<grid, 256, 0, st>>>(x, stride, k, w, span, exps);
-  else
-    k_row_exps<1><<<grid, 256, 0, st>>>(x, stride, k, w, span, exps);
-  check_launch("k_row_exps");
-}
-
 // CTAs a row: a few per SM in all, at least 4096 elements each
 static size_t row_parts(int rows, size_t k) {
   const size_t want = std::max<size_t>(1, (size_t)sm_count() * 8 / rows);
   return std::min<size_t>(want, (k + 4095) / 4096);
 }
+void launch_row_exps(const double* x, int rows, size_t k, const double* w, int* exps, cudaStream_t st) {
+  check_cuda(cudaMemsetAsync(exps, 0, (size_t)rows * sizeof(int), st), "row exponents");
+  const size_t ny = row_parts(rows, k), span = (k + ny - 1) / ny;
+  k_row_exps<<<dim3(rows, (unsigned)ny), 256, 0, st>>>(x, k, w, span, exps);
+  check_launch("k_row_exps");
+}
+
 size_t row_spread_bytes(int rows, size_t k) { return (size_t)rows * row_parts(rows, k) * sizeof(RowSpread); }
 
 void launch_row_spreads(const double* x, int rows, size_t stride, size_t k, double chunk, void* scratch, int* exps,

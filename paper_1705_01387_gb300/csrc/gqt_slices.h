@@ -27,10 +27,8 @@ struct SliceParts {
 };
 
 size_t slice_bytes(int rows, int planes, int nchunk);
-// Largest biased exponents (times weights w [k], or null) of the rows of x [rows][k],
-// comp doubles per element (interleaved planes), rows `stride` elements apart.
-void launch_row_exps(const double* x, int comp, int rows, size_t stride, size_t k, const double* w, int* exps,
-                     cudaStream_t st);
+// Largest biased exponents of the rows of x [rows][k] times weights w [k].
+void launch_row_exps(const double* x, int rows, size_t k, const double* w, int* exps, cudaStream_t st);
 // The same exponents of complex rows, and how unevenly their values spread: spread[r] =
 // (2^exponent / rms) / n^(1/4) over the row's nonzero values, n of them (complex) in a sum
 // of `chunk` elements; infinite for a row with an infinity or a NaN or nothing but
