@@ -326,7 +326,9 @@ gqt_status gqt_sigma_msd(const double* d_msd, const double* dt, int Nt, int NE, 
  * (a real bond's hopping t_ij has dJ/dt = Re(G_ij + G_ji)).  *loss receives J.
  * Intermediate Chebyshev vectors are recomputed from checkpoints taken every
  * `stride` orders; stride <= 0 keeps all of them where they take at most 4 GiB and a
- * quarter of the free memory, else takes ceil(sqrt(M)).  beta may be host or device memory. */
+ * quarter of the memory that is free beside the call's other buffers, else takes
+ * ceil(sqrt(M)).  The handle keeps their buffer for the next gradient until another of
+ * its allocations needs the room.  beta may be host or device memory. */
 gqt_status gqt_vac_loss_grad(gqt_ham* ham, const void* d_phi, const double* dt, const int* Np, int Nt, int M,
                              const double* beta, int stride, double* loss, double* d_g_onsite, double* d_g_slot,
                              void* stream);

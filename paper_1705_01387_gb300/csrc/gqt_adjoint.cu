@@ -444,8 +444,26 @@ extern "C" gqt_status gqt_vac_loss_grad(gqt_ham* h, const void* d_phi, const dou
   const int nb = T.nblocks;
   const int* blk = (const int*)T.d_blk.p;
   const int thr = h->threads;
+  std::vector<double> hbeta;
+  if (!is_host_ptr(beta)) {  // device weights: one copy to the host (they become kernel arguments)
+    hbeta.resize((size_t)Nt * M);
+    check_cuda(cudaMemcpy(hbeta.data(), beta, hbeta.size() * sizeof(double), cudaMemcpyDeviceToHost), "beta");
+    beta = hbeta.data();
+  }
+  char* A = (char*)h->ws(WS_ADJ0 + 4, (size_t)Nt * vb).p;
+  char* B = (char*)h->ws(WS_ADJ0 + 5, (size_t)Nt * vb).p;
+  double* gdiag = (double*)h->ws(WS_ADJ0 + 6, (size_t)n * sizeof(double)).p;
+  double2* gslot = (double2*)h->ws(WS_ADJ0 + 7, (size_t)n * K * sizeof(double2)).p;
+  void* abar = h->ws(WS_ADJ0 + 8, vb).p;
+  void* bbar = h->ws(WS_ADJ0 + 9, vb).p;
+  double2* LB = (double2*)h->ws(WS_ADJ0 + 10, (size_t)n * sizeof(double2)).p;
+  void* tmp = h->ws(WS_ADJ0 + 11, vb).p;
+  void* l = h->ws(WS_L, vb).p;
+  double* dpart = (double*)h->ws(WS_ADJ0 + 12, (size_t)Nt * nb * sizeof(double)).p;  // loss partials per row
   // orders between checkpoints: the caller's, else all orders are kept where they fit
-  // ADJ_KEEP and a quarter of the free memory, and sqrt of the orders is the rule
+  // ADJ_KEEP and a quarter of the memory that is free once the buffers above are there
+  // (the rest of the call takes a dozen vectors, or as much as it would with checkpoints),
+  // and sqrt of the orders is the rule
   auto spacing = [&](int orders) {
     const int root = std::max(2, (int)std::ceil(std::sqrt((double)orders)));
     if (stride > 0) return root;
@@ -463,24 +481,9 @@ extern "C" gqt_status gqt_vac_loss_grad(gqt_ham* h, const void* d_phi, const dou
     nps[k] = resolve_np(h, dt[k], Np ? Np[k] : 0);
     if (k + 1 < Nt) most = std::max(most, nps[k]);
   }
+  const SpareInUse used(h->spare_in_use, WS_ADJ0 + 1);
   if (spacing(most) >= most) h->ws(WS_ADJ0 + 1, (size_t)std::max(2, most) * vb);
   const int row_stride = stride > 0 ? stride : spacing(M);
-  std::vector<double> hbeta;
-  if (!is_host_ptr(beta)) {  // device weights: one copy to the host (they become kernel arguments)
-    hbeta.resize((size_t)Nt * M);
-    check_cuda(cudaMemcpy(hbeta.data(), beta, hbeta.size() * sizeof(double), cudaMemcpyDeviceToHost), "beta");
-    beta = hbeta.data();
-  }
-  char* A = (char*)h->ws(WS_ADJ0 + 4, (size_t)Nt * vb).p;
-  char* B = (char*)h->ws(WS_ADJ0 + 5, (size_t)Nt * vb).p;
-  double* gdiag = (double*)h->ws(WS_ADJ0 + 6, (size_t)n * sizeof(double)).p;
-  double2* gslot = (double2*)h->ws(WS_ADJ0 + 7, (size_t)n * K * sizeof(double2)).p;
-  void* abar = h->ws(WS_ADJ0 + 8, vb).p;
-  void* bbar = h->ws(WS_ADJ0 + 9, vb).p;
-  double2* LB = (double2*)h->ws(WS_ADJ0 + 10, (size_t)n * sizeof(double2)).p;
-  void* tmp = h->ws(WS_ADJ0 + 11, vb).p;
-  void* l = h->ws(WS_L, vb).p;
-  double* dpart = (double*)h->ws(WS_ADJ0 + 12, (size_t)Nt * nb * sizeof(double)).p;  // loss partials per row
   auto Ak = [&](int k) { return (void*)(A + (size_t)k * vb); };
   auto Bk = [&](int k) { return (void*)(B + (size_t)k * vb); };
   // forward states a_k = U(-t_k) phi, b_k = U(-t_k) V phi

@@ -48,7 +48,8 @@ using gqt::set_error;
 
 namespace {
 
-enum { WS_HALL_P = 40, WS_HALL_B, WS_HALL_Q, WS_HALL_PART, WS_HALL_F, WS_HALL_W, WS_HALL_S };
+enum { WS_HALL_P = 40, WS_HALL_B, WS_HALL_Q, WS_HALL_PART, WS_HALL_F, WS_HALL_W };
+static_assert(WS_HALL_W < WS_HALL_S, "workspace slots");
 
 // H~ of a handle in the chain kernels: FP64 (double, double2 vectors) or FP32
 // storage (float, float2 vectors; the tensor-core contraction only).
@@ -863,6 +864,7 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
       cap = std::min(cap, std::max(held, free_b / 2));
     }
     const int blk = (int)std::min<size_t>(nk, std::max<size_t>(64, cap / per_chunk));
+    const SpareInUse used(h->spare_in_use, WS_HALL_S);
     char* sl = (char*)h->ws(WS_HALL_S, std::max(per_chunk * blk, mm * sizeof(double2))).p;
     const int S = slice_splits(M, M, 2, blk);
     double* part = (double*)h->ws(WS_HALL_PART, (size_t)S * 2 * mm * sizeof(double)).p;

@@ -428,13 +428,32 @@ DevBuf& gqt_ham::ws(int slot, size_t bytes) {
   DevBuf& b = *work[slot];
   const void* before = b.p;
   try {
-    b.ensure(bytes);
+    try {
+      b.ensure(bytes);
+    } catch (const Error& e) {
+      if (e.code != GQT_ENOMEM || !release_spare(slot)) throw;
+      b.ensure(bytes);
+    }
   } catch (...) {
     if (before) drop_graphs();  // the growth has freed the buffer
     throw;
   }
   if (before && b.p != before) drop_graphs();
   return b;
+}
+
+// Gives back the buffers that calls keep where memory allows and do without otherwise
+// (kept forward vectors, digit slices), except slot and the one that the running call
+// uses.  False: there were none.
+bool gqt_ham::release_spare(int slot) {
+  bool any = false;
+  for (int s : {(int)WS_ADJ0 + 1, (int)WS_HALL_S}) {
+    if (s == slot || s == spare_in_use || s >= (int)work.size() || !work[s] || !work[s]->p) continue;
+    drop_graphs();
+    work[s] = std::make_unique<DevBuf>();
+    any = true;
+  }
+  return any;
 }
 
 // Retires the captured graphs: a setting has changed which kernels run or their

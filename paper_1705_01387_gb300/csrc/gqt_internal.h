@@ -50,6 +50,15 @@ inline void check_waits(int flag, const char* what) {
   if (flag & 16) throw Error(GQT_ETIMEOUT, std::string(what) + ": a bounded device wait gave up");
 }
 
+// Marks a spare buffer of a handle as used until the end of the scope.
+struct SpareInUse {
+  int& slot;
+  SpareInUse(int& s, int v) : slot(s) { slot = v; }
+  ~SpareInUse() { slot = -1; }
+  SpareInUse(const SpareInUse&) = delete;
+  SpareInUse& operator=(const SpareInUse&) = delete;
+};
+
 // Stream-ordered scratch of one call, given back on every way out (scratch pool of the
 // current device, gqt_host.cu).
 struct StreamScratch {
@@ -96,6 +105,7 @@ enum WorkSlot {
   WS_PA1 = 18,  // chain A buffers of the two-recurrence (pair) moment rows
   WS_PA2 = 19,
   WS_ADJ0 = 20,  // adjoint workspace slots start here
+  WS_HALL_S = 46,  // digit slices of the Hall contraction (the other Hall slots: gqt_hall.cu)
   WS_STAGE0 = 96,  // +0, +1: host-resident VAC/MSD state staged on the device
   WS_TILE0 = 98,   // +0..+3: the third and fourth chain buffers of the tiled rows
   WS_TILE_SCRATCH = 102,  // per-CTA partial dots of a tiled grid larger than the single-order grid
@@ -169,6 +179,9 @@ struct gqt_ham {
   const gqt::BlockTable& table(int R, int grid_per_sm = 0);
   gqt::DevBuf& ws(int slot, size_t bytes);
   void drop_graphs();
+  // slot of the spare buffer (release_spare) that the running call uses, else -1
+  int spare_in_use = -1;
+  bool release_spare(int slot);
   size_t vec_bytes(int R) const;
   ~gqt_ham();
 };
