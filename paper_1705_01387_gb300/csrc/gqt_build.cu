@@ -561,6 +561,7 @@ extern "C" gqt_status gqt_build_hamiltonian(const gqt_lattice* lattice, double e
     h->d_flag.ensure(16);
     check_cuda(cudaMemset(h->d_flag.p, 0, 16), "memset");
     check_cuda(cudaMallocHost((void**)&h->h_flag, 16), "cudaMallocHost");
+    gqt::count_handle(h->device, +1);
     *out = h.release();
     return GQT_OK;
   } catch (const Error& e) {

@@ -67,7 +67,8 @@ void check_launch(const char* what) {
 // between calls: the device's default pool gives everything back at each
 // synchronisation, and mapping it anew costs 0.1 ms a call.  The pool is stream-ordered
 // and shared by all threads; an allocation that fails for want of memory, here or in
-// DevBuf, empties it and tries again.
+// DevBuf, empties it and tries again, and so does the end of a device's last handle, after
+// which a program that is done with the library holds none of its memory.
 constexpr size_t SCRATCH_KEEP = (size_t)128 << 20;
 constexpr int MAX_DEVICES = 64;
 static std::mutex g_pool_mu;
@@ -96,12 +97,21 @@ static cudaMemPool_t scratch_pool() {
   return g_pools[dev];
 }
 
-// Gives back what the current device's pool holds unused.
-static void trim_scratch() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= MAX_DEVICES) return;
+// Gives back what a device's pool (the current one's) holds unused.
+static void trim_scratch(int dev) {
+  if (dev < 0 || dev >= MAX_DEVICES) return;
   std::lock_guard<std::mutex> lock(g_pool_mu);
   if (g_pools[dev]) cudaMemPoolTrimTo(g_pools[dev], 0);
+}
+static void trim_scratch() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) trim_scratch(dev);
+}
+
+static std::atomic<int> g_handles[MAX_DEVICES] = {};
+void count_handle(int dev, int change) {
+  if (dev < 0 || dev >= MAX_DEVICES) return;
+  if (g_handles[dev].fetch_add(change) + change == 0) trim_scratch(dev);
 }
 
 StreamScratch::StreamScratch(size_t bytes, cudaStream_t s) : st(s) {
@@ -1407,7 +1417,12 @@ gqt_status gqt_profile_stop(double* ms, uint64_t* launches, int ncat) {
 }
 uint64_t gqt_launch_count(void) { return g_launches.load(); }
 
-void gqt_free_hamiltonian(gqt_ham* h) { delete h; }
+void gqt_free_hamiltonian(gqt_ham* h) {
+  if (!h) return;
+  const int dev = h->device;
+  delete h;
+  count_handle(dev, -1);
+}
 
 gqt_status gqt_ham_info(const gqt_ham* h, int64_t* n, double* energy_scale, double* volume, int* nseg, int* precision,
                         int* hop_real) {

@@ -50,6 +50,10 @@ inline void check_waits(int flag, const char* what) {
   if (flag & 16) throw Error(GQT_ETIMEOUT, std::string(what) + ": a bounded device wait gave up");
 }
 
+// A handle of a device was made (+1) or freed (-1); the last one's end empties the device's
+// scratch pool.
+void count_handle(int dev, int change);
+
 // Marks a spare buffer of a handle as used until the end of the scope.
 struct SpareInUse {
   int& slot;
