@@ -848,9 +848,7 @@ void kb_moments_impl(gqt_ham* h, const void* rv, int R, int M, const DA* da, con
     int* exps = (int*)h->ws(WS_HALL_F, (size_t)4 * M * sizeof(int) + row_spread_bytes(M, total)).p;
     float* spread = (float*)(exps + 2 * M);
     void* scratch = exps + 4 * M;  // 16-byte aligned
-    for (int q = 0; q < 2; ++q)
-      launch_row_spreads((const double*)(q ? Bst : Pst), M, total, total, (double)total / Sp, scratch, exps + q * M,
-                         spread + q * M, st);
+    launch_row_spreads((const double*)Pst, (const double*)Bst, M, total, (double)total / Sp, scratch, exps, spread, st);
     // Lambda by exact slices of the stacks on the tensor cores: the contraction in
     // blocks of sites whose slices take at most 1 GiB (and half of the free memory, so
     // that stacks that fill the device still go through), later blocks added to the first

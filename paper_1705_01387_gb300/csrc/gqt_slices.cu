@@ -381,13 +381,13 @@ struct RowSpread {
   }
 };
 
-// Elements [blockIdx.y * span, ..) of row blockIdx.x (two doubles an element) into
-// part[row][blockIdx.y].  A value of nothing but denormals has top 0 and, if not zero, a
-// count of 1.
-__global__ void __launch_bounds__(256) k_row_spreads(const double* __restrict__ x, size_t stride, size_t k, size_t span,
-                                                     RowSpread* __restrict__ part) {
+// Elements [blockIdx.y * span, ..) of row blockIdx.x of x0 and x1, `rows` rows each, into
+// part[row][blockIdx.y].  Nothing but denormals has top 0 and a count of 1.
+__global__ void __launch_bounds__(256) k_row_spreads(const double2* __restrict__ x0, const double2* __restrict__ x1,
+                                                     int rows, size_t k, size_t span, RowSpread* __restrict__ part) {
   __shared__ RowSpread sh[8];
-  const double2* row = reinterpret_cast<const double2*>(x) + (size_t)blockIdx.x * stride;
+  const int r = blockIdx.x;
+  const double2* row = r < rows ? x0 + (size_t)r * k : x1 + (size_t)(r - rows) * k;
   const size_t e0 = (size_t)blockIdx.y * span, e1 = min(k, e0 + span);
   RowSpread a = {0, 0, 0};
   bool tiny = false;
@@ -555,14 +555,18 @@ void launch_row_exps(const double* x, int rows, size_t k, const double* w, int* 
   check_launch("k_row_exps");
 }
 
-size_t row_spread_bytes(int rows, size_t k) { return (size_t)rows * row_parts(rows, k) * sizeof(RowSpread); }
+size_t row_spread_bytes(int rows, size_t k) {
+  return (size_t)2 * rows * row_parts(2 * rows, k) * sizeof(RowSpread);
+}
 
-void launch_row_spreads(const double* x, int rows, size_t stride, size_t k, double chunk, void* scratch, int* exps,
+void launch_row_spreads(const double* x0, const double* x1, int rows, size_t k, double chunk, void* scratch, int* exps,
                         float* spread, cudaStream_t st) {
-  const size_t ny = row_parts(rows, k), span = (k + ny - 1) / ny;
-  k_row_spreads<<<dim3(rows, (unsigned)ny), 256, 0, st>>>(x, stride, k, span, (RowSpread*)scratch);
+  const size_t ny = row_parts(2 * rows, k), span = (k + ny - 1) / ny;
+  k_row_spreads<<<dim3(2 * rows, (unsigned)ny), 256, 0, st>>>((const double2*)x0, (const double2*)x1, rows, k, span,
+                                                              (RowSpread*)scratch);
   check_launch("k_row_spreads");
-  k_row_spread_of<<<(rows + 3) / 4, 128, 0, st>>>((const RowSpread*)scratch, rows, (int)ny, k, chunk, exps, spread);
+  k_row_spread_of<<<(2 * rows + 3) / 4, 128, 0, st>>>((const RowSpread*)scratch, 2 * rows, (int)ny, k, chunk, exps,
+                                                      spread);
   check_launch("k_row_spread_of");
 }
 

@@ -29,15 +29,15 @@ struct SliceParts {
 size_t slice_bytes(int rows, int planes, int nchunk);
 // Largest biased exponents of the rows of x [rows][k] times weights w [k].
 void launch_row_exps(const double* x, int rows, size_t k, const double* w, int* exps, cudaStream_t st);
-// The same exponents of complex rows, and how unevenly their values spread: spread[r] =
-// (2^exponent / rms) / n^(1/4) over the row's nonzero values, n of them (complex) in a sum
-// of `chunk` elements; infinite for a row with an infinity or a NaN or nothing but
-// denormals.  An entry whose two spreads multiply to more than SLICE_SPREAD is summed
-// more exactly by FP64 multiply-adds over such chunks than by slices.  scratch:
-// row_spread_bytes.
+// The same exponents of the complex rows of x0 and x1 [rows][k], and how unevenly their
+// values spread: spread[r] = (2^exponent / rms) / n^(1/4) over the row's nonzero values, n
+// of them (complex) in a sum of `chunk` elements; infinite for a row with an infinity or a
+// NaN or nothing but denormals.  An entry whose two spreads multiply to more than
+// SLICE_SPREAD is summed more exactly by FP64 multiply-adds over such chunks than by
+// slices.  exps, spread: [x0's rows, x1's rows]; scratch: row_spread_bytes.
 constexpr float SLICE_SPREAD = 5.f;
 size_t row_spread_bytes(int rows, size_t k);
-void launch_row_spreads(const double* x, int rows, size_t stride, size_t k, double chunk, void* scratch, int* exps,
+void launch_row_spreads(const double* x0, const double* x1, int rows, size_t k, double chunk, void* scratch, int* exps,
                         float* spread, cudaStream_t st);
 // Slices of elements [k0, k0 + 16 nchunk) of each row (zeros past k).
 void launch_slice_rows(const double* x, int comp, int rows, size_t stride, size_t k, size_t k0, const double* w,
