@@ -5,7 +5,7 @@
 // kernels of a chain are launched with programmatic stream serialisation: a grid is set
 // up while the one before runs out, and waits (chain_wait) until that has ended and its
 // results are visible.  A Kubo-Bastin chain of 256 FP64 orders, 18,432 elements: 3.59 ->
-// 2.83 ms with its contraction; of 500 FP32 orders, 51,200 elements: 5.83 -> 4.59 ms; rows
+// 2.83 ms with its contraction; of 500 FP32 orders, 131,072 elements: 5.83 -> 4.59 ms; rows
 // replayed as graphs gain 1 to 5%.  No kernel lets its dependents start before its own
 // CTAs end (griddepcontrol.launch_dependents): several grids of waiting CTAs then pile
 // up on the SMs, and the same chains take 2.90 and 5.29 ms, those in graphs longer than
