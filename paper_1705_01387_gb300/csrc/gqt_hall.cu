@@ -741,7 +741,8 @@ __global__ void __launch_bounds__(1024) k_kb_scan(const double* __restrict__ F, 
   }
   if (lane == 31) wsum[warp] = inc;
   __syncthreads();
-  double base = inc - run;
+  double base = __shfl_up_sync(0xffffffffu, inc, 1);  // the runs before this one, which may be finite where it is not
+  if (lane == 0) base = 0.0;
   for (int q = 0; q < warp; ++q) base += wsum[q];
   for (int j = j0; j < j1; ++j) {
     base += panel(j);
